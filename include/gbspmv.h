@@ -78,7 +78,7 @@ typedef enum {
   GBS_VARIANT_MERGE_DIRECT = 4, /* merge-path whose threads load their own nonzeros from global
                                   memory in 128-bit groups (no shared-memory staging of vals /
                                   col_idx), so more items per thread fit */
-  GBS_VARIANT_ROWS_DIRECT = 5 /* ROWS without shared memory or barriers: every lane reads its
+  GBS_VARIANT_ROWS_DIRECT = 5, /* ROWS without shared memory or barriers: every lane reads its
                                  row's values and column ids itself through L1 and walks the
                                  whole row; k > 1: `lanes` lanes split the columns, as in ROWS;
                                  k == 1: one lane per row (lanes ignored).  Same results, bit
@@ -86,6 +86,8 @@ typedef enum {
                                  with one lane per row (k == 1); for short rows.  Not a
                                  batched item form, and values are not read through a
                                  permutation (not for the backward pass's A^T) */
+  GBS_VARIANT_SPLIT = 6 /* equal shares of nonzeros per merge thread, from a plan-time index of
+                           the row ends (8 bytes per 32 nonzeros); plans only */
 } gbs_variant;
 
 /*
@@ -97,6 +99,8 @@ typedef enum {
  *   threads      threads per CTA (multiple of 32, <= 1024).
  *   tile_nnz     ROWS: nonzeros staged in shared memory per pass.
  *   items        MERGE: merge-path items (rows + nonzeros) per thread.
+ *                SPLIT: nonzeros per merge thread: 8 for k = 1, a multiple of
+ *                32 up to 256 for k > 1 (0: 8; 64 for doubles, 32 for floats).
  *   emul         ROWS_TMA with double values: in every group of 4 nonzeros
  *                a lane handles, the first `emul` (0..3) products run on the
  *                FP32 pipe as float-float arithmetic (double operands split

@@ -35,6 +35,8 @@ VARIANT_ROWS = 1
 VARIANT_MERGE = 2
 VARIANT_ROWS_TMA = 3
 VARIANT_MERGE_DIRECT = 4
+VARIANT_ROWS_DIRECT = 5
+VARIANT_SPLIT = 6
 
 PLAN_TUNE = 1
 PLAN_CHECK = 2

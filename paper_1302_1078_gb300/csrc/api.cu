@@ -96,6 +96,7 @@ gbs_config normalize(const gbs_config& c, int dtype) {
   gbs_config r = c;
   if (r.threads <= 0) r.threads = 256;
   if (r.variant == GBS_VARIANT_ROWS_DIRECT && r.lanes <= 0) r.lanes = 1;
+  if (c.variant == GBS_VARIANT_SPLIT && c.threads <= 0) r.threads = 128;
   if (r.variant == GBS_VARIANT_ROWS || r.variant == GBS_VARIANT_ROWS_TMA) {
     if (r.lanes <= 0) r.lanes = 1;
     if (r.tile_nnz <= 0) r.tile_nnz = dtype == GBS_F64 ? 2048 : 3072;
@@ -110,8 +111,8 @@ struct MergeGeom {
 
 int check_cfg(const gbs_config& c) {
   if (c.variant != GBS_VARIANT_ROWS && !is_merge(c.variant) && c.variant != GBS_VARIANT_ROWS_TMA &&
-      c.variant != GBS_VARIANT_ROWS_DIRECT)
-    return fail(GBS_EINVAL, "variant must be ROWS, MERGE, ROWS_TMA, MERGE_DIRECT or ROWS_DIRECT after resolution");
+      c.variant != GBS_VARIANT_ROWS_DIRECT && c.variant != GBS_VARIANT_SPLIT)
+    return fail(GBS_EINVAL, "variant must be ROWS, MERGE, ROWS_TMA, MERGE_DIRECT, ROWS_DIRECT or SPLIT after resolution");
   if (c.variant == GBS_VARIANT_ROWS_TMA && c.threads > 256) return fail(GBS_EINVAL, "ROWS_TMA threads must be <= 256");
   if (c.threads % 32 != 0 || c.threads < 32 || c.threads > 1024) return fail(GBS_EINVAL, "threads must be 32..1024, multiple of 32");
   if (is_merge(c.variant) && c.threads > 256) return fail(GBS_EINVAL, "MERGE threads must be <= 256");
@@ -119,6 +120,7 @@ int check_cfg(const gbs_config& c) {
   if ((c.variant == GBS_VARIANT_ROWS || c.variant == GBS_VARIANT_ROWS_TMA) && (c.tile_nnz < 32 || c.tile_nnz > (1 << 14)))
     return fail(GBS_EINVAL, "tile_nnz must be in [32, 16384]");
   if (is_merge(c.variant) && (c.items < 0 || c.items > 256)) return fail(GBS_EINVAL, "items must be in [0, 256]");
+  if (c.variant == GBS_VARIANT_SPLIT && c.threads > 256) return fail(GBS_EINVAL, "SPLIT threads must be <= 256");
   if (c.emul < 0 || c.emul > 3) return fail(GBS_EINVAL, "emul must be in [0, 3]");
   if (c.relabel < 0 || c.relabel > 1024) return fail(GBS_EINVAL, "relabel must be in [0, 1024]");
   return GBS_OK;
@@ -641,6 +643,7 @@ static int product_entry(int m, int n, int nnz, const int* row_ptr, const int* c
     c = *cfg;
   }
   if (c.relabel != 0) return fail(GBS_EINVAL, "relabel needs a plan (gbs_plan_create / gbs_plan_set_config)");
+  if (c.variant == GBS_VARIANT_SPLIT) return fail(GBS_EINVAL, "SPLIT needs a plan (gbs_plan_create / gbs_plan_set_config)");
   c = normalize(c, dtype);
   rc = check_cfg(c);
   if (rc) return rc;
@@ -692,6 +695,11 @@ struct gbs_plan {
   long long ldxp = 1;
   int col_max_deg = -1;  // column-degree statistics, computed on first need
   double col_cv = 0.0;
+  // SPLIT: the index of split_kernel.cuh (words, ids and empty in one allocation) and the carries
+  void* split_base = nullptr;
+  SplitIndex split{};
+  void* split_carry = nullptr;
+  SplitScratch split_scratch{};
   bool tuning = false;   // the tuner is trying configurations: keep the relabelling between them
 };
 
@@ -724,6 +732,64 @@ int relabel_prepare(gbs_plan* p, cudaStream_t s) {
   return GBS_OK;
 }
 
+void split_release(gbs_plan* p) {
+  if (p->split_base) cudaFree(p->split_base);
+  if (p->split_carry) cudaFree(p->split_carry);
+  p->split_base = p->split_carry = nullptr;
+  p->split = SplitIndex{};
+}
+
+// The index (built once) and the carries of a plan whose configuration is SPLIT.
+int split_prepare(gbs_plan* p, cudaStream_t s) {
+  gbs_config& c = p->cfg;
+  if (c.items == 0) c.items = p->k == 1 ? kSplitShare : p->dtype == GBS_F64 ? 64 : 32;
+  if (p->k == 1 ? c.items != kSplitShare : c.items % 32 || c.items < 32 || c.items > 256)
+    return fail(GBS_EINVAL, "SPLIT items must be 8 (k = 1), or a multiple of 32 up to 256 (k > 1)");
+  cudaError_t e = cudaSuccess;
+  if (!p->split_base) {
+    const int nempty = p->stats.empty_rows, nrows = p->m - nempty;
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t b_words = up(sizeof(SplitWord) * (size_t)(((long long)p->nnz + 31) / 32));
+    const size_t b_ids = nempty ? up(sizeof(int) * (size_t)nrows) : 0;
+    const size_t b_empty = up(sizeof(int) * (size_t)nempty);
+    const size_t b_ord = nempty ? up(sizeof(int) * (size_t)p->m) : 0;
+    void* tmp = nullptr;
+    e = cudaMalloc(&p->split_base, b_words + b_ids + b_empty + 256);
+    if (e == cudaSuccess && nempty) e = cudaMallocAsync(&tmp, b_ord + sizeof(int) * scan_workspace_ints(p->m), s);
+    if (e == cudaSuccess) {
+      char* q = static_cast<char*>(p->split_base);
+      SplitWord* words = reinterpret_cast<SplitWord*>(q);
+      int* ids = nempty ? reinterpret_cast<int*>(q + b_words) : nullptr;
+      int* empty = nempty ? reinterpret_cast<int*>(q + b_words + b_ids) : nullptr;
+      p->split = SplitIndex{words, ids, empty, nempty};
+      e = split_build(p->m, p->nnz, p->row_ptr, words, ids, empty, static_cast<int*>(tmp),
+                      reinterpret_cast<int*>(static_cast<char*>(tmp) + b_ord), s);
+    }
+    if (tmp) {
+      const cudaError_t e2 = cudaFreeAsync(tmp, s);
+      if (e == cudaSuccess) e = e2;
+    }
+  }
+  // carries: a call without 128-bit column access has more lanes per merge thread, so more tiles
+  if (p->split_carry) cudaFree(p->split_carry);
+  p->split_carry = nullptr;
+  const int kp = std::min(panel_cols(p->dtype, true), p->k);
+  const int g = p->k == 1 ? 1 : std::min(32, pow2ceil(kp));
+  const size_t tiles = (size_t)split_tiles(p->nnz, g, c.items);
+  const size_t b_row = (sizeof(int) * tiles + 255) & ~(size_t)255;
+  if (e == cudaSuccess) e = cudaMalloc(&p->split_carry, b_row + tiles * (size_t)kp * dsize(p->dtype));
+  if (e == cudaSuccess) {
+    p->split_scratch.carry_row = static_cast<int*>(p->split_carry);
+    p->split_scratch.carry_val = static_cast<char*>(p->split_carry) + b_row;
+    e = cudaStreamSynchronize(s);
+  }
+  if (e != cudaSuccess) {
+    split_release(p);
+    return cuda_fail(e, "SPLIT index");
+  }
+  return GBS_OK;
+}
+
 int plan_prepare(gbs_plan* p, cudaStream_t s) {
   if (p->mb.base) {
     cudaFree(p->mb.base);
@@ -736,6 +802,8 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
     const int rc = relabel_prepare(p, s);
     if (rc) return rc;
   }
+  if (p->cfg.variant == GBS_VARIANT_SPLIT) return split_prepare(p, s);
+  if (!p->tuning) split_release(p);
   if (p->cfg.variant == GBS_VARIANT_ROWS_TMA && p->m > 0) {
     // the tile must hold the largest row block: measure it on the device
     int lanes = p->cfg.lanes;
@@ -790,6 +858,18 @@ int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, 
     ldx = p->ldxp;
   }
   const int as = vec16 ? 1 : 0;
+  if (p->cfg.variant == GBS_VARIANT_SPLIT) {
+    const int P = panel_cols(p->dtype, vec16);
+    const size_t es = dsize(p->dtype);
+    for (int c0 = 0; p->m > 0 && c0 < p->k; c0 += P) {
+      DenseView D{std::min(P, p->k - c0), static_cast<const char*>(X) + c0 * es, ldx, static_cast<char*>(Y) + c0 * es, ldy};
+      const cudaError_t e = p->dtype == GBS_F64
+          ? launch_split_f64(A, p->split, D, vec16, p->cfg.threads, p->cfg.items, p->split_scratch, s)
+          : launch_split_f32(A, p->split, D, vec16, p->cfg.threads, p->cfg.items, p->split_scratch, s);
+      if (e != cudaSuccess) return cuda_fail(e, "SPLIT launch");
+    }
+    return GBS_OK;
+  }
   if (is_merge(p->cfg.variant)) {
     // the partition was made for 128-bit column access; if this call cannot use it the
     // lane count differs and the stream-ordered path is used instead
@@ -840,12 +920,13 @@ std::vector<gbs_config> tune_candidates(const gbs_plan* p) {
               c.back().emul = em;
             }
         }
-    for (int it : {7, 11, 15, 23, 31}) add(GBS_VARIANT_MERGE, 0, 256, 0, it);
-    for (int it : {7, 9, 11, 13, 15, 23, 31, 47, 63}) add(GBS_VARIANT_MERGE_DIRECT, 0, 256, 0, it);
-    // smaller CTAs: the direct walk is held to 40 registers, so twelve 128-thread (or twenty-four
-    // 64-thread) CTAs fill an SM as six of 256 do, with finer tiles at the end of the grid
-    for (int it : {7, 8, 9, 10, 11, 13, 15}) add(GBS_VARIANT_MERGE_DIRECT, 0, 128, 0, it);
-    for (int it : {8, 9, 10, 11}) add(GBS_VARIANT_MERGE_DIRECT, 0, 64, 0, it);
+    // power-law rows: SPLIT won on every skewed matrix measured (R-MAT 20 and 22, FP64 and FP32),
+    // so the merge-path forms, which win where most rows are empty or of one nonzero, are tried
+    // only at the shapes that led before it (15 items staged; the direct walk's 8 to 11)
+    for (int th : {64, 128}) add(GBS_VARIANT_SPLIT, 0, th, 0, 0);
+    add(GBS_VARIANT_MERGE, 0, 256, 0, 15);
+    for (int it : {8, 9, 11}) add(GBS_VARIANT_MERGE_DIRECT, 0, 128, 0, it);
+    add(GBS_VARIANT_MERGE_DIRECT, 0, 64, 0, 8);
     for (int th : {128, 256}) add(GBS_VARIANT_ROWS_DIRECT, 1, th, 0, 0);
   } else {
     add(GBS_VARIANT_ROWS, 0, 256, base_tile, 0);
@@ -860,24 +941,21 @@ std::vector<gbs_config> tune_candidates(const gbs_plan* p) {
           add(GBS_VARIANT_ROWS_TMA, 0, th, 0, 0);
           c.back().emul = em;
         }
+    // longer shares pay for FP64, whose carry scan is a few slots of the scarce pipe per share;
+    // shorter ones for FP32, which wants warps in flight
+    for (int it : {32, 64, 128}) add(GBS_VARIANT_SPLIT, 0, 64, 0, it);
+    add(GBS_VARIANT_SPLIT, 0, 128, 0, p->dtype == GBS_F64 ? 128 : 32);
     add(GBS_VARIANT_MERGE, 0, 256, 0, 0);
-    add(GBS_VARIANT_MERGE, 0, 128, 0, 0);
-    add(GBS_VARIANT_MERGE_DIRECT, 0, 256, 0, 0);
     for (int th : {128, 256}) add(GBS_VARIANT_ROWS_DIRECT, 0, th, 0, 0);
   }
-  // skewed column degrees (a power-law matrix): the merge forms again on columns relabelled
-  // hottest first, with every gather through L1 or with the cold ones bypassing it
+  // skewed column degrees (a power-law matrix): SPLIT again on columns relabelled hottest first
   const double mean_col = p->n > 0 ? (double)p->nnz / p->n : 0.0;
   if (p->col_max_deg > 16.0 * mean_col + 256.0 || p->col_cv > 2.0) {
     std::vector<gbs_config> rl;
     for (const gbs_config& g : c)
-      if (is_merge(g.variant) && g.emul == 0) {
+      if (g.variant == GBS_VARIANT_SPLIT && g.threads == 64) {
         rl.push_back(g);
         rl.back().relabel = 1;
-        if (p->k == 1 && g.variant == GBS_VARIANT_MERGE_DIRECT && g.items <= 15) {
-          rl.push_back(g);
-          rl.back().relabel = 8;
-        }
       }
     c.insert(c.end(), rl.begin(), rl.end());
   }
@@ -1047,6 +1125,7 @@ int plan_create_impl(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr,
   }
   if (rc != GBS_OK) {
     relabel_release(p);
+    split_release(p);
     if (p->mb.base) cudaFree(p->mb.base);
     cudaFree(p->status);
     delete p;
@@ -1068,6 +1147,7 @@ int gbs_plan_create(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr, 
 int gbs_plan_destroy(gbs_plan* plan) {
   if (!plan) return GBS_OK;
   relabel_release(plan);
+  split_release(plan);
   if (plan->mb.base) cudaFree(plan->mb.base);
   if (plan->status) cudaFree(plan->status);
   delete plan;

@@ -30,6 +30,39 @@ struct MergeScratch {
   void* carry_val;  // [ctas * k] elements of the dtype
 };
 
+// Plan-time index of the SPLIT variant (split_kernel.cuh, split_build.cu): one word per 32 nonzeros.
+struct SplitWord {
+  unsigned int ends;  // bit j: nonzero 32 w + j is the last of its row
+  int first;          // ordinal, among the non-empty rows, of the row of nonzero 32 w
+};
+
+struct SplitIndex {
+  const SplitWord* words;  // [ceil(nnz / 32)]
+  const int* ids;          // [non-empty rows] their row numbers; NULL when no row is empty
+  const int* empty;        // [nempty] the empty rows
+  int nempty;
+};
+
+struct SplitScratch {
+  int* carry_row;   // [split_tiles]
+  void* carry_val;  // [split_tiles * k] elements of the dtype
+};
+
+// Nonzeros per merge thread of the SPLIT SpMV (x and y contiguous): one 32-byte sector of column ids.
+constexpr int kSplitShare = 8;
+
+// SPLIT variant.  share: nonzeros per merge thread of SpMM (a multiple of 32).  vec16 as for ROWS; values through A.perm if set.
+cudaError_t launch_split_f64(const CsrView& A, const SplitIndex& I, const DenseView& D, bool vec16, int threads,
+                             int share, const SplitScratch& S, cudaStream_t s);
+cudaError_t launch_split_f32(const CsrView& A, const SplitIndex& I, const DenseView& D, bool vec16, int threads,
+                             int share, const SplitScratch& S, cudaStream_t s);
+// Warps (tiles) of one launch; SpMM: g lanes per merge thread.
+long long split_tiles(int nnz, int g, int share);
+// Fills words (every word), ids (if not NULL) and empty (if not NULL); ord: workspace of m ints and
+// scan_ws of scan_workspace_ints(m), both unused (may be NULL) when the matrix has no empty row.
+cudaError_t split_build(int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* empty, int* ord,
+                        int* scan_ws, cudaStream_t s);
+
 // ROWS variant.  lanes: 1..32 (power of two); k == 1 -> lanes split nonzeros,
 // k > 1 -> lanes split columns (k <= lanes * VEC is required per launch;
 // wider k is done in column panels by the caller).  vec16: use 128-bit

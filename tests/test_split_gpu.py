@@ -1,0 +1,135 @@
+"""SPLIT plans (equal shares of nonzeros per merge thread) against the oracle: nonzero counts at the
+edges of a share, a word and a tile, rows that span many tiles, runs of empty rows, ragged and
+strided columns, arrays off a 32-byte boundary, values through a permutation, relabelled columns."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+NP = {torch.float64: np.float64, torch.float32: np.float32}
+TOL = {torch.float64: 1e-12, torch.float32: 2e-5}
+DT = pytest.mark.parametrize("dtype", [torch.float64, torch.float32], ids=["f64", "f32"])
+
+
+@pytest.fixture(scope="module")
+def gbs():
+    import paper_1302_1078_gb300 as g
+
+    g.lib()
+    return g
+
+
+def from_lengths(lens, n, seed):
+    lens = np.asarray(lens, np.int64)
+    rp = np.zeros(lens.size + 1, np.int64)
+    np.cumsum(lens, out=rp[1:])
+    rng = np.random.default_rng(seed)
+    return synth.CSR(lens.size, n, rp.astype(np.int32), rng.integers(0, n, rp[-1]).astype(np.int32),
+                     rng.uniform(-1, 1, rp[-1]))
+
+
+def hubs():
+    """Rows of tens of thousands of nonzeros (runs of well over eight tiles) between short and empty ones."""
+    rng = np.random.default_rng(3)
+    lens = rng.integers(0, 4, 5000)
+    lens[[0, 700, 701, 4999]] = [33000, 50001, 4096, 20000]
+    lens[1000:3000] = 0
+    return from_lengths(lens, 4000, 4)
+
+
+MATRICES = {f"nnz_{z}": (lambda z=z: from_lengths([0, z - z // 3, 0, z // 3], 50, z))
+            for z in (1, 7, 8, 9, 31, 32, 33, 255, 256, 257, 511, 512, 513, 1024, 1025, 4097)}
+MATRICES |= {
+    "hubs": hubs,
+    "singles": lambda: from_lengths(np.ones(3001, int), 3001, 5),
+    "stencil2d_37": lambda: synth.stencil2d(37),
+    "rmat_13": lambda: synth.rmat(13, ef=16, seed=4),
+    "random_rect": lambda: synth.random_csr(333, 1201, 0.02, 5, empty_rows=0.3),
+    "dup_unsorted": lambda: synth.random_csr(257, 257, 0.05, 6, sorted_cols=False, duplicates=True),
+    "empty_nnz": lambda: synth.random_csr(100, 50, 0.0, 7),
+}
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def within(y, ref, r, dtype, what):
+    got = y.double().cpu().numpy()
+    assert np.all(np.abs(got - ref) <= TOL[dtype] * r), what
+    assert np.all(got[r == 0] == 0.0), what
+
+
+@DT
+@pytest.mark.parametrize("name", list(MATRICES))
+def test_split_spmv(gbs, name, dtype):
+    A = MATRICES[name]()
+    v, x = A.vals.astype(NP[dtype]), synth.uniform(A.n, seed=31).astype(NP[dtype])
+    ref, r = oracle.spmv(A.m, A.row_ptr, A.col_idx, v, x)
+    rp, xd = dev(A.row_ptr), dev(x)
+    for off in (0, 1):  # off a 32-byte boundary: element by element
+        ci = torch.empty(A.nnz + 8, dtype=torch.int32, device="cuda")[off : off + A.nnz].copy_(dev(A.col_idx))
+        vd = torch.empty(A.nnz + 8, dtype=dtype, device="cuda")[off : off + A.nnz].copy_(dev(v))
+        plan = gbs.Plan(rp, ci, A.n, dtype, 1)
+        for cfg in (dict(), dict(items=8, threads=64), dict(items=8, threads=256)):
+            plan.set_config(dict(cfg, variant=6))
+            y = plan.spmv(vd, xd, torch.full((A.m,), float("nan"), dtype=dtype, device="cuda"))
+            within(y, ref, r, dtype, f"{name} {cfg} off={off}")
+            assert torch.equal(y, plan.spmv(vd, xd))
+            plan.set_config(dict(cfg, variant=6, relabel=1))
+            assert torch.equal(y, plan.spmv(vd, xd)), f"{name} {cfg}: relabelled"
+
+
+@DT
+@pytest.mark.parametrize("k", [1, 2, 3, 5, 8, 16, 33, 70])
+@pytest.mark.parametrize("name", ["nnz_1", "nnz_33", "nnz_1025", "hubs", "singles", "rmat_13", "random_rect", "empty_nnz"])
+def test_split_spmm(gbs, name, k, dtype):
+    A = MATRICES[name]()
+    v = A.vals.astype(NP[dtype])
+    ld = -(-(k + 1) // 4) * 4  # a row stride above k that keeps rows on 16 bytes
+    Xw = synth.uniform(A.n * ld, seed=32, stream=k).reshape(A.n, ld).astype(NP[dtype])
+    ref, r = oracle.spmm(A.m, A.row_ptr, A.col_idx, v, Xw[:, :k])
+    rp, ci, vd = dev(A.row_ptr), dev(A.col_idx), dev(v)
+    plan = gbs.Plan(rp, ci, A.n, dtype, k)
+    for items in ((8,) if k == 1 else (32, 64, 256)):
+        plan.set_config(dict(variant=6, items=items))
+        for X in (dev(Xw[:, :k]), dev(Xw)[:, :k]):
+            for Y in (torch.empty((A.m, k), dtype=dtype, device="cuda"),
+                      torch.empty((A.m, ld), dtype=dtype, device="cuda")[:, :k]):
+                Y.fill_(float("nan"))
+                plan.spmm(vd, X, Y)
+                within(Y, ref, r, dtype, f"{name} k={k} items={items} ld={X.stride(0)},{Y.stride(0)}")
+
+
+@DT
+@pytest.mark.parametrize("k", [1, 8])
+@pytest.mark.parametrize("name", ["nnz_513", "hubs", "rmat_13", "random_rect"])
+def test_split_backward(gbs, name, k, dtype):
+    """dX = A^T dY with A's values read through the transpose permutation."""
+    A = MATRICES[name]()
+    v = A.vals.astype(NP[dtype])
+    X = synth.uniform(A.n * k, seed=33).reshape(A.n, k).astype(NP[dtype])
+    W = synth.uniform(A.m * k, seed=34).reshape(A.m, k).astype(NP[dtype])
+    ref, _, r, _ = oracle.backward(A.m, A.n, A.row_ptr, A.col_idx, v, X, W)
+    t = gbs.TransposePlan(dev(A.row_ptr), dev(A.col_idx), A.n)
+    for items in ((0, 8) if k == 1 else (32, 64)):
+        t.set_config(dtype, k, dict(variant=6, items=items))
+        assert t.config(dtype, k)["variant"] == 6
+        dX, _ = t.backward(dev(v), dev(X[:, 0] if k == 1 else X), dev(W[:, 0] if k == 1 else W))
+        within(dX.reshape(A.n, k), ref.reshape(A.n, k), r.reshape(A.n, k), dtype, f"{name} k={k} {items}")
+
+
+def test_split_is_plans_only(gbs):
+    A = MATRICES["singles"]()
+    rp, ci, v = dev(A.row_ptr), dev(A.col_idx), dev(A.vals)
+    x = torch.zeros(A.n, dtype=torch.float64, device="cuda")
+    with pytest.raises(gbs.GbsError):
+        gbs.spmv_csr(rp, ci, v, x, config=dict(variant=6))
+    plan = gbs.Plan(rp, ci, A.n)
+    for bad in (dict(items=7), dict(items=16), dict(threads=512)):
+        with pytest.raises(gbs.GbsError):
+            plan.set_config(dict(bad, variant=6))
