@@ -260,6 +260,49 @@ int run_product(const CsrView& A, int dtype, int k, const void* X, long long ldx
   return rc;
 }
 
+// One product without a plan: the SPLIT index from two passes over row_ptr, then the nonzero-split
+// walk, whatever the row lengths.  GBS_ENOMEM (nothing launched) if its scratch cannot be had.
+int run_split_once(const CsrView& A, int dtype, int k, const void* X, long long ldx, void* Y, long long ldy,
+                   cudaStream_t s) {
+  if (A.m == 0 || k == 0) return GBS_OK;
+  const bool vec16 = dense_vec16(dtype, k, X, ldx, Y, ldy);
+  const int P = panel_cols(dtype, vec16), kp_max = std::min(P, k);
+  const bool spmv = k == 1 && ldx == 1 && ldy == 1;
+  const int g = spmv ? 1 : col_lanes(kp_max, dtype, vec16);
+  // long shares for doubles (their carry scan takes slots of the FP64 pipe) once every SM has its
+  // warps; the shortest otherwise
+  int share = spmv ? kSplitShare : 32;
+  if (!spmv && dtype == GBS_F64 && split_tiles(A.nnz, g, 64) >= 152 * 24) share = 64;
+  const size_t tiles = (size_t)split_tiles(A.nnz, g, share), es = dsize(dtype);
+  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+  const size_t b_words = up(sizeof(SplitWord) * (size_t)(((long long)A.nnz + 31) / 32));
+  const size_t b_ids = up(sizeof(int) * (size_t)A.m), b_counts = sizeof(int) * (kSplitBlocks + 64);
+  const size_t b_row = up(sizeof(int) * tiles);
+  void* base = nullptr;
+  cudaError_t e = cudaMallocAsync(&base, b_words + b_ids + b_counts + b_row + tiles * (size_t)kp_max * es, s);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(GBS_ENOMEM, "scratch of a one-shot product");
+  }
+  char* q = static_cast<char*>(base);
+  SplitWord* words = reinterpret_cast<SplitWord*>(q);
+  int* ids = reinterpret_cast<int*>(q + b_words);
+  int* counts = reinterpret_cast<int*>(q + b_words + b_ids);
+  int* nonempty = counts + kSplitBlocks;
+  q += b_words + b_ids + b_counts;
+  const SplitIndex I{words, ids, nullptr, 0, nonempty};
+  const SplitScratch S{reinterpret_cast<int*>(q), q + b_row};
+  e = split_build_once(dtype, A.m, A.nnz, A.row_ptr, words, ids, nonempty, counts, k, Y, ldy, s);
+  for (int c0 = 0; e == cudaSuccess && c0 < k; c0 += P) {
+    DenseView D{std::min(P, k - c0), static_cast<const char*>(X) + c0 * es, ldx, static_cast<char*>(Y) + c0 * es, ldy};
+    e = dtype == GBS_F64 ? launch_split_f64(A, I, D, vec16, 64, share, S, s)
+                         : launch_split_f32(A, I, D, vec16, 64, share, S, s);
+  }
+  const cudaError_t e2 = cudaFreeAsync(base, s);
+  if (e == cudaSuccess) e = e2;
+  return e == cudaSuccess ? GBS_OK : cuda_fail(e, "one-shot product");
+}
+
 // --------------------------------------------------------------- statistics
 
 __global__ void stats_kernel(const int* __restrict__ rp, int m, unsigned long long* __restrict__ acc, int* __restrict__ maxrow) {
@@ -628,11 +671,23 @@ static int product_entry(int m, int n, int nnz, const int* row_ptr, const int* c
     rc = gbs_validate_csr(m, n, nnz, row_ptr, col_idx, stream);
     if (rc) return rc;
   }
+  CsrView A{m, n, nnz, row_ptr, col_idx, vals};
+  const bool unset = cfg == nullptr ||
+                     (cfg->variant == GBS_VARIANT_AUTO && !cfg->threads && !cfg->items && !cfg->lanes && !cfg->relabel);
+  // a vector product of fewer items than this is bound by its launches, of which merge-path has
+  // three and SPLIT four (64 x 64 grid: 25.1 and 25.5 us; 1.3 M nonzeros: 31.8 and 25.8 us)
+  const bool small = k == 1 && (long long)m + nnz < 400000;
+  if (unset && !small) {
+    // SPLIT, which needs no row statistics and balances any row lengths (27-point 100^3, k = 4:
+    // 353 us staged merge-path, 238 us; R-MAT 20, k = 1: 109 us direct merge walk, 96 us); where
+    // its scratch cannot be had, merge-path below needs a fraction of it
+    rc = run_split_once(A, dtype, k, X, ldx, Y, ldy, s);
+    if (rc != GBS_ENOMEM) return rc;
+  }
   gbs_config c{};
   if (cfg == nullptr || cfg->variant == GBS_VARIANT_AUTO) {
-    // merge-path, which needs no row statistics: SpMV with contiguous x and y takes the direct
-    // walk's SpMV form (128 threads x 9 items; 1.5-2x the staged form on the 27-point stencil,
-    // the banded matrix and R-MAT 22, scratch and partition included), SpMM the staged form
+    // merge-path: SpMV with contiguous x and y takes the direct walk's SpMV form (128 threads x 9
+    // items), SpMM the staged form
     const bool spmv = k == 1 && ldx == 1 && ldy == 1;
     c.variant = spmv ? GBS_VARIANT_MERGE_DIRECT : GBS_VARIANT_MERGE;
     c.threads = cfg && cfg->threads ? cfg->threads : (spmv ? 128 : 256);
@@ -647,7 +702,6 @@ static int product_entry(int m, int n, int nnz, const int* row_ptr, const int* c
   c = normalize(c, dtype);
   rc = check_cfg(c);
   if (rc) return rc;
-  CsrView A{m, n, nnz, row_ptr, col_idx, vals};
   return run_product(A, dtype, k, X, ldx, Y, ldy, c, nullptr, false, s);
 }
 

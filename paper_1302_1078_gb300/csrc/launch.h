@@ -39,8 +39,9 @@ struct SplitWord {
 struct SplitIndex {
   const SplitWord* words;  // [ceil(nnz / 32)]
   const int* ids;          // [non-empty rows] their row numbers; NULL when no row is empty
-  const int* empty;        // [nempty] the empty rows
+  const int* empty;        // [nempty] the empty rows still to be written as zero
   int nempty;
+  const int* nonempty = nullptr;  // if set, the number of non-empty rows, on the device (ids unused when it is m)
 };
 
 struct SplitScratch {
@@ -62,6 +63,11 @@ long long split_tiles(int nnz, int g, int share);
 // scan_ws of scan_workspace_ints(m), both unused (may be NULL) when the matrix has no empty row.
 cudaError_t split_build(int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* empty, int* ord,
                         int* scan_ws, cudaStream_t s);
+// The index of a one-shot call in two launches: words, ids [m], nonempty [1]; counts is a workspace
+// of kSplitBlocks ints.  Also writes the zeros of Y's empty rows (k columns).
+constexpr int kSplitBlocks = 2048;
+cudaError_t split_build_once(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
+                             int* counts, int k, void* Y, long long ldy, cudaStream_t s);
 
 // ROWS variant.  lanes: 1..32 (power of two); k == 1 -> lanes split nonzeros,
 // k > 1 -> lanes split columns (k <= lanes * VEC is required per launch;

@@ -73,6 +73,7 @@ cudaError_t launch_split_t(const CsrView& A, const SplitIndex& I, const DenseVie
   a.words = I.words;
   a.nwords = (int)(((long long)A.nnz + 31) / 32);
   a.ids = I.ids;
+  a.nonempty = I.nonempty;
   a.carry_row = S.carry_row;
   a.carry_val = static_cast<T*>(S.carry_val);
   const void* v = A.perm ? static_cast<const void*>(A.perm) : A.vals;

@@ -16,8 +16,8 @@
 // is then an ordinal plus a population count, and a row end is a bit test on a
 // register where the merge walk re-reads row_ptr.  `ids` maps ordinals to row
 // numbers (NULL when no row is empty); empty rows are written as zero by the
-// fix-up kernel from their own list, so a run of a million empty rows costs
-// its stores and nothing else.
+// fix-up kernel from their own list (a one-shot call: by the pass that makes
+// the index), so a run of a million empty rows costs its stores and nothing else.
 //
 // A warp is on its own: no shared memory and no barrier.  The rows that are
 // split across merge threads are finished as in the merge kernel, by a
@@ -54,6 +54,7 @@ struct SplitArgs {
   const SplitWord* __restrict__ words;
   int nwords;
   const int* __restrict__ ids;  // row number of each non-empty row; NULL: its ordinal
+  const int* __restrict__ nonempty;  // if set, the device's count of non-empty rows: ids unused when it is m
   int share;                    // SpMM: nonzeros per merge thread (multiple of 32)
   int tiles;                    // warps
   int* __restrict__ carry_row;  // [tiles] row still open at the tile's end, or -1
@@ -109,14 +110,16 @@ __device__ __forceinline__ void split_load8(const SplitArgs<T>& a, int p, bool w
 }
 
 template <typename T>
-__device__ __forceinline__ int split_row(const SplitArgs<T>& a, int ord) {
-  return a.ids ? __ldg(a.ids + ord) : ord;
+__device__ __forceinline__ const int* split_ids(const SplitArgs<T>& a) {
+  return a.nonempty && __ldg(a.nonempty) == a.m ? nullptr : a.ids;
 }
+__device__ __forceinline__ int split_row(const int* __restrict__ ids, int ord) { return ids ? __ldg(ids + ord) : ord; }
 
 // SpMV: x and y contiguous, one lane per merge thread, N = 8 nonzeros each.
 template <typename T, bool PERM>
 __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile) {
   constexpr int N = kSplitShare;
+  const int* __restrict__ ids = split_ids(a);
   const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
   const int lane = threadIdx.x & 31;
   // 64-bit: the last tiles' lanes may lie past 2^31
@@ -145,7 +148,7 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
           head = acc.value();
           first = false;
         } else {
-          st_stream(a.Y + split_row(a, ord), acc.value());
+          st_stream(a.Y + split_row(ids, ord), acc.value());
         }
         ++ord;
         acc.reset();
@@ -169,13 +172,13 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
   }
   const T before = __shfl_up_sync(0xffffffffu, S, 1);
   if (ends != 0) {
-    const int r = split_row(a, ord - __popc(ends));
+    const int r = split_row(ids, ord - __popc(ends));
     st_stream(a.Y + r, lane > 0 ? head + before : head);
   }
   if (lane == 31) {
     // the tile's last nonzero lies in a row that goes on unless it ends there or the matrix does
     const bool open = p0 + N < a.nnz && !(ends >> (N - 1) & 1u);
-    a.carry_row[tile] = open ? split_row(a, ord) : -1;
+    a.carry_row[tile] = open ? split_row(ids, ord) : -1;
     a.carry_val[tile] = S;
   }
 }
@@ -191,6 +194,7 @@ __global__ void __launch_bounds__(256, 5) split_spmv_kernel(SplitArgs<T> a) {
 template <typename T, int VEC, int G, bool PERM>
 __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile) {
   constexpr int MT = 32 / G;  // merge threads per warp
+  const int* __restrict__ ids = split_ids(a);
   const uint64_t pol_stream = policy_evict_first(), pol_keep = policy_evict_last();
   const int wl = threadIdx.x & 31, mt = wl / G, c_lo = (wl % G) * VEC;
   const bool col_active = c_lo < a.k, col_full = c_lo + VEC <= a.k;
@@ -199,7 +203,7 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
   const T* __restrict__ Xc = a.X + c_lo;
   T* __restrict__ Yc = a.Y + c_lo;
   auto store_row = [&](int ord, const T* out) {
-    T* y = Yc + (long long)split_row(a, ord) * a.ldy;
+    T* y = Yc + (long long)split_row(ids, ord) * a.ldy;
     if (col_full)
       st_stream_vec<T, VEC>(y, out);
     else
@@ -286,7 +290,7 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
   }
   if (head_ord >= 0 && col_active) store_row(head_ord, head);
   if (mt == MT - 1) {
-    if (wl == 32 - G) a.carry_row[tile] = w1 - w0 == nwp && (long long)w1 * 32 < a.nnz && !last_end ? split_row(a, ord) : -1;
+    if (wl == 32 - G) a.carry_row[tile] = w1 - w0 == nwp && (long long)w1 * 32 < a.nnz && !last_end ? split_row(ids, ord) : -1;
     if (col_active)
       for (int j = 0; j < VEC && c_lo + j < a.k; ++j) a.carry_val[(size_t)tile * a.k + c_lo + j] = S[j];
   }
