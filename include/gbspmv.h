@@ -390,7 +390,7 @@ int spmm_csr_plan(const gbs_plan* plan, const void* vals, const void* X, int ldx
  * row of A^T the entries keep their order of storage in A, so the result is
  * unique and bit-exact (no atomics decide any position).  The plan owns
  *   rowptrT[n+1], colT[nnz] (row of A of each entry), perm[nnz] (position in
- *   A of each entry of A^T) and the row of every nonzero of A (the dvals
+ *   A of each entry of A^T) and the SPLIT index of A's rows (the dvals
  *   pass); plus, only if a configuration that permutes the values first is
  *   chosen, nnz doubles of scratch.
  * It does not keep row_ptr / col_idx.  It also creates a non-blocking

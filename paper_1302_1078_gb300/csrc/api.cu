@@ -1272,7 +1272,7 @@ struct gbs_tplan {
   int* rptrT = nullptr;      // n + 1
   int* colT = nullptr;       // nnz
   int* perm = nullptr;       // nnz
-  int* rows = nullptr;       // nnz: row of every nonzero of A (the dvals pass)
+  SplitIndex index{};        // A's rows (the dvals pass), for m rows
   void* base = nullptr;
   void* valsT = nullptr;     // nnz values, only for a prepared plan that permutes the values first
   gbs_stats statsT{};
@@ -1354,7 +1354,9 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
   cudaGetDevice(&t->device);
   const size_t z = (size_t)std::max(nnz, 1);
   size_t b_rptr = align256(sizeof(int) * ((size_t)n + 1)), b_i = align256(sizeof(int) * z);
-  size_t keep = b_rptr + 3 * b_i;
+  const size_t b_words = align256(sizeof(SplitWord) * (size_t)(((long long)nnz + 31) / 32));
+  const size_t b_ids = align256(sizeof(int) * ((size_t)m + 1)), b_counts = sizeof(int) * (kSplitBlocks + 64);
+  size_t keep = b_rptr + 2 * b_i + b_words + b_ids + b_counts;
   size_t b_hist = align256(sizeof(int) * transpose_hist_ints(nnz));
   size_t b_scan = align256(sizeof(int) * transpose_scan_ws_ints(nnz));
   size_t tmp = 4 * b_i + b_hist + b_scan;
@@ -1370,7 +1372,10 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
   p += b_i;
   t->perm = reinterpret_cast<int*>(p);
   p += b_i;
-  t->rows = reinterpret_cast<int*>(p);
+  SplitWord* words = reinterpret_cast<SplitWord*>(p);
+  int* ids = reinterpret_cast<int*>(p + b_words);
+  int* counts = reinterpret_cast<int*>(p + b_words + b_ids);
+  t->index = SplitIndex{words, ids, nullptr, 0, counts + kSplitBlocks};
   void* work = nullptr;
   e = cudaMallocAsync(&work, tmp, s);
   if (e == cudaSuccess) {
@@ -1381,7 +1386,10 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
     int* vb = reinterpret_cast<int*>(w + 3 * b_i);
     int* hist = reinterpret_cast<int*>(w + 4 * b_i);
     int* ws = reinterpret_cast<int*>(w + 4 * b_i + b_hist);
-    e = transpose_run(m, n, nnz, row_ptr, col_idx, t->rptrT, t->colT, t->perm, t->rows, ka, kb, va, vb, hist, ws, s);
+    e = split_build_once(GBS_F32, m, nnz, row_ptr, words, ids, counts + kSplitBlocks, counts, 0, nullptr, 0, s);
+    if (e == cudaSuccess)
+      e = transpose_run(m, n, nnz, row_ptr, col_idx, t->rptrT, t->colT, t->perm, nullptr, ka, kb, va, vb, hist, ws, s,
+                        &t->index);
     cudaError_t e2 = cudaFreeAsync(work, s);
     if (e == cudaSuccess) e = e2;
   }
@@ -1531,7 +1539,7 @@ int spmv_csr_backward(gbs_tplan* t, const int* row_ptr, const int* col_idx, cons
     e = cudaEventRecord(t->ev_fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->side, t->ev_fork, 0);
     if (e == cudaSuccess)
-      e = launch_sddmm(dtype, t->nnz, k, t->rows, col_idx, X, k == 1 ? 1 : ldx, dY, k == 1 ? 1 : lddy, dvals, t->side);
+      e = launch_sddmm(dtype, t->nnz, k, t->index, t->m, col_idx, X, k == 1 ? 1 : ldx, dY, k == 1 ? 1 : lddy, dvals, t->side);
     if (e == cudaSuccess) e = cudaEventRecord(t->ev_join, t->side);
     if (e != cudaSuccess) return cuda_fail(e, "SDDMM launch (side stream)");
   }
@@ -1563,7 +1571,7 @@ int spmv_csr_backward(gbs_tplan* t, const int* row_ptr, const int* col_idx, cons
     e = cudaStreamWaitEvent(s, t->ev_join, 0);
     if (e != cudaSuccess) return cuda_fail(e, "join of the side stream");
   } else if (dvals) {
-    e = launch_sddmm(dtype, t->nnz, k, t->rows, col_idx, X, k == 1 ? 1 : ldx, dY, k == 1 ? 1 : lddy, dvals, s);
+    e = launch_sddmm(dtype, t->nnz, k, t->index, t->m, col_idx, X, k == 1 ? 1 : ldx, dY, k == 1 ? 1 : lddy, dvals, s);
     if (e != cudaSuccess) return cuda_fail(e, "SDDMM launch");
   }
   return GBS_OK;

@@ -64,7 +64,7 @@ long long split_tiles(int nnz, int g, int share);
 cudaError_t split_build(int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* empty, int* ord,
                         int* scan_ws, cudaStream_t s);
 // The index of a one-shot call in two launches: words, ids [m], nonempty [1]; counts is a workspace
-// of kSplitBlocks ints.  Also writes the zeros of Y's empty rows (k columns).
+// of kSplitBlocks ints.  Also writes the zeros of Y's empty rows (k columns; k may be 0).
 constexpr int kSplitBlocks = 2048;
 cudaError_t split_build_once(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
                              int* counts, int k, void* Y, long long ldy, cudaStream_t s);
@@ -119,9 +119,10 @@ size_t scan_workspace_ints(long long count);
 
 // Transpose (transpose.cu).  Buffer sizes: rptrT n+1, colT/perm/rows/keys_a/keys_b/vals_a/vals_b nnz,
 // hist transpose_hist_ints(nnz), scan_ws transpose_scan_ws_ints(nnz).
+// `index`: if not NULL, the SPLIT index of A, from which the rows are then taken (`rows` unused).
 cudaError_t transpose_run(int m, int n, int nnz, const int* row_ptr, const int* col_idx, int* rptrT, int* colT,
                           int* perm, int* rows, int* keys_a, int* keys_b, int* vals_a, int* vals_b, int* hist,
-                          int* scan_ws, cudaStream_t s);
+                          int* scan_ws, cudaStream_t s, const SplitIndex* index = nullptr);
 size_t transpose_hist_ints(int nnz);
 size_t transpose_scan_ws_ints(int nnz);
 // Stable LSD radix sort of n (key >= 0, value) pairs by the keys' low `bits` bits (transpose.cu);
@@ -142,9 +143,9 @@ cudaError_t relabel_dense(int dtype, int n, int k, const void* X, long long ldx,
 // out[q] = src[perm[q]] for values of `dtype`.
 cudaError_t gather_values(int dtype, const void* src, const int* perm, int nnz, void* out, cudaStream_t s);
 
-// dvals[p] = sum_c dY[rows[p], c] * X[col_idx[p], c]  (backward.cu)
-cudaError_t launch_sddmm(int dtype, int nnz, int k, const int* rows, const int* col_idx, const void* X, long long ldx,
-                         const void* dY, long long lddy, void* dvals, cudaStream_t s);
+// dvals[p] = sum_c dY[row(p), c] * X[col_idx[p], c], row(p) from A's index  (backward.cu)
+cudaError_t launch_sddmm(int dtype, int nnz, int k, const SplitIndex& I, int m, const int* col_idx, const void* X,
+                         long long ldx, const void* dY, long long lddy, void* dvals, cudaStream_t s);
 
 // Batched persistent kernel (batched.cu).  launch == false: set the shared-memory
 // attribute and report the resident CTAs per SM in *blocks_per_sm; launch == true: launch

@@ -85,9 +85,11 @@ cudaError_t launch_split_t(const CsrView& A, const SplitIndex& I, const DenseVie
     if (e != cudaSuccess) return e;
   }
   if (a.tiles <= 1 && I.nempty == 0) return cudaSuccess;
-  const long long work = (((long long)a.tiles * a.k + 31) & ~31LL) + (long long)I.nempty * a.k;
-  split_fixup_kernel<T><<<(unsigned)((work + 255) / 256), 256, 0, s>>>(a.tiles, a.k, a.carry_row, a.carry_val, a.Y,
-                                                                     a.ldy, I.empty, I.nempty);
+  int lg = 0;
+  while (lg < 5 && (1 << lg) < a.k) ++lg;
+  const long long carry_blocks = (((long long)a.tiles << lg) + 255) >> 8, empty_blocks = (((long long)I.nempty << lg) + 255) >> 8;
+  split_fixup_kernel<T><<<(unsigned)(carry_blocks + empty_blocks), 256, 0, s>>>(
+      a.tiles, a.k, lg, a.carry_row, a.carry_val, a.Y, a.ldy, I.empty, I.nempty, (int)carry_blocks);
   return cudaGetLastError();
 }
 

@@ -115,6 +115,40 @@ __device__ __forceinline__ const int* split_ids(const SplitArgs<T>& a) {
 }
 __device__ __forceinline__ int split_row(const int* __restrict__ ids, int ord) { return ids ? __ldg(ids + ord) : ord; }
 
+// The open sum of a merge thread as the carry scan combines it.  float: the accumulator's two parts
+// are added separately, so that the compensation of every share reaches the row and only the few
+// sums of the scan round.
+template <typename T>
+struct Open;
+template <>
+struct Open<double> {
+  double s;
+  __device__ __forceinline__ explicit Open(const Acc<double>& a) : s(a.s) {}
+  __device__ __forceinline__ Open up(int d) const {
+    Open o = *this;
+    o.s = __shfl_up_sync(0xffffffffu, s, d);
+    return o;
+  }
+  __device__ __forceinline__ void add(const Open& o) { s += o.s; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct Open<float> {
+  float s, c;
+  __device__ __forceinline__ explicit Open(const Acc<float>& a) : s(a.s), c(a.c) {}
+  __device__ __forceinline__ Open up(int d) const {
+    Open o = *this;
+    o.s = __shfl_up_sync(0xffffffffu, s, d);
+    o.c = __shfl_up_sync(0xffffffffu, c, d);
+    return o;
+  }
+  __device__ __forceinline__ void add(const Open& o) {
+    s = __fadd_rn(s, o.s);
+    c = __fadd_rn(c, o.c);
+  }
+  __device__ __forceinline__ float value() const { return __fadd_rn(s, c); }
+};
+
 // SpMV: x and y contiguous, one lane per merge thread, N = 8 nonzeros each.
 template <typename T, bool PERM>
 __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile) {
@@ -126,8 +160,7 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
   const long long p0 = (long long)tile * (32 * N) + (long long)lane * N;
   uint32_t ends = 0;
   int ord = 0;
-  T head = T(0);
-  Acc<T> acc;
+  Acc<T> acc, head;
   if (p0 < a.nnz) {
     const int p = (int)p0;
     const uint2 w = __ldg(reinterpret_cast<const uint2*>(a.words) + (p >> 5));
@@ -145,7 +178,7 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
       acc.add(v[u], x[u]);
       if (ends >> u & 1u) {
         if (first) {
-          head = acc.value();
+          head = acc;
           first = false;
         } else {
           st_stream(a.Y + split_row(ids, ord), acc.value());
@@ -161,25 +194,26 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
   const uint32_t closed = __ballot_sync(0xffffffffu, ends != 0);
   const uint32_t upto = closed & (0xffffffffu >> (31 - lane));
   const int hs = upto ? 31 - __clz(upto) : 0;
-  T S = acc.value();
+  Open<T> S(acc);
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const bool take = lane - d >= hs;
     if (__any_sync(0xffffffffu, take)) {
-      const T o = __shfl_up_sync(0xffffffffu, S, d);
-      if (take) S += o;
+      const Open<T> o = S.up(d);
+      if (take) S.add(o);
     }
   }
-  const T before = __shfl_up_sync(0xffffffffu, S, 1);
+  const Open<T> before = S.up(1);
   if (ends != 0) {
-    const int r = split_row(ids, ord - __popc(ends));
-    st_stream(a.Y + r, lane > 0 ? head + before : head);
+    Open<T> out(head);
+    if (lane > 0) out.add(before);
+    st_stream(a.Y + split_row(ids, ord - __popc(ends)), out.value());
   }
   if (lane == 31) {
     // the tile's last nonzero lies in a row that goes on unless it ends there or the matrix does
     const bool open = p0 + N < a.nnz && !(ends >> (N - 1) & 1u);
     a.carry_row[tile] = open ? split_row(ids, ord) : -1;
-    a.carry_val[tile] = S;
+    a.carry_val[tile] = S.value();
   }
 }
 
@@ -209,10 +243,7 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
     else
       for (int j = 0; j < a.k - c_lo; ++j) st_stream(y + j, out[j]);
   };
-  Acc<T> acc[VEC];
-  T head[VEC];
-#pragma unroll
-  for (int j = 0; j < VEC; ++j) head[j] = T(0);
+  Acc<T> acc[VEC], head[VEC];
   int ord = 0, head_ord = -1;
   bool last_end = true;
   for (int w = w0; w < w1; ++w) {
@@ -246,19 +277,18 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
 #pragma unroll
           for (int j = 0; j < VEC; ++j) acc[j].add(v[h + u], x[u].v[j]);
           if (ends >> (h + u) & 1u) {
-            T out[VEC];
-#pragma unroll
-            for (int j = 0; j < VEC; ++j) {
-              out[j] = acc[j].value();
-              acc[j].reset();
-            }
             if (head_ord < 0) {
               head_ord = ord;
 #pragma unroll
-              for (int j = 0; j < VEC; ++j) head[j] = out[j];
+              for (int j = 0; j < VEC; ++j) head[j] = acc[j];
             } else if (col_active) {
+              T out[VEC];
+#pragma unroll
+              for (int j = 0; j < VEC; ++j) out[j] = acc[j].value();
               store_row(ord, out);
             }
+#pragma unroll
+            for (int j = 0; j < VEC; ++j) acc[j].reset();
             ++ord;
           }
         }
@@ -269,61 +299,62 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
   const uint32_t closed = __ballot_sync(0xffffffffu, head_ord >= 0);
   const uint32_t upto = closed & (0xffffffffu >> (31 - wl));
   const int hs = upto ? (31 - __clz(upto)) / G : 0;
-  T S[VEC];
-#pragma unroll
-  for (int j = 0; j < VEC; ++j) S[j] = acc[j].value();
-#pragma unroll
-  for (int d = 1; d < MT; d <<= 1) {
-    const bool take = mt - d >= hs;
-    if (__any_sync(0xffffffffu, take)) {
-#pragma unroll
-      for (int j = 0; j < VEC; ++j) {
-        const T o = __shfl_up_sync(0xffffffffu, S[j], d * G);
-        if (take) S[j] += o;
-      }
-    }
-  }
+  T tail[VEC], out[VEC];
 #pragma unroll
   for (int j = 0; j < VEC; ++j) {
-    const T before = __shfl_up_sync(0xffffffffu, S[j], G);
-    if (mt > 0) head[j] += before;
+    Open<T> S(acc[j]);
+#pragma unroll
+    for (int d = 1; d < MT; d <<= 1) {
+      const bool take = mt - d >= hs;
+      if (__any_sync(0xffffffffu, take)) {
+        const Open<T> o = S.up(d * G);
+        if (take) S.add(o);
+      }
+    }
+    const Open<T> before = S.up(G);
+    Open<T> h(head[j]);
+    if (mt > 0) h.add(before);
+    out[j] = h.value();
+    tail[j] = S.value();
   }
-  if (head_ord >= 0 && col_active) store_row(head_ord, head);
+  if (head_ord >= 0 && col_active) store_row(head_ord, out);
   if (mt == MT - 1) {
     if (wl == 32 - G) a.carry_row[tile] = w1 - w0 == nwp && (long long)w1 * 32 < a.nnz && !last_end ? split_row(ids, ord) : -1;
     if (col_active)
-      for (int j = 0; j < VEC && c_lo + j < a.k; ++j) a.carry_val[(size_t)tile * a.k + c_lo + j] = S[j];
+      for (int j = 0; j < VEC && c_lo + j < a.k; ++j) a.carry_val[(size_t)tile * a.k + c_lo + j] = tail[j];
   }
 }
 
 template <typename T, int VEC, int G, bool PERM>
-__global__ void __launch_bounds__(256, 3) split_spmm_kernel(SplitArgs<T> a) {
+__global__ void __launch_bounds__(256, PERM && sizeof(T) == 8 ? 4 : 3) split_spmm_kernel(SplitArgs<T> a) {
   const int tile = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   if (tile < a.tiles) split_spmm_tile<T, VEC, G, PERM>(a, tile);
 }
 
-// Adds the tiles' carries to the rows they belong to and writes the empty rows' zeros.  One thread
-// per (tile, column): the first tile of a run of equal carry rows sums the run; runs of more than
-// eight tiles (hub rows) are summed by the whole warp, each lane every 32nd carry and then a fixed
-// shuffle tree, so that a hub of hundreds of tiles costs a few round trips.  The row's last tile
-// has written its own part of the row already.
+// Adds the tiles' carries to the rows they belong to and writes the empty rows' zeros.  2^lg lanes
+// share a tile (or an empty row) and take its columns 2^lg apart, so the reads and writes of a warp
+// are coalesced and no index is divided (with a 64-bit division per element it took 22 us of a
+// 271 us R-MAT 20 product of k = 8).  The first tile of a run of equal carry rows sums the run;
+// runs of more than eight tiles (hub rows) are summed by the whole warp, each lane every 32nd
+// carry and then a fixed shuffle tree, so that a hub of hundreds of tiles costs a few round trips.
+// The row's last tile has written its own part of the row already.
 template <typename T>
-__global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, const int* __restrict__ carry_row,
+__global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, int lg, const int* __restrict__ carry_row,
                                                           const T* __restrict__ carry_val, T* __restrict__ Y,
-                                                          long long ldy, const int* __restrict__ empty, int nempty) {
+                                                          long long ldy, const int* __restrict__ empty, int nempty,
+                                                          int carry_blocks) {
   constexpr int W = 8;
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long work = (long long)tiles * k;
-  const long long zero0 = (work + 31) & ~31LL;  // whole warps for the carries
-  if (i >= zero0) {
-    const long long z = i - zero0;
-    if (z < (long long)nempty * k) {
-      const int e = (int)(z / k), c = (int)(z - (long long)e * k);
-      st_stream(Y + (long long)__ldg(empty + e) * ldy + c, T(0));
+  const int lanes = 1 << lg, sub = threadIdx.x & (lanes - 1);
+  if ((int)blockIdx.x >= carry_blocks) {
+    const long long e = (((long long)blockIdx.x - carry_blocks) * 256 + threadIdx.x) >> lg;
+    if (e < nempty) {
+      T* y = Y + (long long)__ldg(empty + e) * ldy;
+      for (int c = sub; c < k; c += lanes) st_stream(y + c, T(0));
     }
     return;
   }
-  const int b = i < work ? (int)(i / k) : tiles, c = i < work ? (int)(i - (long long)b * k) : 0;
+  const long long bl = ((long long)blockIdx.x * 256 + threadIdx.x) >> lg;
+  const int b = bl < tiles ? (int)bl : tiles;
   const int lane = threadIdx.x & 31;
   int r = -1;
   if (b < tiles) {
@@ -335,31 +366,34 @@ __global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, cons
     len = 1;
     while (len <= W && b + len < tiles && __ldcg(carry_row + b + len) == r) ++len;
     if (len <= W) {
-      Acc<T> s;
-      for (int q = 0; q < len; ++q) s.add_partial(__ldcg(carry_val + (size_t)(b + q) * k + c));
-      T* y = Y + (long long)r * ldy + c;
-      *y = __ldcg(y) + s.value();
+      for (int c = sub; c < k; c += lanes) {
+        Acc<T> s;
+        for (int q = 0; q < len; ++q) s.add_partial(__ldcg(carry_val + (size_t)(b + q) * k + c));
+        T* y = Y + (long long)r * ldy + c;
+        *y = __ldcg(y) + s.value();
+      }
     }
   }
-  uint32_t todo = __ballot_sync(0xffffffffu, len > W);
+  uint32_t todo = __ballot_sync(0xffffffffu, len > W && sub == 0);
   while (todo) {
     const int src = __ffs(todo) - 1;
     todo &= todo - 1;
     const int rb = __shfl_sync(0xffffffffu, b, src), rr = __shfl_sync(0xffffffffu, r, src);
-    const int rc = __shfl_sync(0xffffffffu, c, src);
-    Acc<T> s;
-    for (int base = rb; base < tiles; base += 32) {
-      const int t = base + lane;
-      const bool in = t < tiles && __ldcg(carry_row + t) == rr;
-      if (in) s.add_partial(__ldcg(carry_val + (size_t)t * k + rc));
-      if (!__all_sync(0xffffffffu, in)) break;
-    }
-    T sum = s.value();
+    for (int c = 0; c < k; ++c) {
+      Acc<T> s;
+      for (int base = rb; base < tiles; base += 32) {
+        const int t = base + lane;
+        const bool in = t < tiles && __ldcg(carry_row + t) == rr;
+        if (in) s.add_partial(__ldcg(carry_val + (size_t)t * k + c));
+        if (!__all_sync(0xffffffffu, in)) break;
+      }
+      T sum = s.value();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) {
-      T* y = Y + (long long)rr * ldy + rc;
-      *y = __ldcg(y) + sum;
+      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      if (lane == 0) {
+        T* y = Y + (long long)rr * ldy + c;
+        *y = __ldcg(y) + sum;
+      }
     }
   }
 }

@@ -127,6 +127,21 @@ __global__ void gather_int_kernel(const int* __restrict__ src, const int* __rest
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) out[i] = src[idx[i]];
 }
 
+// out[i] = row of nonzero idx[i], from the SPLIT index of A: a 16th of the bytes of a stored row per
+// nonzero, which is neither written nor kept (index and gather take the 25-28 us of the stored rows
+// on R-MAT 17).
+__global__ void gather_rows_kernel(const SplitWord* __restrict__ words, const int* __restrict__ ids_in,
+                                   const int* __restrict__ nonempty, int m, const int* __restrict__ idx, int n,
+                                   int* __restrict__ out) {
+  const int* __restrict__ ids = nonempty && *nonempty == m ? nullptr : ids_in;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const int p = idx[i];
+    const uint2 w = __ldg(reinterpret_cast<const uint2*>(words) + (p >> 5));
+    const int ord = (int)w.y + __popc(w.x & ((1u << (p & 31)) - 1u));
+    out[i] = ids ? __ldg(ids + ord) : ord;
+  }
+}
+
 template <typename T>
 __global__ void gather_vals_kernel(const T* __restrict__ src, const int* __restrict__ idx, int n, T* __restrict__ out) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) out[i] = src[idx[i]];
@@ -166,9 +181,9 @@ cudaError_t radix_sort_pairs(int n, int bits, int* keys_a, int* keys_b, int* val
 // Returns a CUDA error.  tmp must hold 2 * nnz + 2 * nnz ints + hist + scan workspace.
 cudaError_t transpose_run(int m, int n, int nnz, const int* row_ptr, const int* col_idx, int* rptrT, int* colT,
                           int* perm, int* rows, int* keys_a, int* keys_b, int* vals_a, int* vals_b, int* hist,
-                          int* scan_ws, cudaStream_t s) {
+                          int* scan_ws, cudaStream_t s, const SplitIndex* index) {
   cudaError_t e;
-  if (m > 0 && nnz > 0) {
+  if (m > 0 && nnz > 0 && !index) {
     expand_rows_kernel<<<grid_for((long long)m * 32), 256, 0, s>>>(row_ptr, m, rows);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -189,7 +204,10 @@ cudaError_t transpose_run(int m, int n, int nnz, const int* row_ptr, const int* 
   boundaries_kernel<<<grid_for((long long)nnz + 1), 256, 0, s>>>(ki, nnz, n, rptrT);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaMemcpyAsync(perm, vi, sizeof(int) * (size_t)nnz, cudaMemcpyDeviceToDevice, s)) != cudaSuccess) return e;
-  gather_int_kernel<<<grid_for(nnz), 256, 0, s>>>(rows, vi, nnz, colT);
+  if (index)
+    gather_rows_kernel<<<grid_for(nnz), 256, 0, s>>>(index->words, index->ids, index->nonempty, m, vi, nnz, colT);
+  else
+    gather_int_kernel<<<grid_for(nnz), 256, 0, s>>>(rows, vi, nnz, colT);
   return cudaGetLastError();
 }
 

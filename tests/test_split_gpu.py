@@ -133,3 +133,23 @@ def test_split_is_plans_only(gbs):
     for bad in (dict(items=7), dict(items=16), dict(threads=512)):
         with pytest.raises(gbs.GbsError):
             plan.set_config(dict(bad, variant=6))
+
+
+@DT
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5, 8, 13, 16])
+@pytest.mark.parametrize("name", ["nnz_1", "nnz_9", "nnz_257", "hubs", "singles", "rmat_13", "random_rect", "dup_unsorted"])
+def test_dvals_from_the_index(gbs, name, k, dtype):
+    """dvals with the rows taken from A's index: every width of a gathered slice (32 and 16 bytes, one
+    element), column ids on and off a 32-byte boundary."""
+    A = MATRICES[name]()
+    v = A.vals.astype(NP[dtype])
+    for ld in (k, k + 1, -(-k // 4) * 4, -(-k // 8) * 8 + 4):
+        Xw = synth.uniform(A.n * ld, seed=35, stream=ld).reshape(A.n, ld).astype(NP[dtype])
+        Ww = synth.uniform(A.m * ld, seed=36, stream=ld).reshape(A.m, ld).astype(NP[dtype])
+        _, ref, _, r = oracle.backward(A.m, A.n, A.row_ptr, A.col_idx, v, Xw[:, :k].copy(), Ww[:, :k].copy())
+        for off in (0, 1):
+            ci = torch.empty(A.nnz + 8, dtype=torch.int32, device="cuda")[off : off + A.nnz].copy_(dev(A.col_idx))
+            t = gbs.TransposePlan(dev(A.row_ptr), ci, A.n)
+            X, W = dev(Xw)[:, :k], dev(Ww)[:, :k]
+            _, dvals = t.backward(dev(v), X[:, 0] if k == 1 else X, W[:, 0] if k == 1 else W, need_dX=False)
+            within(dvals, ref, r, dtype, f"{name} k={k} ld={ld} off={off}")
