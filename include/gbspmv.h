@@ -191,6 +191,14 @@ int gbs_fp64_probe(double* out, int blocks, int threads, int iters, void* stream
 int gbs_wait_probe(long long limit_ns, void* stream);
 
 /*
+ * The library takes the scratch of calls without a plan, and what plans own,
+ * from a memory pool of its own on each device, which keeps up to 256 MB
+ * that are not in use for the next call.  This gives those back to the
+ * driver (current device; nothing in use is touched).
+ */
+int gbs_release_scratch(void);
+
+/*
  * Diagnostic: useful cacheline density (UCLD, Sec. 4.1, the figure that ties
  * the gain of vectorised SpMV to it).  x is cut into aligned lines of
  * `line_elems` elements (line j = x[j*line_elems .. (j+1)*line_elems - 1]); a

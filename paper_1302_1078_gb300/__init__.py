@@ -27,7 +27,7 @@ __all__ = [
 
 def lib():
     """The loaded C library (built on first use if needed)."""
-    return _capi.load()
+    return _capi._lib or _capi.load()
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -44,24 +44,28 @@ def _ptr(t) -> int:
     return t.data_ptr() if t.numel() else 0
 
 
+# the current stream's handle without a Stream object, whose construction is a good part of the host
+# time of a small call
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None) or \
+    (lambda index: torch.cuda.current_stream(index).cuda_stream)
+
+
 def _stream(device: torch.device, stream=None) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream(device)
-    return int(stream.cuda_stream)
+    return _raw_stream(device.index) if stream is None else int(stream.cuda_stream)
 
 
 def _need_cuda(*ts):
-    dev = None
+    first = index = None
     for t in ts:
         if t is None:
             continue
         if not t.is_cuda:
             raise ValueError("gbspmv operates on CUDA tensors only")
-        if dev is None:
-            dev = t.device
-        elif t.device != dev:
+        if first is None:
+            first, index = t, t.get_device()
+        elif t.get_device() != index:
             raise ValueError("all tensors must be on the same device")
-    return dev
+    return None if first is None else first.device
 
 
 def _check_index(row_ptr: torch.Tensor, col_idx: torch.Tensor):

@@ -3,6 +3,7 @@
 // validation.  Every product runs in the kernels of rows_kernel.cuh and
 // merge_kernel.cuh; nothing here computes on the host.
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cmath>
 #include <cstdint>
@@ -231,8 +232,8 @@ int run_product(const CsrView& A, int dtype, int k, const void* X, long long ldx
   MergeBuffers* use = mb;
   if (use == nullptr) {
     local.bytes = merge_scratch_bytes(ctas, kp_max, dtype);
-    e = cudaMallocAsync(&local.base, local.bytes, s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (merge scratch)");
+    e = scratch_alloc(&local.base, local.bytes, s);
+    if (e != cudaSuccess) return cuda_fail(e, "scratch (merge scratch)");
     merge_carve(local, ctas, kp_max, dtype);
     use = &local;
     coords_ready = false;
@@ -254,8 +255,8 @@ int run_product(const CsrView& A, int dtype, int k, const void* X, long long ldx
     if (e != cudaSuccess) rc = cuda_fail(e, "MERGE launch");
   }
   if (use == &local) {
-    e = cudaFreeAsync(local.base, s);
-    if (e != cudaSuccess && rc == GBS_OK) rc = cuda_fail(e, "cudaFreeAsync");
+    e = scratch_free(local.base, s);
+    if (e != cudaSuccess && rc == GBS_OK) rc = cuda_fail(e, "scratch");
   }
   return rc;
 }
@@ -279,7 +280,7 @@ int run_split_once(const CsrView& A, int dtype, int k, const void* X, long long 
   const size_t b_ids = up(sizeof(int) * (size_t)A.m), b_counts = sizeof(int) * (kSplitBlocks + 64);
   const size_t b_row = up(sizeof(int) * tiles);
   void* base = nullptr;
-  cudaError_t e = cudaMallocAsync(&base, b_words + b_ids + b_counts + b_row + tiles * (size_t)kp_max * es, s);
+  cudaError_t e = scratch_alloc(&base, b_words + b_ids + b_counts + b_row + tiles * (size_t)kp_max * es, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(GBS_ENOMEM, "scratch of a one-shot product");
@@ -292,20 +293,21 @@ int run_split_once(const CsrView& A, int dtype, int k, const void* X, long long 
   q += b_words + b_ids + b_counts;
   const SplitIndex I{words, ids, nullptr, 0, nonempty};
   const SplitScratch S{reinterpret_cast<int*>(q), q + b_row};
-  e = split_build_once(dtype, A.m, A.nnz, A.row_ptr, words, ids, nonempty, counts, k, Y, ldy, s);
+  e = split_build(dtype, A.m, A.nnz, A.row_ptr, words, ids, nonempty, nullptr, counts, k, Y, ldy, s);
   for (int c0 = 0; e == cudaSuccess && c0 < k; c0 += P) {
     DenseView D{std::min(P, k - c0), static_cast<const char*>(X) + c0 * es, ldx, static_cast<char*>(Y) + c0 * es, ldy};
     e = dtype == GBS_F64 ? launch_split_f64(A, I, D, vec16, 64, share, S, s)
                          : launch_split_f32(A, I, D, vec16, 64, share, S, s);
   }
-  const cudaError_t e2 = cudaFreeAsync(base, s);
+  const cudaError_t e2 = scratch_free(base, s);
   if (e == cudaSuccess) e = e2;
   return e == cudaSuccess ? GBS_OK : cuda_fail(e, "one-shot product");
 }
 
 // --------------------------------------------------------------- statistics
 
-__global__ void stats_kernel(const int* __restrict__ rp, int m, unsigned long long* __restrict__ acc, int* __restrict__ maxrow) {
+// acc: sums of squared lengths, empty rows, rows over 32, 256 and 4096, and the longest row.
+__global__ void __launch_bounds__(256) stats_kernel(const int* __restrict__ rp, int m, unsigned long long* __restrict__ acc) {
   unsigned long long sq = 0, empty = 0, o32 = 0, o256 = 0, o4k = 0;
   int mx = 0;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (long long)gridDim.x * blockDim.x) {
@@ -325,13 +327,28 @@ __global__ void stats_kernel(const int* __restrict__ rp, int m, unsigned long lo
     o4k += __shfl_xor_sync(0xffffffffu, o4k, o);
     mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   }
+  // one set of atomics per block: with one per warp they took 15 of the 20 us on 131,072 rows
+  __shared__ unsigned long long part[6][8];
+  const int w = threadIdx.x >> 5;
   if ((threadIdx.x & 31) == 0) {
-    atomicAdd(acc + 0, sq);
-    atomicAdd(acc + 1, empty);
-    atomicAdd(acc + 2, o32);
-    atomicAdd(acc + 3, o256);
-    atomicAdd(acc + 4, o4k);
-    atomicMax(maxrow, mx);
+    part[0][w] = sq;
+    part[1][w] = empty;
+    part[2][w] = o32;
+    part[3][w] = o256;
+    part[4][w] = o4k;
+    part[5][w] = (unsigned long long)mx;
+  }
+  __syncthreads();
+  if (threadIdx.x < 6) {
+    unsigned long long v = part[threadIdx.x][0];
+    for (int i = 1; i < 8; ++i) {
+      const unsigned long long o = part[threadIdx.x][i];
+      v = threadIdx.x == 5 ? max(v, o) : v + o;
+    }
+    if (threadIdx.x == 5)
+      atomicMax(acc + 5, v);
+    else
+      atomicAdd(acc + threadIdx.x, v);
   }
 }
 
@@ -359,25 +376,22 @@ int compute_stats(int m, int n, int nnz, const int* rp, gbs_stats* out, cudaStre
   out->nnz = nnz;
   if (m == 0) return GBS_OK;
   void* buf = nullptr;
-  cudaError_t e = cudaMallocAsync(&buf, 64, s);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (stats)");
+  cudaError_t e = scratch_alloc(&buf, 64, s);
+  if (e != cudaSuccess) return cuda_fail(e, "scratch (stats)");
   unsigned long long* acc = static_cast<unsigned long long*>(buf);
-  int* mx = reinterpret_cast<int*>(acc + 5);
-  unsigned long long h[5];
-  int hm = 0;
+  unsigned long long h[6];
   e = cudaMemsetAsync(buf, 0, 64, s);
   if (e == cudaSuccess) {
-    int blocks = std::min(1024, (m + 255) / 256);
-    stats_kernel<<<blocks, 256, 0, s>>>(rp, m, acc, mx);
+    const int blocks = std::min(152 * 2, (m + 255) / 256);
+    stats_kernel<<<blocks, 256, 0, s>>>(rp, m, acc);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(h, acc, sizeof(h), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&hm, mx, sizeof(int), cudaMemcpyDeviceToHost, s);
-  cudaError_t e2 = cudaFreeAsync(buf, s);
+  cudaError_t e2 = scratch_free(buf, s);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "CSR statistics");
-  out->max_row = hm;
+  out->max_row = (int)h[5];
   out->empty_rows = (int)h[1];
   out->mean_row = (double)nnz / m;
   double var = (double)h[0] / m - out->mean_row * out->mean_row;
@@ -416,8 +430,8 @@ __global__ void block_max_nnz_kernel(const int* __restrict__ rp, int m, int rpc,
 // Largest nonzero count of a block of rpc consecutive rows (synchronises s).
 int block_max_nnz(const int* rp, int m, int rpc, int* out, cudaStream_t s) {
   int* d = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d), sizeof(int), s);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (block max)");
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&d), sizeof(int), s);
+  if (e != cudaSuccess) return cuda_fail(e, "scratch (block max)");
   e = cudaMemsetAsync(d, 0, sizeof(int), s);
   if (e == cudaSuccess) {
     const int nb = (m + rpc - 1) / rpc;
@@ -425,7 +439,7 @@ int block_max_nnz(const int* rp, int m, int rpc, int* out, cudaStream_t s) {
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, d, sizeof(int), cudaMemcpyDeviceToHost, s);
-  cudaError_t e2 = cudaFreeAsync(d, s);
+  cudaError_t e2 = scratch_free(d, s);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return e == cudaSuccess ? GBS_OK : cuda_fail(e, "block max nnz");
@@ -512,8 +526,8 @@ int gbs_wait_probe(long long limit_ns, void* stream) {
   if (limit_ns < 1 || limit_ns > 2000000000LL) return fail(GBS_EINVAL, "limit_ns must be in [1, 2e9]");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int* d = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d), sizeof(int), s);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (wait probe)");
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&d), sizeof(int), s);
+  if (e != cudaSuccess) return cuda_fail(e, "scratch (wait probe)");
   e = cudaMemsetAsync(d, 0xff, sizeof(int), s);
   if (e == cudaSuccess) {
     wait_probe_kernel<<<1, 32, 0, s>>>(d, (unsigned long long)limit_ns);
@@ -521,7 +535,7 @@ int gbs_wait_probe(long long limit_ns, void* stream) {
   }
   int h = -1;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(int), cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(d, s);
+  scratch_free(d, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "wait probe");
   if (h == 1) return fail(GBS_ETIMEOUT, "wait probe: the bounded wait gave up (expected)");
@@ -558,8 +572,8 @@ int gbs_validate_csr(int m, int n, int nnz, const int* row_ptr, const int* col_i
   if (row_ptr == nullptr || (nnz > 0 && col_idx == nullptr)) return fail(GBS_EINVAL, "NULL pointer");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int* flags = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&flags), sizeof(int), s);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (validate)");
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&flags), sizeof(int), s);
+  if (e != cudaSuccess) return cuda_fail(e, "scratch (validate)");
   int h = 0;
   e = cudaMemsetAsync(flags, 0, sizeof(int), s);
   if (e == cudaSuccess) {
@@ -569,7 +583,7 @@ int gbs_validate_csr(int m, int n, int nnz, const int* row_ptr, const int* col_i
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, flags, sizeof(int), cudaMemcpyDeviceToHost, s);
-  cudaError_t e2 = cudaFreeAsync(flags, s);
+  cudaError_t e2 = scratch_free(flags, s);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "validate");
@@ -600,12 +614,12 @@ int gbs_ucld(int m, int n, int nnz, const int* row_ptr, const int* col_idx, int 
   unsigned long long h[3] = {0, 0, 0};
   if (m > 0 && nnz > 0) {
     unsigned long long* d = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&d), sizeof(h), s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync (ucld)");
+    cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&d), sizeof(h), s);
+    if (e != cudaSuccess) return cuda_fail(e, "scratch (ucld)");
     e = cudaMemsetAsync(d, 0, sizeof(h), s);
     if (e == cudaSuccess) e = launch_ucld(row_ptr, col_idx, m, line_elems, d, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
-    cudaError_t e2 = cudaFreeAsync(d, s);
+    cudaError_t e2 = scratch_free(d, s);
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "ucld");
@@ -755,16 +769,40 @@ struct gbs_plan {
   void* split_carry = nullptr;
   SplitScratch split_scratch{};
   bool tuning = false;   // the tuner is trying configurations: keep the relabelling between them
+  // What the plan owns is stream-ordered memory.  It is freed on the stream that makes the plan
+  // while it is being made and on the legacy default stream afterwards, which is ordered behind
+  // every use of the plan only if there was none on another stream; if there was (away), the
+  // device is waited for first.
+  cudaStream_t owner = nullptr;
+  mutable std::atomic<bool> away{false};
 };
 
 namespace {
 
+void plan_free(gbs_plan* p, void* q) { scratch_free(q, p->owner); }
+
+// Before memory that earlier products of a plan may still read is freed.
+void quiesce(std::atomic<bool>& away) {
+  if (away.exchange(false)) cudaDeviceSynchronize();
+}
+
+// The current device is `dev` for the guard's lifetime.
+struct DeviceGuard {
+  int prev = -1, dev;
+  explicit DeviceGuard(int d) : dev(d) {
+    if (cudaGetDevice(&prev) == cudaSuccess && prev != dev) cudaSetDevice(dev);
+  }
+  ~DeviceGuard() {
+    if (prev >= 0 && prev != dev) cudaSetDevice(prev);
+  }
+};
+
 // Allocate (or free) the plan's merge scratch for its configuration and compute the
 // partition.  Scratch is sized for 128-bit column panels, the widest case.
 void relabel_release(gbs_plan* p) {
-  if (p->newid) cudaFree(p->newid);
-  if (p->col_rl) cudaFree(p->col_rl);
-  if (p->xbuf) cudaFree(p->xbuf);
+  if (p->newid) plan_free(p, p->newid);
+  if (p->col_rl) plan_free(p, p->col_rl);
+  if (p->xbuf) plan_free(p, p->xbuf);
   p->newid = p->col_rl = nullptr;
   p->xbuf = nullptr;
 }
@@ -775,9 +813,9 @@ int relabel_prepare(gbs_plan* p, cudaStream_t s) {
   const size_t es = dsize(p->dtype);
   const int v = (int)(16 / es);
   p->ldxp = p->k == 1 ? 1 : (long long)((p->k + v - 1) / v) * v;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&p->newid), sizeof(int) * (size_t)p->n);
-  if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&p->col_rl), sizeof(int) * (size_t)std::max(p->nnz, 1));
-  if (e == cudaSuccess) e = cudaMalloc(&p->xbuf, es * (size_t)p->n * (size_t)p->ldxp);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&p->newid), sizeof(int) * (size_t)p->n, s);
+  if (e == cudaSuccess) e = scratch_alloc(reinterpret_cast<void**>(&p->col_rl), sizeof(int) * (size_t)std::max(p->nnz, 1), s);
+  if (e == cudaSuccess) e = scratch_alloc(&p->xbuf, es * (size_t)p->n * (size_t)p->ldxp, s);
   if (e == cudaSuccess) e = relabel_build(p->n, p->nnz, p->col_idx, p->newid, p->col_rl, s);
   if (e != cudaSuccess) {
     relabel_release(p);
@@ -787,8 +825,8 @@ int relabel_prepare(gbs_plan* p, cudaStream_t s) {
 }
 
 void split_release(gbs_plan* p) {
-  if (p->split_base) cudaFree(p->split_base);
-  if (p->split_carry) cudaFree(p->split_carry);
+  if (p->split_base) plan_free(p, p->split_base);
+  if (p->split_carry) plan_free(p, p->split_carry);
   p->split_base = p->split_carry = nullptr;
   p->split = SplitIndex{};
 }
@@ -806,32 +844,31 @@ int split_prepare(gbs_plan* p, cudaStream_t s) {
     const size_t b_words = up(sizeof(SplitWord) * (size_t)(((long long)p->nnz + 31) / 32));
     const size_t b_ids = nempty ? up(sizeof(int) * (size_t)nrows) : 0;
     const size_t b_empty = up(sizeof(int) * (size_t)nempty);
-    const size_t b_ord = nempty ? up(sizeof(int) * (size_t)p->m) : 0;
-    void* tmp = nullptr;
-    e = cudaMalloc(&p->split_base, b_words + b_ids + b_empty + 256);
-    if (e == cudaSuccess && nempty) e = cudaMallocAsync(&tmp, b_ord + sizeof(int) * scan_workspace_ints(p->m), s);
+    void* counts = nullptr;
+    e = scratch_alloc(&p->split_base, b_words + b_ids + b_empty, s);
+    if (e == cudaSuccess) e = scratch_alloc(&counts, sizeof(int) * kSplitBlocks, s);
     if (e == cudaSuccess) {
       char* q = static_cast<char*>(p->split_base);
       SplitWord* words = reinterpret_cast<SplitWord*>(q);
       int* ids = nempty ? reinterpret_cast<int*>(q + b_words) : nullptr;
       int* empty = nempty ? reinterpret_cast<int*>(q + b_words + b_ids) : nullptr;
       p->split = SplitIndex{words, ids, empty, nempty};
-      e = split_build(p->m, p->nnz, p->row_ptr, words, ids, empty, static_cast<int*>(tmp),
-                      reinterpret_cast<int*>(static_cast<char*>(tmp) + b_ord), s);
+      e = split_build(p->dtype, p->m, p->nnz, p->row_ptr, words, ids, nullptr, empty, static_cast<int*>(counts), 0,
+                      nullptr, 0, s);
     }
-    if (tmp) {
-      const cudaError_t e2 = cudaFreeAsync(tmp, s);
+    if (counts) {
+      const cudaError_t e2 = scratch_free(counts, s);
       if (e == cudaSuccess) e = e2;
     }
   }
   // carries: a call without 128-bit column access has more lanes per merge thread, so more tiles
-  if (p->split_carry) cudaFree(p->split_carry);
+  if (p->split_carry) plan_free(p, p->split_carry);
   p->split_carry = nullptr;
   const int kp = std::min(panel_cols(p->dtype, true), p->k);
   const int g = p->k == 1 ? 1 : std::min(32, pow2ceil(kp));
   const size_t tiles = (size_t)split_tiles(p->nnz, g, c.items);
   const size_t b_row = (sizeof(int) * tiles + 255) & ~(size_t)255;
-  if (e == cudaSuccess) e = cudaMalloc(&p->split_carry, b_row + tiles * (size_t)kp * dsize(p->dtype));
+  if (e == cudaSuccess) e = scratch_alloc(&p->split_carry, b_row + tiles * (size_t)kp * dsize(p->dtype), s);
   if (e == cudaSuccess) {
     p->split_scratch.carry_row = static_cast<int*>(p->split_carry);
     p->split_scratch.carry_val = static_cast<char*>(p->split_carry) + b_row;
@@ -846,7 +883,7 @@ int split_prepare(gbs_plan* p, cudaStream_t s) {
 
 int plan_prepare(gbs_plan* p, cudaStream_t s) {
   if (p->mb.base) {
-    cudaFree(p->mb.base);
+    plan_free(p, p->mb.base);
     p->mb = MergeBuffers{};
   }
   p->coords_ready = false;
@@ -863,6 +900,11 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
     int lanes = p->cfg.lanes;
     if (p->k > 1) lanes = std::max(lanes, col_lanes(std::min(panel_cols(p->dtype, true), p->k), p->dtype, true));
     const int rpc = p->cfg.threads / lanes;
+    if (!p->status) {
+      cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&p->status), 256, s);
+      if (e == cudaSuccess) e = cudaMemsetAsync(p->status, 0, 256, s);
+      if (e != cudaSuccess) return cuda_fail(e, "plan status word");
+    }
     int mx = 0;
     int rc = block_max_nnz(p->row_ptr, p->m, rpc, &mx, s);
     if (rc) return rc;
@@ -882,7 +924,7 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
   // cannot use it take the stream-ordered path
   const MergeGeom G = merge_geom(p->cfg, p->m, p->nnz, p->dtype, p->k, p->k > 1);
   p->mb.bytes = merge_scratch_bytes(G.ctas, G.kp_max, p->dtype);
-  cudaError_t e = cudaMalloc(&p->mb.base, p->mb.bytes);
+  cudaError_t e = scratch_alloc(&p->mb.base, p->mb.bytes, s);
   if (e != cudaSuccess) {
     p->mb = MergeBuffers{};
     return cuda_fail(e, "cudaMalloc (plan scratch)");
@@ -897,6 +939,7 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
 }
 
 int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, void* Y, long long ldy, cudaStream_t s) {
+  if (s != nullptr) p->away.store(true, std::memory_order_relaxed);
   CsrView A{p->m, p->n, p->nnz, p->row_ptr, p->col_idx, vals, p->perm};
   // the caller's operands decide the column access (and with it the merge geometry), also when
   // the product reads the relabelled copy of X, so that relabelling never changes a result
@@ -932,6 +975,19 @@ int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, 
     return run_product(A, p->dtype, p->k, X, ldx, Y, ldy, p->cfg, &mb, p->coords_ready, s, nullptr, as);
   }
   return run_product(A, p->dtype, p->k, X, ldx, Y, ldy, p->cfg, nullptr, false, s, p->status, as);
+}
+
+// The untuned configuration of a plan: heuristic_config's, except that skewed rows take the forms a
+// plan can afford: SPLIT for block vectors (R-MAT 20, k = 8, FP32: 223 us staged merge-path, 134 us
+// SPLIT); a vector takes the direct merge walk, which needs no index beyond the tiles' coordinates.
+gbs_config plan_default_config(const gbs_plan* p) {
+  gbs_config c = heuristic_config(p->stats, p->dtype, p->k);
+  if (c.variant != GBS_VARIANT_MERGE) return c;
+  c = gbs_config{};
+  c.variant = p->k > 1 ? GBS_VARIANT_SPLIT : GBS_VARIANT_MERGE_DIRECT;
+  c.threads = 128;
+  c.items = p->k > 1 ? 0 : 8;
+  return normalize(c, p->dtype);
 }
 
 // Candidate configurations for the tuner.
@@ -1135,6 +1191,16 @@ int plan_tune(gbs_plan* p, cudaStream_t s) {
   return rc;
 }
 
+void plan_destroy_impl(gbs_plan* p) {
+  DeviceGuard guard(p->device);
+  quiesce(p->away);
+  relabel_release(p);
+  split_release(p);
+  if (p->mb.base) plan_free(p, p->mb.base);
+  if (p->status) plan_free(p, p->status);
+  delete p;
+}
+
 // gbs_plan_create with an optional permutation through which the values are read
 // (perm != nullptr: the plan is restricted to the ROWS and MERGE_DIRECT variants).
 int plan_create_impl(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr, const int* col_idx, int dtype, int k,
@@ -1162,29 +1228,18 @@ int plan_create_impl(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr,
   p->flags = flags;
   p->perm = perm;
   cudaGetDevice(&p->device);
-  if (cudaMalloc(reinterpret_cast<void**>(&p->status), 256) != cudaSuccess ||
-      cudaMemsetAsync(p->status, 0, 256, s) != cudaSuccess) {
-    if (p->status) cudaFree(p->status);
-    delete p;
-    return fail(GBS_ENOMEM, "plan status word");
-  }
+  p->owner = s;
   rc = compute_stats(m, n, nnz, row_ptr, &p->stats, s);
   if (rc == GBS_OK) {
-    p->cfg = heuristic_config(p->stats, dtype, k);
-    // values through a permutation: the direct merge form gathers them in its walk, with
-    // more of them in flight than the staged form's synchronous gather (the tuner may still
-    // pick the staged form)
-    if (perm && p->cfg.variant == GBS_VARIANT_MERGE) p->cfg.variant = GBS_VARIANT_MERGE_DIRECT;
+    p->cfg = plan_default_config(p);
     rc = (flags & GBS_PLAN_TUNE) && m > 0 ? plan_tune(p, s) : plan_prepare(p, s);
   }
   if (rc != GBS_OK) {
-    relabel_release(p);
-    split_release(p);
-    if (p->mb.base) cudaFree(p->mb.base);
-    cudaFree(p->status);
-    delete p;
+    plan_destroy_impl(p);
     return rc;
   }
+  p->owner = nullptr;  // made, and its stream waited for
+  p->away.store(false, std::memory_order_relaxed);
   *plan = p;
   return GBS_OK;
 }
@@ -1200,17 +1255,19 @@ int gbs_plan_create(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr, 
 
 int gbs_plan_destroy(gbs_plan* plan) {
   if (!plan) return GBS_OK;
-  relabel_release(plan);
-  split_release(plan);
-  if (plan->mb.base) cudaFree(plan->mb.base);
-  if (plan->status) cudaFree(plan->status);
-  delete plan;
+  plan_destroy_impl(plan);
   return GBS_OK;
 }
 
 int gbs_plan_status(gbs_plan* plan, int* status, void* stream) {
   if (!plan || !status) return fail(GBS_EINVAL, "NULL pointer");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  *status = 0;
+  if (!plan->status) {  // no bounded waits in the plan's configuration
+    const cudaError_t e = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? GBS_OK : cuda_fail(e, "plan status");
+  }
+  if (s != nullptr) plan->away.store(true, std::memory_order_relaxed);
   cudaError_t e = cudaMemcpyAsync(status, plan->status, sizeof(int), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(plan->status, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -1241,10 +1298,11 @@ int gbs_plan_relabel_ids(const gbs_plan* plan, int* newid, void* stream) {
 
 int gbs_plan_set_config(gbs_plan* plan, const gbs_config* cfg) {
   if (!plan || !cfg) return fail(GBS_EINVAL, "NULL pointer");
-  gbs_config c = cfg->variant == GBS_VARIANT_AUTO ? heuristic_config(plan->stats, plan->dtype, plan->k)
-                                                  : normalize(*cfg, plan->dtype);
+  gbs_config c = cfg->variant == GBS_VARIANT_AUTO ? plan_default_config(plan) : normalize(*cfg, plan->dtype);
   int rc = check_cfg(c);
   if (rc) return rc;
+  DeviceGuard guard(plan->device);
+  quiesce(plan->away);
   plan->cfg = c;
   return plan_prepare(plan, nullptr);
 }
@@ -1273,6 +1331,7 @@ struct gbs_tplan {
   int* colT = nullptr;       // nnz
   int* perm = nullptr;       // nnz
   SplitIndex index{};        // A's rows (the dvals pass), for m rows
+  std::atomic<bool> away{false};  // used on another stream than the legacy default one (see gbs_plan)
   void* base = nullptr;
   void* valsT = nullptr;     // nnz values, only for a prepared plan that permutes the values first
   gbs_stats statsT{};
@@ -1289,6 +1348,10 @@ struct gbs_tplan {
 };
 
 namespace {
+// Nonzeros from which a backward pass runs dvals beside dX on a second stream.  Below, the overlap
+// gives less than the stream, its events and their calls cost (R-MAT 17, 1.9 M nonzeros: dvals 15 us).
+constexpr int kForkNnz = 4000000;
+
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Time `fn` (enqueued on s) as the median of 3 runs after one warm-up; returns ms or -1.
@@ -1317,10 +1380,12 @@ float time_median(F fn, cudaStream_t s) {
 
 // Keep `plan` as the prepared plan of A^T for (dtype, k), replacing an earlier one.
 int tplan_install(gbs_tplan* t, int dtype, int k, gbs_plan* plan, bool gather) {
-  if (gather && !t->valsT && cudaMalloc(&t->valsT, (size_t)std::max(t->nnz, 1) * 8) != cudaSuccess) {
+  // (waited for, as the next product may run on any stream)
+  if (gather && !t->valsT &&
+      (scratch_alloc(&t->valsT, (size_t)std::max(t->nnz, 1) * 8, nullptr) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)) {
     t->valsT = nullptr;
     gbs_plan_destroy(plan);
-    return fail(GBS_ENOMEM, "cudaMalloc (permuted values)");
+    return fail(GBS_ENOMEM, "memory of the permuted values");
   }
   for (auto& pp : t->plans)
     if (pp.dtype == dtype && pp.k == k) {
@@ -1360,10 +1425,10 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
   size_t b_hist = align256(sizeof(int) * transpose_hist_ints(nnz));
   size_t b_scan = align256(sizeof(int) * transpose_scan_ws_ints(nnz));
   size_t tmp = 4 * b_i + b_hist + b_scan;
-  cudaError_t e = cudaMalloc(&t->base, keep);
+  cudaError_t e = scratch_alloc(&t->base, keep, s);
   if (e != cudaSuccess) {
     delete t;
-    return cuda_fail(e, "cudaMalloc (transpose plan)");
+    return cuda_fail(e, "memory of the transpose plan");
   }
   char* p = static_cast<char*>(t->base);
   t->rptrT = reinterpret_cast<int*>(p);
@@ -1377,7 +1442,7 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
   int* counts = reinterpret_cast<int*>(p + b_words + b_ids);
   t->index = SplitIndex{words, ids, nullptr, 0, counts + kSplitBlocks};
   void* work = nullptr;
-  e = cudaMallocAsync(&work, tmp, s);
+  e = scratch_alloc(&work, tmp, s);
   if (e == cudaSuccess) {
     char* w = static_cast<char*>(work);
     int* ka = reinterpret_cast<int*>(w);
@@ -1386,21 +1451,21 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
     int* vb = reinterpret_cast<int*>(w + 3 * b_i);
     int* hist = reinterpret_cast<int*>(w + 4 * b_i);
     int* ws = reinterpret_cast<int*>(w + 4 * b_i + b_hist);
-    e = split_build_once(GBS_F32, m, nnz, row_ptr, words, ids, counts + kSplitBlocks, counts, 0, nullptr, 0, s);
+    e = split_build(GBS_F32, m, nnz, row_ptr, words, ids, counts + kSplitBlocks, nullptr, counts, 0, nullptr, 0, s);
     if (e == cudaSuccess)
       e = transpose_run(m, n, nnz, row_ptr, col_idx, t->rptrT, t->colT, t->perm, nullptr, ka, kb, va, vb, hist, ws, s,
                         &t->index);
-    cudaError_t e2 = cudaFreeAsync(work, s);
+    cudaError_t e2 = scratch_free(work, s);
     if (e == cudaSuccess) e = e2;
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
-    cudaFree(t->base);
+    scratch_free(t->base, s);
     delete t;
     return cuda_fail(e, "transpose");
   }
-  rc = compute_stats(n, m, nnz, t->rptrT, &t->statsT, s);
-  if (rc == GBS_OK) {
+  rc = compute_stats(n, m, nnz, t->rptrT, &t->statsT, s);  // waits for s (without columns: nothing ran)
+  if (rc == GBS_OK && n == 0 && cudaStreamSynchronize(s) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "transpose");
+  if (rc == GBS_OK && nnz >= kForkNnz) {
     e = cudaStreamCreateWithFlags(&t->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->ev_join, cudaEventDisableTiming);
@@ -1416,6 +1481,7 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
 
 int gbs_tplan_arrays(const gbs_tplan* t, const int** rowptrT, const int** colT, const int** perm) {
   if (!t) return fail(GBS_EINVAL, "plan is NULL");
+  const_cast<gbs_tplan*>(t)->away.store(true, std::memory_order_relaxed);  // the caller may read them on any stream
   if (rowptrT) *rowptrT = t->rptrT;
   if (colT) *colT = t->colT;
   if (perm) *perm = t->perm;
@@ -1425,6 +1491,7 @@ int gbs_tplan_arrays(const gbs_tplan* t, const int** rowptrT, const int** colT, 
 int gbs_tplan_export(const gbs_tplan* t, int* rowptrT, int* colT, int* perm, void* stream) {
   if (!t) return fail(GBS_EINVAL, "plan is NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (s != nullptr) const_cast<gbs_tplan*>(t)->away.store(true, std::memory_order_relaxed);
   cudaError_t e = cudaSuccess;
   if (rowptrT) e = cudaMemcpyAsync(rowptrT, t->rptrT, sizeof(int) * ((size_t)t->n + 1), cudaMemcpyDefault, s);
   if (e == cudaSuccess && colT && t->nnz)
@@ -1440,8 +1507,10 @@ int gbs_tplan_destroy(gbs_tplan* t) {
   if (t->ev_join) cudaEventDestroy(t->ev_join);
   if (t->side) cudaStreamDestroy(t->side);
   for (auto& pp : t->plans) gbs_plan_destroy(pp.plan);
-  if (t->valsT) cudaFree(t->valsT);
-  if (t->base) cudaFree(t->base);
+  DeviceGuard guard(t->device);
+  quiesce(t->away);
+  if (t->valsT) scratch_free(t->valsT, nullptr);
+  if (t->base) scratch_free(t->base, nullptr);
   delete t;
   return GBS_OK;
 }
@@ -1530,6 +1599,7 @@ int spmv_csr_backward(gbs_tplan* t, const int* row_ptr, const int* col_idx, cons
   if (dX && t->m > 0 && !dY) return fail(GBS_EINVAL, "dY is NULL");
   (void)row_ptr;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (s != nullptr) t->away.store(true, std::memory_order_relaxed);
   cudaError_t e;
   // both outputs: the dvals pass runs on the plan's side stream while dX runs on `stream`; the
   // two read the same inputs and write different outputs, and `stream` waits for the side
@@ -1559,8 +1629,12 @@ int spmv_csr_backward(gbs_tplan* t, const int* row_ptr, const int* col_idx, cons
       // A's values read in place through perm, configuration from A^T's row statistics
       CsrView AT{t->n, t->m, t->nnz, t->rptrT, t->colT, vals, t->perm};
       gbs_config c = heuristic_config(t->statsT, dtype, k);
+      rc = GBS_ENOMEM;
+      // skewed rows: the nonzero-split walk on an index made by this call (merge-path if its
+      // scratch cannot be had)
+      if (c.variant == GBS_VARIANT_MERGE) rc = run_split_once(AT, dtype, k, dY, k == 1 ? 1 : lddy, dX, k == 1 ? 1 : lddx, s);
       if (c.variant == GBS_VARIANT_MERGE) c.variant = GBS_VARIANT_MERGE_DIRECT;
-      rc = run_product(AT, dtype, k, dY, k == 1 ? 1 : lddy, dX, k == 1 ? 1 : lddx, c, nullptr, false, s);
+      if (rc == GBS_ENOMEM) rc = run_product(AT, dtype, k, dY, k == 1 ? 1 : lddy, dX, k == 1 ? 1 : lddx, c, nullptr, false, s);
     }
     if (rc) {
       if (fork) cudaStreamWaitEvent(s, t->ev_join, 0);  // never leave the side stream unjoined
@@ -1641,7 +1715,7 @@ int gbs_bcsr_create(gbs_bcsr** out, int m, int n, int nnz, const int* row_ptr, c
       e = bcsr_fill(m, n, nnz, row_ptr, col_idx, vals, dtype, a, b, h->bptr, h->bcol, h->bval, nb, scratch, s);
   }
   if (scratch) {
-    cudaError_t e2 = cudaFreeAsync(scratch, s);
+    cudaError_t e2 = scratch_free(scratch, s);
     if (e == cudaSuccess) e = e2;
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

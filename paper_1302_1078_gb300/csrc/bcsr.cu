@@ -184,7 +184,7 @@ cudaError_t bcsr_count(int m, int n, int nnz, const int* row_ptr, const int* col
   const size_t ints = (mb + 1) + c + (nbc + 1) + 2 * c + (mb + 1) + 2 * c + (mb + 1) + 64 +
                       scan_workspace_ints((long long)mb + 1) + tx_ints(nnz);
   int* base = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&base), ints * sizeof(int), s);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&base), ints * sizeof(int), s);
   if (e != cudaSuccess) return e;
   *scratch = base;
   int* p = base;

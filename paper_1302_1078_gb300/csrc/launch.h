@@ -5,6 +5,10 @@
 
 namespace gbs {
 
+// Stream-ordered device memory from the library's own pool (scratch.cu).
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t s);
+cudaError_t scratch_free(void* p, cudaStream_t s);
+
 struct CsrView {
   int m, n, nnz;
   const int* row_ptr;
@@ -59,15 +63,12 @@ cudaError_t launch_split_f32(const CsrView& A, const SplitIndex& I, const DenseV
                              int share, const SplitScratch& S, cudaStream_t s);
 // Warps (tiles) of one launch; SpMM: g lanes per merge thread.
 long long split_tiles(int nnz, int g, int share);
-// Fills words (every word), ids (if not NULL) and empty (if not NULL); ord: workspace of m ints and
-// scan_ws of scan_workspace_ints(m), both unused (may be NULL) when the matrix has no empty row.
-cudaError_t split_build(int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* empty, int* ord,
-                        int* scan_ws, cudaStream_t s);
-// The index of a one-shot call in two launches: words, ids [m], nonempty [1]; counts is a workspace
-// of kSplitBlocks ints.  Also writes the zeros of Y's empty rows (k columns; k may be 0).
+// The index in two launches: words, ids [m] (the non-empty rows; may be NULL when there is no empty
+// row), nonempty [1] and empty (either may be NULL); counts is a workspace of kSplitBlocks ints.
+// Also writes the zeros of Y's empty rows (k columns; k may be 0).
 constexpr int kSplitBlocks = 2048;
-cudaError_t split_build_once(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
-                             int* counts, int k, void* Y, long long ldy, cudaStream_t s);
+cudaError_t split_build(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
+                        int* empty, int* counts, int k, void* Y, long long ldy, cudaStream_t s);
 
 // ROWS variant.  lanes: 1..32 (power of two); k == 1 -> lanes split nonzeros,
 // k > 1 -> lanes split columns (k <= lanes * VEC is required per launch;

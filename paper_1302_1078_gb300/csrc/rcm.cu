@@ -301,7 +301,7 @@ cudaError_t rcm_run(int n, int nnz, const int* row_ptr, const int* col_idx, int*
   const size_t ints = (nn + 2 * c) * 2 + (nn + c) + 7 * nn + 2 * nn + 2 * nn + (nn + c) + (nn + 2 * c) + c + 64 +
                       scan_workspace_ints((long long)nn) + tx_ints(cap);
   int* base = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&base), ints * sizeof(int), s);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&base), ints * sizeof(int), s);
   if (e != cudaSuccess) return e;
   int* p = base;
   auto take = [&](size_t k) {
@@ -451,7 +451,7 @@ cudaError_t rcm_run(int n, int nnz, const int* row_ptr, const int* col_idx, int*
     reverse_k<<<grid_for(n), kThreads, 0, s>>>(n, order, perm);
     e = cudaGetLastError();
   } while (false);
-  cudaError_t e2 = cudaFreeAsync(base, s);
+  cudaError_t e2 = scratch_free(base, s);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return e;
@@ -464,7 +464,7 @@ cudaError_t permute_run(int n, int nnz, const int* row_ptr, const int* col_idx, 
   // iperm, lengths, U (ucol, usrc), T1 (rp, col, perm), T2 (perm), small, transpose scratch
   const size_t ints = nn + nn + 2 * c + (nn + 2 * c) + c + 64 + scan_workspace_ints((long long)nn) + tx_ints(nnz);
   int* base = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&base), ints * sizeof(int), s);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&base), ints * sizeof(int), s);
   if (e != cudaSuccess) return e;
   int* p = base;
   auto take = [&](size_t k) {
@@ -498,7 +498,7 @@ cudaError_t permute_run(int n, int nnz, const int* row_ptr, const int* col_idx, 
       e = cudaGetLastError();
     }
   } while (false);
-  cudaError_t e2 = cudaFreeAsync(base, s);
+  cudaError_t e2 = scratch_free(base, s);
   if (e == cudaSuccess) e = e2;
   return e;
 }

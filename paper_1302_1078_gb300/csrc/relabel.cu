@@ -118,7 +118,7 @@ cudaError_t col_degree_stats(int n, int nnz, const int* col_idx, int* max_deg, d
   if (n <= 0 || nnz <= 0) return cudaSuccess;
   void* buf = nullptr;
   const size_t bdeg = ((size_t)n * sizeof(int) + 255) & ~(size_t)255;
-  cudaError_t e = cudaMallocAsync(&buf, bdeg + 64, s);
+  cudaError_t e = scratch_alloc(&buf, bdeg + 64, s);
   if (e != cudaSuccess) return e;
   int* deg = static_cast<int*>(buf);
   unsigned long long* acc = reinterpret_cast<unsigned long long*>(static_cast<char*>(buf) + bdeg);
@@ -136,7 +136,7 @@ cudaError_t col_degree_stats(int n, int nnz, const int* col_idx, int* max_deg, d
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h_sq, acc, sizeof(h_sq), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h_mx, mx, sizeof(h_mx), cudaMemcpyDeviceToHost, s);
-  cudaError_t e2 = cudaFreeAsync(buf, s);
+  cudaError_t e2 = scratch_free(buf, s);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return e;
@@ -153,7 +153,7 @@ cudaError_t relabel_build(int n, int nnz, const int* col_idx, int* newid, int* c
   const size_t bh = (transpose_hist_ints(n) * sizeof(int) + 255) & ~(size_t)255;
   const size_t bw = (transpose_scan_ws_ints(n) * sizeof(int) + 255) & ~(size_t)255;
   void* buf = nullptr;
-  cudaError_t e = cudaMallocAsync(&buf, 5 * bi + bh + bw + 256, s);
+  cudaError_t e = scratch_alloc(&buf, 5 * bi + bh + bw + 256, s);
   if (e != cudaSuccess) return e;
   char* b = static_cast<char*>(buf);
   int* deg = reinterpret_cast<int*>(b);
@@ -194,7 +194,7 @@ cudaError_t relabel_build(int n, int nnz, const int* col_idx, int* newid, int* c
     relabel_cols_kernel<<<grid_for(nnz), 256, 0, s>>>(col_idx, newid, nnz, col_rl);
     e = cudaGetLastError();
   }
-  cudaError_t e2 = cudaFreeAsync(buf, s);
+  cudaError_t e2 = scratch_free(buf, s);
   if (e == cudaSuccess) e = e2;
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return e;

@@ -1,17 +1,15 @@
-// Plan-time index of the SPLIT variant (see split_kernel.cuh): per 32 nonzeros, the bitmap of row
-// ends and the ordinal of the first nonzero's row; the row numbers of the non-empty rows; the
-// empty rows.  One thread per row, the words of a long row written by its whole warp.
+// The index of the SPLIT variant (see split_kernel.cuh): per 32 nonzeros, the bitmap of row ends and
+// the ordinal of the first nonzero's row; the row numbers of the non-empty rows; the empty rows.
+// A one-shot call makes it each time and cannot afford a general scan's launches: at most
+// kSplitBlocks blocks of consecutive rows, whose non-empty rows the first kernel counts (it also
+// clears the words); in the second every block adds up the counts before its own, and the words of
+// a long row are written by its whole warp.
 #include <algorithm>
 
 #include "gbspmv.h"
 #include "launch.h"
 
 namespace gbs {
-
-__global__ void __launch_bounds__(256) nonempty_kernel(const int* __restrict__ rp, int m, int* __restrict__ flag) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) flag[i] = rp[i + 1] > rp[i];
-}
 
 // Marks the row's end in its word and numbers the words that begin in it (the whole warp calls it).
 __device__ __forceinline__ void split_mark(int s, int e, int number, SplitWord* __restrict__ words) {
@@ -35,27 +33,6 @@ __device__ __forceinline__ void split_mark(int s, int e, int number, SplitWord* 
   }
 }
 
-__global__ void __launch_bounds__(256) split_words_kernel(const int* __restrict__ rp, int m,
-                                                          const int* __restrict__ ord, SplitWord* __restrict__ words,
-                                                          int* __restrict__ ids, int* __restrict__ empty) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  int s = 0, e = 0, o = 0;
-  if (i < m) {
-    s = rp[i];
-    e = rp[i + 1];
-    o = ord ? ord[i] : i;
-    if (e > s) {
-      if (ids) ids[o] = i;
-    } else if (empty) {
-      empty[i - o] = i;
-    }
-  }
-  split_mark(s, e, o, words);
-}
-
-// ---- the index of a one-shot call, which cannot afford a general scan's launches: at most
-// kSplitBlocks blocks of consecutive rows, whose non-empty rows the first kernel counts (it also
-// clears the words); in the second every block adds up the counts before its own.
 __global__ void __launch_bounds__(256) split_count_kernel(const int* __restrict__ rp, int m, int rows_per_block,
                                                           SplitWord* __restrict__ words, int nwords,
                                                           int* __restrict__ counts) {
@@ -75,10 +52,11 @@ __global__ void __launch_bounds__(256) split_count_kernel(const int* __restrict_
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) split_once_kernel(const int* __restrict__ rp, int m, int rows_per_block,
+__global__ void __launch_bounds__(256) split_number_kernel(const int* __restrict__ rp, int m, int rows_per_block,
                                                          SplitWord* __restrict__ words, int* __restrict__ ids,
-                                                         int* __restrict__ nonempty, const int* __restrict__ counts,
-                                                         int k, T* __restrict__ Y, long long ldy) {
+                                                         int* __restrict__ nonempty, int* __restrict__ empty,
+                                                         const int* __restrict__ counts, int k, T* __restrict__ Y,
+                                                         long long ldy) {
   __shared__ int part[2][8];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int before = 0;
@@ -107,32 +85,19 @@ __global__ void __launch_bounds__(256) split_once_kernel(const int* __restrict__
       before += c;
     }
     buf ^= 1;
-    if (e > s)
-      ids[ord] = (int)i;
-    else if (i < r1)
+    if (e > s) {
+      if (ids) ids[ord] = (int)i;
+    } else if (i < r1) {
+      if (empty) empty[i - ord] = (int)i;
       for (int c = 0; c < k; ++c) Y[i * ldy + c] = T(0);
+    }
     split_mark(s, e, ord, words);
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *nonempty = before;
+  if (nonempty && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *nonempty = before;
 }
 
-cudaError_t split_build(int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* empty, int* ord,
-                        int* scan_ws, cudaStream_t s) {
-  if (m <= 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(words, 0, sizeof(SplitWord) * (size_t)(((long long)nnz + 31) / 32), s);
-  if (e != cudaSuccess) return e;
-  const int grid = (m + 255) / 256;
-  if (ord) {
-    nonempty_kernel<<<grid, 256, 0, s>>>(row_ptr, m, ord);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = exclusive_scan_i32(ord, ord, m, scan_ws, s)) != cudaSuccess) return e;
-  }
-  split_words_kernel<<<grid, 256, 0, s>>>(row_ptr, m, ord, words, ids, empty);
-  return cudaGetLastError();
-}
-
-cudaError_t split_build_once(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
-                             int* counts, int k, void* Y, long long ldy, cudaStream_t s) {
+cudaError_t split_build(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
+                        int* empty, int* counts, int k, void* Y, long long ldy, cudaStream_t s) {
   if (m <= 0) return cudaSuccess;
   const int per = (int)std::max<long long>(256, (((long long)m + kSplitBlocks - 1) / kSplitBlocks + 255) / 256 * 256);
   const int grid = (int)(((long long)m + per - 1) / per);
@@ -140,10 +105,10 @@ cudaError_t split_build_once(int dtype, int m, int nnz, const int* row_ptr, Spli
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (dtype == GBS_F64)
-    split_once_kernel<double><<<grid, 256, 0, s>>>(row_ptr, m, per, words, ids, nonempty, counts, k,
+    split_number_kernel<double><<<grid, 256, 0, s>>>(row_ptr, m, per, words, ids, nonempty, empty, counts, k,
                                                    static_cast<double*>(Y), ldy);
   else
-    split_once_kernel<float><<<grid, 256, 0, s>>>(row_ptr, m, per, words, ids, nonempty, counts, k,
+    split_number_kernel<float><<<grid, 256, 0, s>>>(row_ptr, m, per, words, ids, nonempty, empty, counts, k,
                                                   static_cast<float*>(Y), ldy);
   return cudaGetLastError();
 }
