@@ -688,6 +688,10 @@ static int product_entry(int m, int n, int nnz, const int* row_ptr, const int* c
   CsrView A{m, n, nnz, row_ptr, col_idx, vals};
   const bool unset = cfg == nullptr ||
                      (cfg->variant == GBS_VARIANT_AUTO && !cfg->threads && !cfg->items && !cfg->lanes && !cfg->relabel);
+  if (unset && k == 1 && ldx == 1 && ldy == 1 && m > 0 && nnz <= kSmallNnz && m <= 4 * kSmallNnz) {
+    const cudaError_t e = launch_small_spmv(dtype, A, X, Y, s);
+    return e == cudaSuccess ? GBS_OK : cuda_fail(e, "small SpMV launch");
+  }
   // a vector product of fewer items than this is bound by its launches, of which merge-path has
   // three and SPLIT four (64 x 64 grid: 25.1 and 25.5 us; 1.3 M nonzeros: 31.8 and 25.8 us)
   const bool small = k == 1 && (long long)m + nnz < 400000;

@@ -70,6 +70,10 @@ constexpr int kSplitBlocks = 2048;
 cudaError_t split_build(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
                         int* empty, int* counts, int k, void* Y, long long ldy, cudaStream_t s);
 
+// y = A x of a small matrix in one launch, without scratch (small.cu; contiguous x and y).
+constexpr int kSmallNnz = 98304;
+cudaError_t launch_small_spmv(int dtype, const CsrView& A, const void* x, void* y, cudaStream_t s);
+
 // ROWS variant.  lanes: 1..32 (power of two); k == 1 -> lanes split nonzeros,
 // k > 1 -> lanes split columns (k <= lanes * VEC is required per launch;
 // wider k is done in column panels by the caller).  vec16: use 128-bit
