@@ -117,7 +117,8 @@ __device__ __forceinline__ int split_row(const int* __restrict__ ids, int ord) {
 
 // The open sum of a merge thread as the carry scan combines it.  float: the accumulator's two parts
 // are added separately, so that the compensation of every share reaches the row and only the few
-// sums of the scan round.
+// sums of the scan round; SpMV, whose shares are short and their sums many, adds them with Knuth's
+// TwoSum (200,003 x 41 banded: error against 64 bits 6.0e-8 without it, 3.6e-8 with it; merge-path had 5.8e-8).
 template <typename T>
 struct Open;
 template <>
@@ -130,6 +131,7 @@ struct Open<double> {
     return o;
   }
   __device__ __forceinline__ void add(const Open& o) { s += o.s; }
+  __device__ __forceinline__ void add_exact(const Open& o) { s += o.s; }
   __device__ __forceinline__ double value() const { return s; }
 };
 template <>
@@ -145,6 +147,11 @@ struct Open<float> {
   __device__ __forceinline__ void add(const Open& o) {
     s = __fadd_rn(s, o.s);
     c = __fadd_rn(c, o.c);
+  }
+  __device__ __forceinline__ void add_exact(const Open& o) {
+    const float t = __fadd_rn(s, o.s), b = __fsub_rn(t, s);
+    c = __fadd_rn(__fadd_rn(c, o.c), __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(o.s, b)));
+    s = t;
   }
   __device__ __forceinline__ float value() const { return __fadd_rn(s, c); }
 };
@@ -200,13 +207,13 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
     const bool take = lane - d >= hs;
     if (__any_sync(0xffffffffu, take)) {
       const Open<T> o = S.up(d);
-      if (take) S.add(o);
+      if (take) S.add_exact(o);
     }
   }
   const Open<T> before = S.up(1);
   if (ends != 0) {
     Open<T> out(head);
-    if (lane > 0) out.add(before);
+    if (lane > 0) out.add_exact(before);
     st_stream(a.Y + split_row(ids, ord - __popc(ends)), out.value());
   }
   if (lane == 31) {
