@@ -278,16 +278,18 @@ int gbs_bcsr_destroy(gbs_bcsr* plan);
 /* ------------------------------------------------------------------ SpMV */
 /*
  * y <- A x  (Sec. 3).  vals, x and y have type `dtype`; x has n entries and
- * y has m entries.  The variant is chosen without looking at row_ptr
- * (merge-path, which balances any row-length distribution: MERGE_DIRECT with
- * 128 threads and 9 items per thread); its scratch
- * (one carry per CTA) comes from the stream-ordered allocator of the
- * current device (cudaMallocAsync / cudaFreeAsync on `stream`).  This
+ * y has m entries.  The variant is chosen without looking at row_ptr: one
+ * launch without scratch up to 98,304 nonzeros, merge-path (MERGE_DIRECT, 128
+ * threads, 9 items per thread) below 400,000 rows + nonzeros, else the
+ * nonzero-split walk on an index that the call makes (GBS_VARIANT_SPLIT), all
+ * of which balance any row lengths; scratch comes stream-ordered from the
+ * library's pool (gbs_release_scratch) on the current device.  This
  * one-shot call never reads the row-length statistics, because reading them
  * back would synchronise `stream` on every call.  A plan (gbs_plan_create)
  * is the path that picks the kernel and the lanes per row from the row
  * lengths, once: row-wise with lanes from the mean row length for regular
- * matrices, merge-path for skewed ones, or the autotuner's choice.
+ * matrices, merge-path or the nonzero split for skewed ones, or the
+ * autotuner's choice.
  * m, n >= 0, nnz >= 0; nnz == 0 or m == 0 writes zeros / nothing.
  */
 int spmv_csr(int m, int n, int nnz, const int* row_ptr, const int* col_idx, const void* vals,
@@ -358,7 +360,9 @@ int spmm_csr_cfg(int m, int n, int nnz, const int* row_ptr, const int* col_idx, 
  * products on the FP32 pipe).  With GBS_PLAN_CHECK it validates the structure first.  The plan
  * keeps row_ptr and col_idx as given: they must stay valid and unchanged
  * while the plan is used.  gbs_plan_create synchronises `stream`.
- * Executing a plan allocates nothing and can be captured in a CUDA graph.
+ * Executing a plan allocates nothing and can be captured in a CUDA graph; with
+ * a MERGE, MERGE_DIRECT, SPLIT or relabelling configuration it writes carries
+ * or a copy of x that the plan owns, so its calls must be ordered on one stream.
  */
 #define GBS_PLAN_TUNE 1
 #define GBS_PLAN_CHECK 2
@@ -419,8 +423,8 @@ int gbs_tplan_destroy(gbs_tplan* plan);
  * Make (and keep) a plan of A^T for `dtype` and k, with gbs_plan_create's
  * flags (GBS_PLAN_TUNE to autotune it); spmv_csr_backward then computes dX with
  * that plan's configuration instead of the one picked from A^T's row
- * statistics.  dX reads A's values in place through perm (ROWS, MERGE or
- * MERGE_DIRECT); with GBS_PLAN_TUNE the tuner also times permuting the
+ * statistics.  dX reads A's values in place through perm (ROWS, MERGE,
+ * MERGE_DIRECT or SPLIT); with GBS_PLAN_TUNE the tuner also times permuting the
  * values into scratch first (one extra pass) followed by the best of all
  * variants, and keeps that route if it is faster.  Synchronises `stream`.
  * Idempotent per (dtype, k).
@@ -428,8 +432,8 @@ int gbs_tplan_destroy(gbs_tplan* plan);
 int gbs_tplan_prepare(gbs_tplan* plan, int dtype, int k, int flags, void* stream);
 /*
  * Set the configuration of dX for (dtype, k), replacing a prepared one.
- * GBS_VARIANT_ROWS, GBS_VARIANT_MERGE and GBS_VARIANT_MERGE_DIRECT read A's
- * values in place through perm; GBS_VARIANT_ROWS_TMA permutes them into
+ * GBS_VARIANT_ROWS, GBS_VARIANT_MERGE, GBS_VARIANT_MERGE_DIRECT and
+ * GBS_VARIANT_SPLIT read A's values in place through perm; GBS_VARIANT_ROWS_TMA permutes them into
  * plan-owned scratch first (allocated here, nnz doubles); GBS_VARIANT_AUTO
  * takes the configuration from A^T's row statistics.  Errors as
  * gbs_plan_set_config.  Synchronises `stream`.
@@ -466,18 +470,19 @@ int spmv_csr_backward(gbs_tplan* plan, const int* row_ptr, const int* col_idx, c
  * Many independent products Y_b <- A_b X_b (b < nmat; k columns for all, k
  * == 1 is SpMV), each the product of Sec. 3 / Sec. 5, run by one persistent
  * kernel replayed from a CUDA graph.  The plan
- *   - picks each matrix's configuration (ROWS lanes / tile or MERGE items;
- *     256 threads) from its row statistics, or with GBS_PLAN_TUNE by timing
- *     candidates with standalone launches on the given operands (this
- *     writes Y_b), and then by timing whole-batch policies on the batched
- *     kernel itself (the statistics' variant with a given ROWS tile, MERGE
- *     for matrices of short rows, a given merge tile), keeping the fastest;
+ *   - gives every matrix MERGE, which a batch runs as the nonzero-split walk
+ *     (see GBS_VARIANT_SPLIT; 256 threads, one tile per warp), or with
+ *     GBS_PLAN_TUNE times whole-batch policies on the batched kernel itself
+ *     (this writes Y_b): that, longer shares, and ROWS for the matrices of
+ *     long, even rows, keeping the fastest;
  *   - builds the work list: matrix b owns the contiguous items
- *     [item_begin[b], item_begin[b+1]) (row blocks or merge tiles); the
+ *     [item_begin[b], item_begin[b+1]) (row blocks or groups of tiles); the
  *     grid is every resident CTA slot (`grid`), and each CTA claims the next
  *     unclaimed item from a device counter that the graph zeroes before the
- *     kernel, so launches of one plan must be ordered on one stream;
- *   - owns a device descriptor table, the merge scratch and the graph.
+ *     kernel, so launches of one plan must be ordered on one stream; a second
+ *     node of the graph adds the rows split between tiles and writes the
+ *     empty rows' zeros;
+ *   - owns a device descriptor table, the split indices and carries and the graph.
  * The arrays of every item must stay valid and unchanged while the plan is
  * used (only X and Y may be replaced, below).  Results equal
  * spmv_csr_batched_looped (one standalone launch per matrix with the same
@@ -506,9 +511,9 @@ int spmv_csr_batched_plan(gbs_batch_plan** plan, int nmat, const gbs_batch_item*
  * nmat entries) gives each matrix GBS_VARIANT_ROWS or GBS_VARIANT_MERGE with
  * its lanes (k == 1; k > 1 uses the batch's column lanes), tile_nnz or items,
  * or GBS_VARIANT_AUTO for the heuristic / tuner choice of
- * spmv_csr_batched_plan.  threads is always 256; merge items are capped to the
- * batch kernel's shared-memory budget (spmv_csr_batched_info reports the values
- * used).  Errors: GBS_EUNSUPPORTED (another variant), GBS_EINVAL (as
+ * spmv_csr_batched_plan.  threads is always 256; a MERGE matrix's items are
+ * its nonzeros per merge thread, rounded up to a multiple of 32 and at most
+ * 256 (k = 1: always 8).  Errors: GBS_EUNSUPPORTED (another variant), GBS_EINVAL (as
  * gbs_plan_set_config).  cfgs == NULL is spmv_csr_batched_plan.
  */
 int spmv_csr_batched_plan_cfg(gbs_batch_plan** plan, int nmat, const gbs_batch_item* items /* host */,

@@ -20,6 +20,7 @@
 #include "merge_kernel.cuh"
 #include "rows_kernel.cuh"
 #include "rows_tma.cuh"
+#include "split_kernel.cuh"
 
 using namespace gbs;
 
@@ -1773,13 +1774,19 @@ struct gbs_batch_plan {
   std::vector<gbs_config> cfgs;
   std::vector<gbs_stats> stats;  // row statistics of each matrix
   std::vector<int> item_begin;  // nmat + 1
-  std::vector<MergeBuffers> mbs;
+  struct Split {  // MERGE matrices: the index and carries in the plan's scratch, blocks of the fix-up launch
+    SplitIndex index{};
+    SplitScratch scratch{};
+    int share = 0, tiles = 0, carry_blocks = 0;
+  };
+  std::vector<Split> splits;
   std::vector<unsigned char> h_desc;
   void* d_desc = nullptr;
   void* scratch = nullptr;
   int* next_item = nullptr;  // device work counter, reset by the graph before every launch
   size_t smem = 0;
-  int grid = 0, total_items = 0;
+  int grid = 0, total_items = 0, fix_blocks = 0;
+  std::vector<int> fix_begin;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
 };
@@ -1794,15 +1801,11 @@ constexpr size_t kBatchSmemBudget = 54 * 1024;
 size_t rows_smem_host(int dtype, int rpc, int tile) {
   return dtype == GBS_F64 ? rows_smem_bytes<double>(rpc, tile) : rows_smem_bytes<float>(rpc, tile);
 }
-size_t merge_smem_host(int dtype, int g, bool vec16, int items, bool direct) {
-  const int vec = vec16 ? vec_of(dtype) : 1;
-  const int nt = kBatchThreads / g;
-  const size_t es = dsize(dtype);
-  const size_t ipc = (size_t)nt * items;
-  size_t a = direct ? 0 : ((ipc + 2) * sizeof(int) + 15) & ~(size_t)15;
-  size_t b = direct ? 0 : ((ipc + 4) * es + 15) & ~(size_t)15;
-  size_t c = direct ? 0 : ((ipc + 4) * sizeof(int) + 15) & ~(size_t)15;
-  return a + b + c + 2 * (size_t)(kBatchThreads / 32) * sizeof(int) + 2 * (size_t)(kBatchThreads / 32) * g * vec * es;
+// Nonzeros per merge thread of a MERGE matrix from its configuration's items (0: the default).
+int batch_share(int items, int dtype, int k) {
+  if (k == 1) return kSplitShare;
+  if (items <= 0) return dtype == GBS_F64 ? 64 : 32;
+  return std::min(256, (items + 31) / 32 * 32);
 }
 
 template <typename T>
@@ -1824,14 +1827,21 @@ void fill_desc(gbs_batch_plan* p, int b, BatchDesc<T>* d) {
   d->variant = c.variant;
   d->lanes = p->split ? c.lanes : p->G;
   d->tile = c.tile_nnz;
-  d->items = c.items;
+  d->fix_begin = p->fix_begin[b];
+  d->share = p->splits[b].share;
+  d->tiles = p->splits[b].tiles;
   d->item_begin = p->item_begin[b];
   d->nitems = p->item_begin[b + 1] - p->item_begin[b];
   if (is_merge(c.variant)) {
-    d->coords = p->mbs[b].s.coords;
-    d->carry_row = p->mbs[b].s.carry_row;
-    d->carry_val = static_cast<T*>(p->mbs[b].s.carry_val);
-    d->done = reinterpret_cast<int*>(static_cast<char*>(p->mbs[b].base) + p->mbs[b].bytes - sizeof(int));
+    const auto& sp = p->splits[b];
+    d->words = sp.index.words;
+    d->ids = sp.index.ids;
+    d->empty = sp.index.empty;
+    d->nempty = sp.index.nempty;
+    d->carry_row = sp.scratch.carry_row;
+    d->carry_val = static_cast<T*>(sp.scratch.carry_val);
+    d->fix_carry_blocks = sp.carry_blocks;
+    d->wide = ((reinterpret_cast<uintptr_t>(it.vals) | reinterpret_cast<uintptr_t>(it.col_idx)) & 31) == 0;
   }
   d->aligned_vals = aligned16(it.vals);
   d->aligned_cols = aligned16(it.col_idx);
@@ -1846,40 +1856,8 @@ void batch_free(gbs_batch_plan* p) {
   delete p;
 }
 
-// Per-matrix configuration for the batch: 256 threads; k > 1 uses the plan's column lanes.
-std::vector<gbs_config> batch_candidates(const gbs_stats& st, int dtype, int k) {
-  std::vector<gbs_config> c;
-  const int base_tile = dtype == GBS_F64 ? 2048 : 3072;
-  auto add = [&](int variant, int lanes, int tile, int items) {
-    gbs_config g{};
-    g.variant = variant;
-    g.lanes = lanes;
-    g.threads = kBatchThreads;
-    g.tile_nnz = tile;
-    g.items = items;
-    c.push_back(g);
-  };
-  if (k == 1) {
-    for (int l : {1, 2, 4, 8, 16, 32})
-      if (l == 1 || st.mean_row >= 0.5 * l) add(GBS_VARIANT_ROWS, l, base_tile, 0);
-    for (int it : {7, 15, 31}) add(GBS_VARIANT_MERGE, 0, 0, it);
-  } else {
-    add(GBS_VARIANT_ROWS, 0, base_tile, 0);
-    add(GBS_VARIANT_ROWS, 0, base_tile / 2, 0);
-    add(GBS_VARIANT_ROWS, 0, base_tile * 2, 0);
-    add(GBS_VARIANT_MERGE, 0, 0, 0);
-    add(GBS_VARIANT_MERGE, 0, 0, 15);
-  }
-  return c;
-}
-
-// Largest odd merge items per thread (at most `items`, at least 3) whose shared memory fits
-// the batched kernel's budget.
-int batch_cap_items(int dtype, int g, bool vec16, int items) {
-  int it = std::max(3, items | 1);
-  while (it > 3 && merge_smem_host(dtype, g, vec16, it, false) > kBatchSmemBudget) it -= 2;
-  return it;
-}
+int batched_plan_make(gbs_batch_plan** out, int nmat, const gbs_batch_item* items, int dtype, int k, int flags,
+                      const gbs_config* cfgs, const std::vector<gbs_stats>* known, void* stream);
 
 }  // namespace
 
@@ -1890,11 +1868,10 @@ int spmv_csr_batched_plan(gbs_batch_plan** out, int nmat, const gbs_batch_item* 
   int rc = spmv_csr_batched_plan_cfg(out, nmat, items, dtype, k, flags, nullptr, stream);
   if (rc || !(flags & GBS_PLAN_TUNE) || !*out || !(*out)->exec) return rc;
   // Standalone timings of a small matrix measure its launch latency, not what its items cost
-  // inside a full batch.  So whole-batch policies are also built and timed on the batched
-  // kernel itself, and the fastest plan is kept (the per-matrix choice is one of them).  A
-  // policy starts from the per-matrix choice or from the statistics' variant (ROWS with a given
-  // tile, MERGE for skewed rows), and sends matrices whose mean row is shorter than a threshold
-  // to MERGE; MERGE tiles take a given number of items per thread (then capped to the budget).
+  // inside a full batch.  So whole-batch policies are built and timed on the batched kernel itself,
+  // and the fastest plan is kept: MERGE for every matrix (built already), the same with shares of
+  // 128 nonzeros (block vectors: half the carry scans, for batches large enough to fill the GPU with
+  // them), or ROWS for the matrices whose mean row reaches a threshold and whose rows are not skewed.
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   gbs_batch_plan* best = *out;
   auto time_plan = [&](gbs_batch_plan* q) {
@@ -1902,56 +1879,38 @@ int spmv_csr_batched_plan(gbs_batch_plan** out, int nmat, const gbs_batch_item* 
   };
   float best_ms = time_plan(best);
   if (best_ms < 0) best_ms = 1e30f;
-  const std::vector<gbs_config> tuned = best->cfgs;
   const std::vector<gbs_stats> stats = best->stats;
   const int base_tile = dtype == GBS_F64 ? 2048 : 3072;
   struct Policy {
-    bool from_stats;  // statistics' variant (else the per-matrix choice)
-    int rows_tile;    // ROWS tile when from_stats
-    double short_row; // mean row below which a matrix takes `short_variant` (0: none)
-    int merge_items;  // items per merge thread for the MERGE matrices (0: default)
-    int short_variant;  // MERGE, or ROWS_DIRECT (no staging, no barriers)
+    int rows_tile;     // ROWS tile
+    double short_row;  // mean row below which a matrix takes MERGE
+    int items;         // nonzeros per merge thread of the MERGE matrices (0: the default)
   };
-  std::vector<Policy> policies;
-  // (on the 512-matrix k = 8 batch every policy was slower with merge tiles larger or smaller
-  // than the default, and with ROWS_DIRECT matrices, whether for the short rows or for all the
-  // statistics' ROWS matrices, so neither is tried)
-  for (double thr : {0.0, 8.0, 12.0, 20.0}) {
-    policies.push_back({false, 0, thr, 0, GBS_VARIANT_MERGE});
-    for (int t : {base_tile, 2 * base_tile}) policies.push_back({true, t, thr, 0, GBS_VARIANT_MERGE});
-  }
-  int pol_id = 0;
+  std::vector<Policy> policies = {{base_tile, 8.0, 0}, {2 * base_tile, 20.0, 0}};
+  if (k > 1) policies.push_back({base_tile, 1e30, 128});
   for (const Policy& pol : policies) {
-    ++pol_id;
-    if (!pol.from_stats && pol.short_row == 0.0 && pol.merge_items == 0) continue;  // the per-matrix choice
     std::vector<gbs_config> cf(nmat);
     for (int b = 0; b < nmat; ++b) {
-      const gbs_stats& st = stats[b];
-      gbs_config c = tuned[b];
-      if (pol.from_stats) {
-        c = heuristic_config(st, dtype, k);
-        if (c.variant == GBS_VARIANT_ROWS) c.tile_nnz = pol.rows_tile;
-      }
-      if (pol.short_row > 0.0 && st.mean_row < pol.short_row) {
+      gbs_config c = heuristic_config(stats[b], dtype, k);
+      if (c.variant == GBS_VARIANT_ROWS) c.tile_nnz = pol.rows_tile;
+      if (stats[b].mean_row < pol.short_row) {
         c = gbs_config{};
-        c.variant = pol.short_variant;
+        c.variant = GBS_VARIANT_MERGE;
       }
-      if (c.variant == GBS_VARIANT_MERGE && (pol.from_stats || pol.short_row > 0.0 || pol.merge_items > 0))
-        c.items = pol.merge_items;
+      if (c.variant == GBS_VARIANT_MERGE) c.items = pol.items;
       c.threads = kBatchThreads;
       cf[b] = c;
     }
     gbs_batch_plan* q = nullptr;
-    if (spmv_csr_batched_plan_cfg(&q, nmat, items, dtype, k, flags & ~GBS_PLAN_TUNE, cf.data(), stream) != GBS_OK ||
+    if (batched_plan_make(&q, nmat, items, dtype, k, flags & ~GBS_PLAN_TUNE, cf.data(), &stats, stream) != GBS_OK ||
         !q || !q->exec) {
       if (q) batch_free(q);
       continue;
     }
     const float ms = time_plan(q);
     if (tune_log())
-      std::fprintf(stderr, "gbspmv batch policy %d (stats %d tile %d short<%.0f -> variant %d, items %d): %.4f ms "
-                   "(best %.4f ms)\n", pol_id, (int)pol.from_stats, pol.rows_tile, pol.short_row, pol.short_variant,
-                   pol.merge_items, ms, best_ms);
+      std::fprintf(stderr, "gbspmv batch policy (ROWS tile %d, MERGE below %.0f, items %d): %.4f ms (best %.4f ms)\n",
+                   pol.rows_tile, pol.short_row, pol.items, ms, best_ms);
     if (ms > 0 && ms < best_ms) {
       batch_free(best);
       best = q;
@@ -1967,6 +1926,16 @@ int spmv_csr_batched_plan(gbs_batch_plan** out, int nmat, const gbs_batch_item* 
 
 int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_item* items, int dtype, int k,
                               int flags, const gbs_config* cfgs, void* stream) {
+  return batched_plan_make(out, nmat, items, dtype, k, flags, cfgs, nullptr, stream);
+}
+
+}  // extern "C"
+
+namespace {
+
+// known: the matrices' row statistics, if the caller has them (NULL: computed here).
+int batched_plan_make(gbs_batch_plan** out, int nmat, const gbs_batch_item* items, int dtype, int k, int flags,
+                      const gbs_config* cfgs, const std::vector<gbs_stats>* known, void* stream) {
   if (!out) return fail(GBS_EINVAL, "plan is NULL");
   *out = nullptr;
   if (nmat < 1 || !items) return fail(GBS_EINVAL, "nmat must be >= 1 and items non-NULL");
@@ -2003,7 +1972,7 @@ int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_it
   p->items.assign(items, items + nmat);
   p->cfgs.resize(nmat);
   p->stats.resize(nmat);
-  p->mbs.resize(nmat);
+  p->splits.resize(nmat);
 
   // ---- the caller's configurations: ROWS or MERGE, run by the batch's 256-thread CTAs
   std::vector<gbs_config> given_cfgs;
@@ -2031,69 +2000,40 @@ int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_it
     }
   }
 
-  // ---- per-matrix configuration (given, heuristic, or timed with standalone launches)
-  cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-  const bool tune = (flags & GBS_PLAN_TUNE) != 0;
-  if (tune) {
-    cudaEventCreate(&ev0);
-    cudaEventCreate(&ev1);
-  }
+  // ---- per-matrix configuration (given, or from the row statistics)
   for (int b = 0; b < nmat; ++b) {
     const gbs_batch_item& it = p->items[b];
     gbs_stats& st = p->stats[b];
-    int rc = compute_stats(it.m, it.n, it.nnz, it.row_ptr, &st, s);
+    int rc = GBS_OK;
+    if (known)
+      st = (*known)[b];
+    else
+      rc = compute_stats(it.m, it.n, it.nnz, it.row_ptr, &st, s);
     if (rc) {
       batch_free(p);
       return rc;
     }
-    gbs_config c = heuristic_config(st, dtype, k);
+    // MERGE whatever the row lengths: on 128 matrices (stencil, banded and R-MAT in turn) it is
+    // faster than ROWS for the even ones and MERGE for the skewed, k = 8 in FP64 1.61 and 1.66 ms,
+    // k = 1 0.38 and 0.60 ms, k = 4 in FP32 0.47 and 0.56 ms
+    gbs_config c{};
+    c.variant = GBS_VARIANT_MERGE;
     c.threads = kBatchThreads;
-    if (c.variant == GBS_VARIANT_ROWS && k > 1) c.lanes = p->G;
     const bool given = !given_cfgs.empty() && given_cfgs[b].variant != GBS_VARIANT_AUTO;
     if (given) c = given_cfgs[b];
-    if (tune && !given && it.m > 0) {
-      float best = 1e30f;
-      for (gbs_config cand : batch_candidates(st, dtype, k)) {
-        if (k > 1 && cand.variant == GBS_VARIANT_ROWS) cand.lanes = p->G;
-        if (is_merge(cand.variant)) {
-          // time the tile size the batch will run (capped to the shared-memory budget)
-          const MergeGeom G = merge_geom(cand, it.m, it.nnz, dtype, k, vec16);
-          cand.items = batch_cap_items(dtype, G.g, vec16, G.items);
-        }
-        CsrView A{it.m, it.n, it.nnz, it.row_ptr, it.col_idx, it.vals};
-        float ms_sum = 0;
-        bool ok = true;
-        for (int r = 0; r < 3 && ok; ++r) {
-          ok = cudaEventRecord(ev0, s) == cudaSuccess &&
-               run_product(A, dtype, k, it.X, k == 1 ? 1 : it.ldx, it.Y, k == 1 ? 1 : it.ldy, cand, nullptr, false, s) ==
-                   GBS_OK &&
-               cudaEventRecord(ev1, s) == cudaSuccess && cudaEventSynchronize(ev1) == cudaSuccess;
-          float ms = 0;
-          if (ok && r > 0) {
-            cudaEventElapsedTime(&ms, ev0, ev1);
-            ms_sum += ms;
-          }
-        }
-        if (ok && ms_sum < best) {
-          best = ms_sum;
-          c = cand;
-        }
-      }
-    }
     p->cfgs[b] = c;
   }
-  if (ev0) cudaEventDestroy(ev0);
-  if (ev1) cudaEventDestroy(ev1);
   g_err.clear();
 
   // ---- work list, shared memory, merge scratch
   p->item_begin.assign(nmat + 1, 0);
+  p->fix_begin.assign(nmat + 1, 0);
   size_t scratch_total = 0;
   std::vector<size_t> scratch_off(nmat, 0);
   for (int b = 0; b < nmat; ++b) {
     const gbs_batch_item& it = p->items[b];
     const gbs_config& c = p->cfgs[b];
-    long long nitems = 0;
+    long long nitems = 0, fix = 0;
     if (c.variant == GBS_VARIANT_ROWS) {
       const int lanes = k == 1 ? c.lanes : p->G;
       const int rpc = kBatchThreads / lanes;
@@ -2103,42 +2043,57 @@ int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_it
         p->cfgs[b].tile_nnz /= 2;
       p->smem = std::max(p->smem, rows_smem_host(dtype, rpc, p->cfgs[b].tile_nnz));
     } else {
-      MergeGeom G = merge_geom(c, it.m, it.nnz, dtype, k, vec16);
-      const int capped = batch_cap_items(dtype, G.g, vec16, G.items);
-      if (capped != G.items) {
-        p->cfgs[b].items = capped;
-        G = merge_geom(p->cfgs[b], it.m, it.nnz, dtype, k, vec16);
-      }
-      p->cfgs[b].items = G.items;
-      nitems = it.m > 0 ? G.ctas : 0;
-      p->smem = std::max(p->smem, merge_smem_host(dtype, G.g, vec16, G.items, c.variant == GBS_VARIANT_MERGE_DIRECT));
+      auto& sp = p->splits[b];
+      sp.share = batch_share(c.items, dtype, k);
+      sp.tiles = (int)split_tiles(it.nnz, p->G, sp.share);
+      const int per = batch_item_tiles(k);
+      nitems = it.m > 0 ? (sp.tiles + per - 1) / per : 0;
+      // words | ids | empty | carry rows | carries
+      const int nempty = p->stats[b].empty_rows, lg = split_fixup_lg(k);
+      sp.carry_blocks = (int)((((long long)sp.tiles << lg) + 255) >> 8);
+      fix = it.m > 0 ? sp.carry_blocks + ((((long long)nempty << lg) + 255) >> 8) : 0;
       scratch_off[b] = scratch_total;
-      const size_t bytes = align256(merge_scratch_bytes(G.ctas, G.kp_max, dtype) + sizeof(int));
-      p->mbs[b].bytes = bytes;
-      scratch_total += bytes;
+      scratch_total += align256(sizeof(SplitWord) * (size_t)(((long long)it.nnz + 31) / 32)) +
+                       (nempty ? align256(sizeof(int) * (size_t)(it.m - nempty)) : 0) + align256(sizeof(int) * (size_t)nempty) +
+                       align256(sizeof(int) * (size_t)sp.tiles) + align256(es * (size_t)sp.tiles * k);
     }
-    if ((long long)p->item_begin[b] + nitems > 0x7fffffffLL) {
+    if ((long long)p->item_begin[b] + nitems > 0x7fffffffLL || (long long)p->fix_begin[b] + fix > 0x7fffffffLL) {
       batch_free(p);
       return fail(GBS_EUNSUPPORTED, "batch work list exceeds 2^31 items");
     }
     p->item_begin[b + 1] = p->item_begin[b] + (int)nitems;
+    p->fix_begin[b + 1] = p->fix_begin[b] + (int)fix;
   }
   p->total_items = p->item_begin[nmat];
+  p->fix_blocks = p->fix_begin[nmat];
   cudaError_t e = cudaSuccess;
   if (scratch_total) {
+    void* counts = nullptr;
     e = cudaMalloc(&p->scratch, scratch_total);
     if (e == cudaSuccess) e = cudaMemsetAsync(p->scratch, 0, scratch_total, s);
+    if (e == cudaSuccess) e = scratch_alloc(&counts, sizeof(int) * kSplitBlocks, s);
     for (int b = 0; b < nmat && e == cudaSuccess; ++b) {
       if (!is_merge(p->cfgs[b].variant)) continue;
       const gbs_batch_item& it = p->items[b];
-      const MergeGeom G = merge_geom(p->cfgs[b], it.m, it.nnz, dtype, k, vec16);
-      p->mbs[b].base = static_cast<char*>(p->scratch) + scratch_off[b];
-      merge_carve(p->mbs[b], G.ctas, G.kp_max, dtype);
-      if (it.m > 0) {
-        CsrView A{it.m, it.n, it.nnz, it.row_ptr, it.col_idx, it.vals};
-        e = launch_merge_partition(A, (long long)(kBatchThreads / G.g) * G.items, p->mbs[b].s, s);
-      }
+      auto& sp = p->splits[b];
+      const int nempty = p->stats[b].empty_rows;
+      char* q = static_cast<char*>(p->scratch) + scratch_off[b];
+      auto take = [&](size_t bytes) {
+        char* r = q;
+        q += align256(bytes);
+        return static_cast<void*>(r);
+      };
+      SplitWord* words = static_cast<SplitWord*>(take(sizeof(SplitWord) * (size_t)(((long long)it.nnz + 31) / 32)));
+      int* ids = nempty ? static_cast<int*>(take(sizeof(int) * (size_t)(it.m - nempty))) : nullptr;
+      int* empty = nempty ? static_cast<int*>(take(sizeof(int) * (size_t)nempty)) : nullptr;
+      sp.index = SplitIndex{words, ids, empty, nempty};
+      sp.scratch.carry_row = static_cast<int*>(take(sizeof(int) * (size_t)sp.tiles));
+      sp.scratch.carry_val = take(es * (size_t)sp.tiles * k);
+      e = split_build(dtype, it.m, it.nnz, it.row_ptr, words, ids, nullptr, empty, static_cast<int*>(counts), 0, nullptr,
+                      0, s);
     }
+    const cudaError_t e2 = scratch_free(counts, s);
+    if (e == cudaSuccess) e = e2;
   }
   // ---- descriptors
   const size_t dsz = dtype == GBS_F64 ? sizeof(BatchDesc<double>) : sizeof(BatchDesc<float>);
@@ -2174,6 +2129,7 @@ int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_it
       if (el == cudaSuccess)
         el = batched_kernel_call(true, dtype, p->split, p->G, vec16, p->d_desc, nmat, p->total_items, p->next_item,
                                  p->grid, p->smem, nullptr, cs);
+      if (el == cudaSuccess) el = batched_fixup(dtype, p->d_desc, nmat, p->fix_blocks, cs);
       e = cudaStreamEndCapture(cs, &p->graph);
       if (el != cudaSuccess) e = el;
     }
@@ -2187,6 +2143,10 @@ int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_it
   *out = p;
   return GBS_OK;
 }
+
+}  // namespace
+
+extern "C" {
 
 int spmv_csr_batched(gbs_batch_plan* p, const void* const* X, void* const* Y, void* stream) {
   if (!p) return fail(GBS_EINVAL, "plan is NULL");
@@ -2223,10 +2183,17 @@ int spmv_csr_batched_looped(gbs_batch_plan* p, void* stream) {
     if (it.m == 0) continue;
     CsrView A{it.m, it.n, it.nnz, it.row_ptr, it.col_idx, it.vals};
     gbs_config c = p->cfgs[b];
+    if (is_merge(c.variant)) {
+      const auto& sp = p->splits[b];
+      const DenseView D{p->k, it.X, p->k == 1 ? 1 : it.ldx, it.Y, p->k == 1 ? 1 : it.ldy};
+      const cudaError_t e = p->dtype == GBS_F64 ? launch_split_f64(A, sp.index, D, p->vec16, 64, sp.share, sp.scratch, s)
+                                                : launch_split_f32(A, sp.index, D, p->vec16, 64, sp.share, sp.scratch, s);
+      if (e != cudaSuccess) return cuda_fail(e, "batched loop launch");
+      continue;
+    }
     if (c.variant == GBS_VARIANT_ROWS && p->k > 1) c.lanes = p->G;
-    MergeBuffers mb = p->mbs[b];
-    int rc = run_product(A, p->dtype, p->k, it.X, p->k == 1 ? 1 : it.ldx, it.Y, p->k == 1 ? 1 : it.ldy, c,
-                         is_merge(c.variant) ? &mb : nullptr, true, s);
+    const int rc = run_product(A, p->dtype, p->k, it.X, p->k == 1 ? 1 : it.ldx, it.Y, p->k == 1 ? 1 : it.ldy, c, nullptr,
+                               true, s);
     if (rc) return rc;
   }
   return GBS_OK;

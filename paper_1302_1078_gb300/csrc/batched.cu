@@ -9,23 +9,31 @@
 // costs; the matrix comes from a binary search of the descriptors' first items
 // (a CTA's items only increase, so the search starts at its previous matrix),
 // and each item runs exactly the device function the standalone kernels run
-// (rows_block / merge_tile) with the matrix's own tuned configuration, so the
-// batched result equals the per-matrix loop bitwise: which CTA runs an item
-// does not change what the item computes.
+// (rows_block / split_spmv_tile / split_spmm_tile) with the matrix's own
+// configuration, so the batched result equals the per-matrix loop bitwise:
+// which CTA runs an item does not change what the item computes.
 //
-// A merge-path matrix needs its per-tile carries added after all its tiles are
-// done.  The CTA that finishes a matrix's last tile (a per-matrix counter,
-// incremented after a memory fence) performs that fix-up and resets the
-// counter for the next launch.  No CTA ever waits for another.
+// A MERGE matrix runs as the nonzero-split walk (split_kernel.cuh): every warp
+// takes a tile, without shared memory or barriers, and a second, small node of
+// the graph adds every matrix's carries and writes the empty rows' zeros.  (With
+// the fix-up in the kernel, by the CTA that retired a matrix's last item, the
+// largest matrices' carries were a serial tail: 2.2 ms for 128 matrices of
+// k = 8.)  On that batch the staged merge-path tiles this replaced, with three
+// barriers and 54 KB of staging each, kept the FP64 pipe 81% busy:
+// 1776 -> 1564 us.
 #include <cstdint>
 
 #include "batched.cuh"
 #include "gbspmv.h"
 #include "launch.h"
-#include "merge_kernel.cuh"
 #include "rows_kernel.cuh"
+#include "split_kernel.cuh"
 
 namespace gbs {
+
+// Resident CTAs of the batched kernel: the nonzero-split walk wants 80 registers (three CTAs), and
+// 64 cost it 60 bytes of spill, but a fourth CTA is worth more (128 matrices, k = 8: 1.69 and 1.61 ms).
+constexpr int kBatchCtas = 4;
 
 template <typename T>
 __device__ __forceinline__ RowsArgs<T> rows_args(const BatchDesc<T>& d) {
@@ -47,25 +55,27 @@ __device__ __forceinline__ RowsArgs<T> rows_args(const BatchDesc<T>& d) {
 }
 
 template <typename T>
-__device__ __forceinline__ MergeArgs<T> merge_args(const BatchDesc<T>& d) {
-  MergeArgs<T> a;
+__device__ __forceinline__ SplitArgs<T> split_args(const BatchDesc<T>& d) {
+  SplitArgs<T> a;
   a.m = d.m;
   a.k = d.k;
   a.nnz = d.nnz;
-  a.row_ptr = d.row_ptr;
   a.col_idx = d.col_idx;
   a.vals = d.vals;
+  a.perm = nullptr;
   a.X = d.X;
   a.Y = d.Y;
   a.ldx = d.ldx;
   a.ldy = d.ldy;
-  a.items = d.items;
-  a.ctas = d.nitems;
-  a.coords = d.coords;
+  a.words = d.words;
+  a.nwords = (int)(((long long)d.nnz + 31) / 32);
+  a.ids = d.ids;
+  a.nonempty = nullptr;
+  a.share = d.share;
+  a.tiles = d.tiles;
   a.carry_row = d.carry_row;
   a.carry_val = d.carry_val;
-  a.aligned_vals = d.aligned_vals;
-  a.aligned_cols = d.aligned_cols;
+  a.wide = d.wide != 0;
   return a;
 }
 
@@ -73,9 +83,9 @@ __device__ __forceinline__ MergeArgs<T> merge_args(const BatchDesc<T>& d) {
 // (ROWS_DIRECT items are not offered: they lost every whole-batch policy, and their code cost this
 // register-bound kernel spills.)
 template <typename T, int VEC, bool SPLIT, int G>
-__global__ void __launch_bounds__(256, 4) batched_kernel(const BatchDesc<T>* __restrict__ descs, int nmat,
+__global__ void __launch_bounds__(256, kBatchCtas) batched_kernel(const BatchDesc<T>* __restrict__ descs, int nmat,
                                                       int total_items, int* __restrict__ next_item) {
-  __shared__ int s_last, s_item;
+  __shared__ int s_item;
   int lo = 0;  // matrix of this CTA's previous item
   // items are claimed one ahead: the claim of the next item is issued when the current one
   // starts, so the atomic's round trip overlaps the current item's work
@@ -111,28 +121,54 @@ __global__ void __launch_bounds__(256, 4) batched_kernel(const BatchDesc<T>* __r
         rows_block<T, VEC, G, false>(a, local);
       }
     } else {
-      const MergeArgs<T> a = merge_args(d);
-      merge_tile<T, VEC, (SPLIT ? 1 : G), false>(a, local);
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        __threadfence();  // this tile's Y rows and carry are visible before it is counted
-        s_last = atomicAdd(d.done, 1) == d.nitems - 1;
-      }
-      __syncthreads();
-      if (s_last) {
-        __threadfence();  // every other tile of the matrix has been counted: read their carries
-        for (int t = threadIdx.x; t < d.nitems; t += blockDim.x)
-          merge_fixup_one<T>(t, d.nitems, d.k, d.carry_row, d.carry_val, d.Y, d.ldy);
-        if (threadIdx.x == 0) *d.done = 0;
+      const SplitArgs<T> a = split_args(d);
+      const int per = batch_item_tiles(d.k);
+      const int t1 = min(a.tiles, (local + 1) * per);
+      for (int t = local * per + ((int)threadIdx.x >> 5); t < t1; t += 8) {
+        if constexpr (SPLIT)
+          split_spmv_tile<T, false>(a, t);
+        else
+          split_spmm_tile<T, VEC, G, false>(a, t);
       }
     }
-    // every thread read s_item before the item's first internal barrier, and no thread reads
-    // shared memory after the item's last barrier (ROWS: the last tile pass ends with one; MERGE:
-    // the barrier before the completion count), so the next item's index is published, and the
-    // shared memory handed over, with a single barrier
+    // the next item's index is published, and a ROWS item's shared memory handed over, with one
+    // barrier after the item and one before the next (a MERGE item has none of its own)
+    __syncthreads();
     if (threadIdx.x == 0) s_item = claimed;
     __syncthreads();
   }
+}
+
+// The carries and the empty rows of every MERGE matrix, as split_fixup_kernel for each: block b
+// belongs to the last matrix whose fix_begin is at most b (ROWS matrices have no blocks).
+template <typename T>
+__global__ void __launch_bounds__(256) batched_fixup_kernel(const BatchDesc<T>* __restrict__ descs, int nmat) {
+  int lo = 0, hi = nmat - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (__ldg(&descs[mid].fix_begin) <= (int)blockIdx.x)
+      lo = mid;
+    else
+      hi = mid - 1;
+  }
+  const BatchDesc<T>& d = descs[lo];
+  const int lg = split_fixup_lg(d.k), sub = threadIdx.x & ((1 << lg) - 1), local = (int)blockIdx.x - d.fix_begin;
+  if (local >= d.fix_carry_blocks) {
+    split_zero_row<T>((((long long)local - d.fix_carry_blocks) * 256 + threadIdx.x) >> lg, d.k, lg, sub, d.empty, d.nempty,
+                      d.Y, d.ldy);
+    return;
+  }
+  const long long b = ((long long)local * 256 + threadIdx.x) >> lg;
+  split_fixup_tile<T>(b < d.tiles ? (int)b : d.tiles, d.tiles, d.k, lg, sub, d.carry_row, d.carry_val, d.Y, d.ldy);
+}
+
+cudaError_t batched_fixup(int dtype, const void* descs, int nmat, int blocks, cudaStream_t s) {
+  if (blocks <= 0) return cudaSuccess;
+  if (dtype == GBS_F64)
+    batched_fixup_kernel<double><<<blocks, 256, 0, s>>>(static_cast<const BatchDesc<double>*>(descs), nmat);
+  else
+    batched_fixup_kernel<float><<<blocks, 256, 0, s>>>(static_cast<const BatchDesc<float>*>(descs), nmat);
+  return cudaGetLastError();
 }
 
 template <typename T, int VEC, bool SPLIT, int G>

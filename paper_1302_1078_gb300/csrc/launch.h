@@ -160,6 +160,9 @@ cudaError_t batched_kernel_call(bool launch, int dtype, bool split, int G, bool 
                                 int total_items, int* next_item, int grid, size_t smem, int* blocks_per_sm,
                                 cudaStream_t s);
 
+// The fix-up launch of a batch's MERGE matrices (`blocks` of 256 threads over the same descriptors).
+cudaError_t batched_fixup(int dtype, const void* descs, int nmat, int blocks, cudaStream_t s);
+
 // UCLD sums (ucld.cu): acc[0] += sum of nnz_i / (line * lines_i) over non-empty rows in 2^-31
 // fixed point, acc[1] += sum of lines_i, acc[2] += non-empty rows.
 cudaError_t launch_ucld(const int* row_ptr, const int* col_idx, int m, int line, unsigned long long* acc,

@@ -85,8 +85,7 @@ cudaError_t launch_split_t(const CsrView& A, const SplitIndex& I, const DenseVie
     if (e != cudaSuccess) return e;
   }
   if (a.tiles <= 1 && I.nempty == 0) return cudaSuccess;
-  int lg = 0;
-  while (lg < 5 && (1 << lg) < a.k) ++lg;
+  const int lg = split_fixup_lg(a.k);
   const long long carry_blocks = (((long long)a.tiles << lg) + 255) >> 8, empty_blocks = (((long long)I.nempty << lg) + 255) >> 8;
   split_fixup_kernel<T><<<(unsigned)(carry_blocks + empty_blocks), 256, 0, s>>>(
       a.tiles, a.k, lg, a.carry_row, a.carry_val, a.Y, a.ldy, I.empty, I.nempty, (int)carry_blocks);

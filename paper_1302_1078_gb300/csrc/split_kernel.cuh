@@ -338,30 +338,18 @@ __global__ void __launch_bounds__(256, PERM && sizeof(T) == 8 ? 4 : 3) split_spm
   if (tile < a.tiles) split_spmm_tile<T, VEC, G, PERM>(a, tile);
 }
 
-// Adds the tiles' carries to the rows they belong to and writes the empty rows' zeros.  2^lg lanes
-// share a tile (or an empty row) and take its columns 2^lg apart, so the reads and writes of a warp
-// are coalesced and no index is divided (with a 64-bit division per element it took 22 us of a
+// Adds the tiles' carries to the rows they belong to: lanes sub, sub + 2^lg, ... of the columns of
+// tile b (2^lg lanes share a tile; b >= tiles for none), so the reads and writes of a warp are
+// coalesced and no index is divided (with a 64-bit division per element the fix-up took 22 us of a
 // 271 us R-MAT 20 product of k = 8).  The first tile of a run of equal carry rows sums the run;
 // runs of more than eight tiles (hub rows) are summed by the whole warp, each lane every 32nd
 // carry and then a fixed shuffle tree, so that a hub of hundreds of tiles costs a few round trips.
-// The row's last tile has written its own part of the row already.
+// The row's last tile has written its own part of the row already.  Whole warps call it.
 template <typename T>
-__global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, int lg, const int* __restrict__ carry_row,
-                                                          const T* __restrict__ carry_val, T* __restrict__ Y,
-                                                          long long ldy, const int* __restrict__ empty, int nempty,
-                                                          int carry_blocks) {
+__device__ __forceinline__ void split_fixup_tile(int b, int tiles, int k, int lg, int sub,
+                                                 const int* __restrict__ carry_row, const T* __restrict__ carry_val,
+                                                 T* __restrict__ Y, long long ldy) {
   constexpr int W = 8;
-  const int lanes = 1 << lg, sub = threadIdx.x & (lanes - 1);
-  if ((int)blockIdx.x >= carry_blocks) {
-    const long long e = (((long long)blockIdx.x - carry_blocks) * 256 + threadIdx.x) >> lg;
-    if (e < nempty) {
-      T* y = Y + (long long)__ldg(empty + e) * ldy;
-      for (int c = sub; c < k; c += lanes) st_stream(y + c, T(0));
-    }
-    return;
-  }
-  const long long bl = ((long long)blockIdx.x * 256 + threadIdx.x) >> lg;
-  const int b = bl < tiles ? (int)bl : tiles;
   const int lane = threadIdx.x & 31;
   int r = -1;
   if (b < tiles) {
@@ -373,7 +361,7 @@ __global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, int 
     len = 1;
     while (len <= W && b + len < tiles && __ldcg(carry_row + b + len) == r) ++len;
     if (len <= W) {
-      for (int c = sub; c < k; c += lanes) {
+      for (int c = sub; c < k; c += 1 << lg) {
         Acc<T> s;
         for (int q = 0; q < len; ++q) s.add_partial(__ldcg(carry_val + (size_t)(b + q) * k + c));
         T* y = Y + (long long)r * ldy + c;
@@ -403,6 +391,36 @@ __global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, int 
       }
     }
   }
+}
+
+// The zeros of empty row e (e >= nempty: none), its columns shared like a tile's.
+template <typename T>
+__device__ __forceinline__ void split_zero_row(long long e, int k, int lg, int sub, const int* __restrict__ empty,
+                                               int nempty, T* __restrict__ Y, long long ldy) {
+  if (e >= nempty) return;
+  T* y = Y + (long long)__ldg(empty + e) * ldy;
+  for (int c = sub; c < k; c += 1 << lg) st_stream(y + c, T(0));
+}
+
+// Lanes that share a tile in the fix-up, as a power of two.
+__host__ __device__ inline int split_fixup_lg(int k) {
+  int lg = 0;
+  while (lg < 5 && (1 << lg) < k) ++lg;
+  return lg;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, int lg, const int* __restrict__ carry_row,
+                                                          const T* __restrict__ carry_val, T* __restrict__ Y,
+                                                          long long ldy, const int* __restrict__ empty, int nempty,
+                                                          int carry_blocks) {
+  const int sub = threadIdx.x & ((1 << lg) - 1);
+  if ((int)blockIdx.x >= carry_blocks) {
+    split_zero_row<T>((((long long)blockIdx.x - carry_blocks) * 256 + threadIdx.x) >> lg, k, lg, sub, empty, nempty, Y, ldy);
+    return;
+  }
+  const long long b = ((long long)blockIdx.x * 256 + threadIdx.x) >> lg;
+  split_fixup_tile<T>(b < tiles ? (int)b : tiles, tiles, k, lg, sub, carry_row, carry_val, Y, ldy);
 }
 
 }  // namespace gbs

@@ -153,3 +153,20 @@ def test_dvals_from_the_index(gbs, name, k, dtype):
             X, W = dev(Xw)[:, :k], dev(Ww)[:, :k]
             _, dvals = t.backward(dev(v), X[:, 0] if k == 1 else X, W[:, 0] if k == 1 else W, need_dX=False)
             within(dvals, ref, r, dtype, f"{name} k={k} ld={ld} off={off}")
+
+
+@DT
+@pytest.mark.parametrize("nnz", [98303, 98304, 98305])
+@pytest.mark.parametrize("shape", ["one_row", "even", "front"])
+def test_small_one_shot(gbs, nnz, shape, dtype):
+    """The single-launch SpMV at its largest sizes and one past them: every nonzero in one row, even
+    rows, and long rows gathered in the first block among short and empty ones."""
+    lens = {"one_row": [0, nnz, 0], "even": np.full(nnz // 7 + 1, 7), "front": [nnz // 8] * 5 + [0, 1, 2, 3] * 900}[shape]
+    lens = np.asarray(lens, np.int64)
+    lens[-1 if shape != "one_row" else 1] += nnz - lens.sum()
+    A = from_lengths(lens, 5000, 7)
+    v, x = A.vals.astype(NP[dtype]), synth.uniform(A.n, seed=37).astype(NP[dtype])
+    ref, r = oracle.spmv(A.m, A.row_ptr, A.col_idx, v, x)
+    y = torch.full((A.m,), float("nan"), dtype=dtype, device="cuda")
+    gbs.spmv_csr(dev(A.row_ptr), dev(A.col_idx), dev(v), dev(x), y)
+    within(y, ref, r, dtype, f"{shape} {nnz}")
