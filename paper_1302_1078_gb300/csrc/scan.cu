@@ -1,5 +1,7 @@
-// Exclusive prefix sum of int32 on the device (reduce, scan of block sums,
-// apply), used by the transpose's radix sort.  Integer only, in place allowed.
+// Exclusive prefix sum of int32 on the device, used by the transpose's radix
+// sort: block sums, then an apply in which each block adds up the sums before
+// its own (a launch less than a separate scan of them, which is kept for more
+// blocks than kScanDirect).  Integer only, in place allowed.
 #include <algorithm>
 
 #include "launch.h"
@@ -9,6 +11,7 @@ namespace gbs {
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
 constexpr int kScanTile = kScanThreads * kScanItems;
+constexpr int kScanDirect = 4096;  // every block reads at most 16 KB of block sums
 
 // Exclusive scan of v across the CTA (every thread calls it); returns the CTA total in *total.
 __device__ __forceinline__ int cta_exclusive_scan(int v, int* total) {
@@ -62,8 +65,17 @@ __global__ void __launch_bounds__(kScanThreads) scan_bsums_kernel(int* __restric
   }
 }
 
+// direct: bsum holds the blocks' sums, not their scan.
 __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const int* in, int* out, long long count,
-                                                                  const int* __restrict__ bsum) {
+                                                                  const int* __restrict__ bsum, bool direct) {
+  int before = 0;
+  if (direct) {
+    int part = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += kScanThreads) part += bsum[b];
+    cta_exclusive_scan(part, &before);
+  } else {
+    before = bsum[blockIdx.x];
+  }
   const long long base = (long long)blockIdx.x * kScanTile + (long long)threadIdx.x * kScanItems;
   int v[kScanItems];
   int s = 0;
@@ -73,7 +85,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_apply_kernel(const int* in,
     s += v[i];
   }
   int total;
-  int ex = cta_exclusive_scan(s, &total) + bsum[blockIdx.x];
+  int ex = cta_exclusive_scan(s, &total) + before;
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
     if (base + i < count) out[base + i] = ex;
@@ -89,9 +101,12 @@ cudaError_t exclusive_scan_i32(const int* in, int* out, long long count, int* ws
   scan_reduce_kernel<<<nb, kScanThreads, 0, s>>>(in, count, ws);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  scan_bsums_kernel<<<1, kScanThreads, 0, s>>>(ws, nb);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  scan_apply_kernel<<<nb, kScanThreads, 0, s>>>(in, out, count, ws);
+  const bool direct = nb <= kScanDirect;
+  if (!direct) {
+    scan_bsums_kernel<<<1, kScanThreads, 0, s>>>(ws, nb);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  scan_apply_kernel<<<nb, kScanThreads, 0, s>>>(in, out, count, ws, direct);
   return cudaGetLastError();
 }
 

@@ -155,6 +155,21 @@ def test_dvals_from_the_index(gbs, name, k, dtype):
             within(dvals, ref, r, dtype, f"{name} k={k} ld={ld} off={off}")
 
 
+@pytest.mark.parametrize("n", [1, 2, 512, 513, 131072, 131073, 262145])
+@pytest.mark.parametrize("nnz", [1, 4095, 4096, 4097, 70001])
+def test_transpose_tile_and_digit_edges(gbs, nnz, n):
+    """The transpose's sort at the edges of its tiles (4096 nonzeros) and digits (9 bits): the stable
+    order, the row pointers and the rows, against numpy."""
+    rng = np.random.default_rng(nnz + n)
+    lens = np.bincount(rng.integers(0, 301, nnz), minlength=301)
+    A = from_lengths(lens, n, 6)
+    rpT, ciT, perm = (t.cpu().numpy() for t in gbs.TransposePlan(dev(A.row_ptr), dev(A.col_idx), n).arrays())
+    order = np.argsort(A.col_idx, kind="stable")
+    assert np.array_equal(perm, order)
+    assert np.array_equal(ciT, np.repeat(np.arange(A.m), lens)[order])
+    assert np.array_equal(rpT, np.concatenate([[0], np.cumsum(np.bincount(A.col_idx, minlength=n))]))
+
+
 @DT
 @pytest.mark.parametrize("nnz", [98303, 98304, 98305])
 @pytest.mark.parametrize("shape", ["one_row", "even", "front"])
