@@ -244,4 +244,17 @@ struct Acc<float> {
   __device__ __forceinline__ void reset() { s = 0.f; c = 0.f; }
 };
 
+// The accumulator of the row-wise kernels (ROWS, ROWS_TMA, ROWS_DIRECT).  float: the product is
+// rounded once and added with Knuth's TwoSum, eight operations.  Their walks issue the next
+// nonzeros' loads before the current ones' sums; with Acc's two fused operations per product, both
+// on the running sum, the compiler gives that up in several instances (200,003 x 41 banded: ROWS_TMA
+// k = 2 31 -> 52 us, ROWS k = 4 60 -> 71 us).
+template <typename T>
+struct RowAcc : Acc<T> {};
+
+template <>
+struct RowAcc<float> : Acc<float> {
+  __device__ __forceinline__ void add(float a, float x) { add_partial(__fmul_rn(a, x)); }
+};
+
 }  // namespace gbs

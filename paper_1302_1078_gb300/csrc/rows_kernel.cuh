@@ -84,7 +84,7 @@ __device__ __forceinline__ void rows_block(const RowsArgs<T>& a, int block) {
   const bool col_active = SPLIT ? true : (c_lo < a.k);
   const bool col_full = SPLIT ? true : (c_lo + VEC <= a.k);
 
-  Acc<T> acc[VEC];
+  RowAcc<T> acc[VEC];
   // value of the staged entry at offset i of the tile
   auto val_at = [&](int i) -> T {
     if constexpr (PERM)
@@ -218,7 +218,7 @@ __device__ __forceinline__ void rows_direct_block(const RowsArgs<T>& a, int bloc
       return ld_keep(a.vals + p, pol_stream);
   };
   const T* __restrict__ Xc = a.X + c_lo;
-  Acc<T> acc[VEC];
+  RowAcc<T> acc[VEC];
   int p = rs;
   if (col_full) {
     for (; p + kUnroll <= re; p += kUnroll) {

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256) rows_tma_kernel(RowsArgs<T> a, int nblock
 
     // ---- compute the rows of block blk from stage st
     const bool active = g < nr;
-    Acc<T> acc[VEC];
+    RowAcc<T> acc[VEC];
     DFAcc eacc[EMUL > 0 ? VEC : 1];
     if constexpr (SPLIT) {
       {
