@@ -766,6 +766,7 @@ struct gbs_plan {
   int* col_rl = nullptr;
   void* xbuf = nullptr;
   long long ldxp = 1;
+  bool alternate = false;  // ROWS_TMA: half-warps take alternate rows
   int col_max_deg = -1;  // column-degree statistics, computed on first need
   double col_cv = 0.0;
   // SPLIT: the index of split_kernel.cuh (words, ids and empty in one allocation) and the carries
@@ -917,10 +918,13 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
     const size_t smem = rows_tma_smem(p->dtype, rpc, tile);
     // 227 KB per CTA, less the kernel's static shared memory (two blocks of row partials, and
     // of float-float pairs when emulating)
-    const size_t stat = 2 * 256 * 8 + (p->cfg.emul ? 2 * 256 * 8 : 0) + 64;
+    const size_t stat = 2 * (256 + 64) * 8 + (p->cfg.emul ? 2 * 256 * 8 : 0) + 64;
     if (tile > (1 << 14) || smem > 227 * 1024 - stat)
       return fail(GBS_EUNSUPPORTED, "row blocks too large for ROWS_TMA");
     p->cfg.tile_nnz = tile;
+    // rows of (nearly) one length: that length decides which rows of a warp share banks
+    p->alternate = p->k == 1 && p->stats.cv_row < 0.02 &&
+                   alternate_rows(lanes, (int)dsize(p->dtype), std::llround(p->stats.mean_row) * (long long)dsize(p->dtype));
     return GBS_OK;
   }
   if (!is_merge(p->cfg.variant) || p->m == 0) return GBS_OK;
@@ -946,6 +950,7 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
 int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, void* Y, long long ldy, cudaStream_t s) {
   if (s != nullptr) p->away.store(true, std::memory_order_relaxed);
   CsrView A{p->m, p->n, p->nnz, p->row_ptr, p->col_idx, vals, p->perm};
+  A.alternate = p->alternate;
   // the caller's operands decide the column access (and with it the merge geometry), also when
   // the product reads the relabelled copy of X, so that relabelling never changes a result
   const bool vec16 = dense_vec16(p->dtype, p->k, X, ldx, Y, ldy);

@@ -17,6 +17,7 @@ struct CsrView {
   const int* perm = nullptr;  // if set, the value of entry p is vals[perm[p]] (ROWS, MERGE, MERGE_DIRECT)
   int hot_cols = 0;           // > 0: columns relabelled hottest first; MERGE_DIRECT SpMV gathers
                               // columns >= hot_cols without L1 allocation
+  bool alternate = false;     // ROWS_TMA SpMV: half-warps take alternate rows
 };
 
 struct DenseView {

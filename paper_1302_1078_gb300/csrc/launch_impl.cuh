@@ -285,6 +285,7 @@ cudaError_t launch_rows_tma_t(const CsrView& A, const DenseView& D, int lanes, b
   a.row_base = 0;
   a.aligned_vals = true;
   a.aligned_cols = true;
+  a.alternate = A.alternate;
   const int rpc = threads / lanes;
   const int nblocks = (A.m + rpc - 1) / rpc;
   const size_t smem = rows_tma_smem_bytes<T>(rpc, tile);

@@ -42,6 +42,7 @@ struct RowsArgs {
   bool aligned_vals;   // vals (perm when PERM) 16-byte aligned
   bool aligned_cols;   // col_idx 16-byte aligned
   const int* __restrict__ perm = nullptr;  // PERM: value of entry p is vals[perm[p]]
+  bool alternate = false;                  // ROWS_TMA: half-warps take alternate rows (alternate_rows)
 };
 
 // Shared-memory layout: s_rp[rows + 1] | s_val[tile + 4] | s_col[tile + 4]

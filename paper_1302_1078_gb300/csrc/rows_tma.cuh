@@ -27,6 +27,8 @@
 // never masks an FP64 instruction.  The float-float partial sums are flushed
 // into the double accumulator every 16 groups (at most 48 terms).
 #pragma once
+#include <algorithm>
+
 #include "df64.cuh"
 #include "device_common.cuh"
 #include "rows_kernel.cuh"
@@ -100,6 +102,28 @@ __host__ __device__ inline size_t rows_tma_smem_bytes(int rpc, int tile) {
   size_t val = (((size_t)tile + 8) * sizeof(T) + 15) & ~(size_t)15;
   size_t col = (((size_t)tile + 8) * sizeof(int) + 15) & ~(size_t)15;
   return bars + rp + 2 * (val + col);
+}
+
+// SpMV with several lanes per row reads a value of LANES consecutive ones of each of its 32 / LANES
+// rows per step, half a warp (128 bytes) at a time.  Whether those fall on different banks depends
+// on the row length: rows of 50 doubles start 16 bytes further round the banks than the one before,
+// so four neighbouring rows overlap pairwise and rows 0, 2, 4, 6 do not at all.  Returns whether
+// half-warps should take alternate rows instead of neighbouring ones, for rows of `pitch` bytes.
+inline bool alternate_rows(int lanes, int elem, long long pitch) {
+  const int half = 16 / lanes;  // rows per half-warp
+  if (lanes < 2 || lanes > 8 || elem != 8) return false;
+  auto passes = [&](int stride) {
+    int worst = 0;
+    for (int h = 0; h < 2; ++h) {
+      int bank[16] = {};
+      for (int j = 0; j < half; ++j) {
+        const long long row = stride == 2 ? 2 * j + h : half * h + j;
+        for (int l = 0; l < lanes; ++l) worst = std::max(worst, ++bank[(row * pitch / elem + l) % 16]);
+      }
+    }
+    return worst;
+  };
+  return passes(2) < passes(1);
 }
 
 // UNIT (SpMV with contiguous x and y): the strides are 1 and drop out of every address.
@@ -177,14 +201,26 @@ __global__ void __launch_bounds__(256) rows_tma_kernel(RowsArgs<T> a, int nblock
   __syncthreads();
   if (tid == 0 && blk_of(0) < nblocks) issue(blk_of(0), 0, 0);
 
-  const int g = tid / LANES;
+  int g = tid / LANES;
+  if constexpr (SPLIT && LANES > 1 && LANES <= 8) {
+    constexpr int HALF = 16 / LANES;
+    const int w = g % (2 * HALF);  // row group inside the warp
+    if (a.alternate) g += 2 * (w % HALF) + w / HALF - w;
+  }
   const int lane = tid % LANES;
   const int c_lo = SPLIT ? 0 : lane * VEC;
   const bool col_active = SPLIT ? true : (c_lo < a.k);
   const bool col_full = SPLIT ? true : (c_lo + VEC <= a.k);
   const T* __restrict__ Xc = a.X + c_lo;
-  // row partials of the last two blocks (SpMV with LANES > 1), summed one iteration later
-  __shared__ T s_red[SPLIT && LANES > 1 ? 2 * 256 : 1];
+  // row partials of the last two blocks (SpMV with LANES > 1), summed one iteration later.  Two and
+  // four lanes: a lane's partials lie side by side, so that the summing threads, one per row, read
+  // consecutive words, and the lanes' runs are set apart by 128 / LANES bytes round the banks.
+  constexpr bool BY_LANE = SPLIT && (LANES == 2 || LANES == 4);
+  constexpr int RED = BY_LANE ? 256 + 16 * LANES : 256;
+  __shared__ T s_red[SPLIT && LANES > 1 ? 2 * RED : 1];
+  constexpr int RQ = BY_LANE ? 16 / LANES : 0;
+  const int rstride = BY_LANE ? (rpc - RQ + 15) / 16 * 16 + RQ : 1;
+  auto red_at = [&](int row, int l) { return BY_LANE ? l * rstride + row : row * LANES + l; };
   __shared__ float2 s_redf[SPLIT && LANES > 1 && EMUL > 0 ? 2 * 256 : 1];  // the lanes' float-float pairs
 
   // Wait (bounded) for block j's copy in stage j & 1 and add the arrays' last <= 3 nonzeros
@@ -212,11 +248,11 @@ __global__ void __launch_bounds__(256) rows_tma_kernel(RowsArgs<T> a, int nblock
     if constexpr (SPLIT && LANES > 1) {
       const int bj = blk_of(j);
       const int nr = rows_of(bj);
-      const T* red = s_red + (j & 1) * 256;
+      const T* red = s_red + (j & 1) * RED;
       if (tid < nr) {
-        T sum = red[tid * LANES];
+        T sum = red[red_at(tid, 0)];
 #pragma unroll
-        for (int l = 1; l < LANES; ++l) sum += red[tid * LANES + l];
+        for (int l = 1; l < LANES; ++l) sum += red[red_at(tid, l)];
         if constexpr (EMUL > 0) {
           const float2* rf = s_redf + (j & 1) * 256;
           DFAcc e;
@@ -469,8 +505,8 @@ __global__ void __launch_bounds__(256) rows_tma_kernel(RowsArgs<T> a, int nblock
     }
     const int r0 = blk * rpc;
     if constexpr (SPLIT && LANES > 1) {
-      s_red[st * 256 + tid] = acc[0].value();
-      if constexpr (EMUL > 0) s_redf[st * 256 + tid] = make_float2(eacc[0].s, eacc[0].c);
+      s_red[st * RED + red_at(g, lane)] = acc[0].value();
+      if constexpr (EMUL > 0) s_redf[st * 256 + g * LANES + lane] = make_float2(eacc[0].s, eacc[0].c);
     } else if constexpr (SPLIT) {
       if (active) st_stream(a.Y + (long long)(r0 + g) * ldy, acc[0].value());
     } else {

@@ -185,3 +185,18 @@ def test_small_one_shot(gbs, nnz, shape, dtype):
     y = torch.full((A.m,), float("nan"), dtype=dtype, device="cuda")
     gbs.spmv_csr(dev(A.row_ptr), dev(A.col_idx), dev(v), dev(x), y)
     within(y, ref, r, dtype, f"{shape} {nnz}")
+
+
+@DT
+@pytest.mark.parametrize("length", [5, 20, 27, 50, 52])
+@pytest.mark.parametrize("lanes", [2, 4, 8])
+def test_rows_tma_row_order_in_a_warp(gbs, lanes, length, dtype):
+    """SpMV with half-warps on alternate rows (decided by the row length) and the partial sums' layout:
+    every product is the one of ROWS with the same lanes within rounding, and the oracle's."""
+    A = from_lengths(np.full(777, length), 900, length)
+    v, x = A.vals.astype(NP[dtype]), synth.uniform(A.n, seed=39).astype(NP[dtype])
+    ref, r = oracle.spmv(A.m, A.row_ptr, A.col_idx, v, x)
+    plan = gbs.Plan(dev(A.row_ptr), dev(A.col_idx), A.n, dtype, 1)
+    for threads in (32, 96, 160, 256):
+        plan.set_config(dict(variant=3, lanes=lanes, threads=threads))
+        within(plan.spmv(dev(v), dev(x)), ref, r, dtype, f"lanes={lanes} threads={threads}")
