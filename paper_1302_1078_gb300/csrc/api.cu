@@ -189,10 +189,12 @@ int run_product(const CsrView& A, int dtype, int k, const void* X, long long ldx
   if (perm && cfg.variant == GBS_VARIANT_ROWS_TMA)
     return fail(GBS_EUNSUPPORTED, "values read through a permutation need the ROWS, MERGE or MERGE_DIRECT variant");
   if (cfg.variant == GBS_VARIANT_ROWS_TMA && status && aligned16(A.vals) && aligned16(A.col_idx)) {
+    // the widest panel's lanes for every panel: the tile holds the row blocks of that many lanes,
+    // and a narrower last panel with its own fewer lanes would have longer ones
+    int lanes = cfg.lanes;
+    if (k > 1) lanes = std::max(lanes, col_lanes(std::min(P, k), dtype, vec16));
     for (int c0 = 0; c0 < k; c0 += P) {
       const int kp = std::min(P, k - c0);
-      int lanes = cfg.lanes;
-      if (k > 1) lanes = std::max(lanes, col_lanes(kp, dtype, vec16));
       DenseView D{kp, static_cast<const char*>(X) + c0 * es, ldx, static_cast<char*>(Y) + c0 * es, ldy};
       e = dtype == GBS_F64 ? launch_rows_tma_f64(A, D, lanes, vec16, cfg.threads, cfg.tile_nnz, cfg.emul, status, s)
                            : launch_rows_tma_f32(A, D, lanes, vec16, cfg.threads, cfg.tile_nnz, 0, status, s);
@@ -262,6 +264,12 @@ int run_product(const CsrView& A, int dtype, int k, const void* X, long long ldx
   return rc;
 }
 
+// Nonzeros per merge thread of a block-vector product with g lanes: long shares for doubles (their
+// carry scan takes slots of the FP64 pipe) once every SM has its warps; the shortest otherwise.
+int split_block_share(long long nnz, int dtype, int g) {
+  return dtype == GBS_F64 && nnz >= 152LL * 24 * (32 / g) * 64 ? 64 : 32;
+}
+
 // One product without a plan: the SPLIT index from two passes over row_ptr, then the nonzero-split
 // walk, whatever the row lengths.  GBS_ENOMEM (nothing launched) if its scratch cannot be had.
 int run_split_once(const CsrView& A, int dtype, int k, const void* X, long long ldx, void* Y, long long ldy,
@@ -271,10 +279,7 @@ int run_split_once(const CsrView& A, int dtype, int k, const void* X, long long 
   const int P = panel_cols(dtype, vec16), kp_max = std::min(P, k);
   const bool spmv = k == 1 && ldx == 1 && ldy == 1;
   const int g = spmv ? 1 : col_lanes(kp_max, dtype, vec16);
-  // long shares for doubles (their carry scan takes slots of the FP64 pipe) once every SM has its
-  // warps; the shortest otherwise
-  int share = spmv ? kSplitShare : 32;
-  if (!spmv && dtype == GBS_F64 && split_tiles(A.nnz, g, 64) >= 152 * 24) share = 64;
+  const int share = spmv ? kSplitShare : split_block_share(A.nnz, dtype, g);
   const size_t tiles = (size_t)split_tiles(A.nnz, g, share), es = dsize(dtype);
   auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
   const size_t b_words = up(sizeof(SplitWord) * (size_t)(((long long)A.nnz + 31) / 32));
@@ -767,6 +772,7 @@ struct gbs_plan {
   void* xbuf = nullptr;
   long long ldxp = 1;
   bool alternate = false;  // ROWS_TMA: half-warps take alternate rows
+  int tile_scalar = 0;     // ROWS_TMA: the tile of calls without 128-bit column access (more lanes, fewer rows)
   int col_max_deg = -1;  // column-degree statistics, computed on first need
   double col_cv = 0.0;
   // SPLIT: the index of split_kernel.cuh (words, ids and empty in one allocation) and the carries
@@ -840,7 +846,10 @@ void split_release(gbs_plan* p) {
 // The index (built once) and the carries of a plan whose configuration is SPLIT.
 int split_prepare(gbs_plan* p, cudaStream_t s) {
   gbs_config& c = p->cfg;
-  if (c.items == 0) c.items = p->k == 1 ? kSplitShare : p->dtype == GBS_F64 ? 64 : 32;
+  if (c.items == 0) {
+    const int g = std::min(32, pow2ceil((std::min(p->k, 64) + vec_of(p->dtype) - 1) / vec_of(p->dtype)));
+    c.items = p->k == 1 ? kSplitShare : split_block_share(p->nnz, p->dtype, g);
+  }
   if (p->k == 1 ? c.items != kSplitShare : c.items % 32 || c.items < 32 || c.items > 256)
     return fail(GBS_EINVAL, "SPLIT items must be 8 (k = 1), or a multiple of 32 up to 256 (k > 1)");
   cudaError_t e = cudaSuccess;
@@ -903,9 +912,11 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
   if (!p->tuning) split_release(p);
   if (p->cfg.variant == GBS_VARIANT_ROWS_TMA && p->m > 0) {
     // the tile must hold the largest row block: measure it on the device
-    int lanes = p->cfg.lanes;
-    if (p->k > 1) lanes = std::max(lanes, col_lanes(std::min(panel_cols(p->dtype, true), p->k), p->dtype, true));
-    const int rpc = p->cfg.threads / lanes;
+    auto lanes_of = [&](bool vec16) {
+      return p->k == 1 ? p->cfg.lanes
+                       : std::max(p->cfg.lanes, col_lanes(std::min(panel_cols(p->dtype, vec16), p->k), p->dtype, vec16));
+    };
+    const int lanes = lanes_of(true), rpc = p->cfg.threads / lanes;
     if (!p->status) {
       cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&p->status), 256, s);
       if (e == cudaSuccess) e = cudaMemsetAsync(p->status, 0, 256, s);
@@ -922,6 +933,14 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
     if (tile > (1 << 14) || smem > 227 * 1024 - stat)
       return fail(GBS_EUNSUPPORTED, "row blocks too large for ROWS_TMA");
     p->cfg.tile_nnz = tile;
+    // a call without 128-bit column access has more lanes per row and so shorter row blocks: its own
+    // tile, as a larger one would only hold fewer CTAs (banded 200,003 x 41, FP32, k = 3: 61 -> 37 us)
+    p->tile_scalar = tile;
+    if (p->k > 1 && lanes_of(false) > lanes) {
+      rc = block_max_nnz(p->row_ptr, p->m, p->cfg.threads / lanes_of(false), &mx, s);
+      if (rc) return rc;
+      p->tile_scalar = std::min(tile, ((mx + 8 + 31) / 32) * 32);
+    }
     // rows of (nearly) one length: that length decides which rows of a warp share banks
     p->alternate = p->k == 1 && p->stats.cv_row < 0.02 &&
                    alternate_rows(lanes, (int)dsize(p->dtype), std::llround(p->stats.mean_row) * (long long)dsize(p->dtype));
@@ -984,7 +1003,9 @@ int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, 
     MergeBuffers mb = p->mb;
     return run_product(A, p->dtype, p->k, X, ldx, Y, ldy, p->cfg, &mb, p->coords_ready, s, nullptr, as);
   }
-  return run_product(A, p->dtype, p->k, X, ldx, Y, ldy, p->cfg, nullptr, false, s, p->status, as);
+  gbs_config c = p->cfg;
+  if (c.variant == GBS_VARIANT_ROWS_TMA && p->k > 1 && !vec16) c.tile_nnz = p->tile_scalar;
+  return run_product(A, p->dtype, p->k, X, ldx, Y, ldy, c, nullptr, false, s, p->status, as);
 }
 
 // The untuned configuration of a plan: heuristic_config's, except that skewed rows take the forms a
@@ -992,12 +1013,42 @@ int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, 
 // SPLIT); a vector takes the direct merge walk, which needs no index beyond the tiles' coordinates.
 gbs_config plan_default_config(const gbs_plan* p) {
   gbs_config c = heuristic_config(p->stats, p->dtype, p->k);
-  if (c.variant != GBS_VARIANT_MERGE) return c;
+  if (c.variant != GBS_VARIANT_MERGE) {
+    if (p->k == 1 || p->perm) return c;
+    // block vectors on even rows: short rows without staging (1400^2 grid, FP64, k = 4: ROWS 102 us,
+    // ROWS_DIRECT 74; 300,000 x 12 banded, k = 8: 56 and 54), longer ones through the bulk-copy
+    // pipeline, whose row blocks then fit (200,003 x 41 banded, FP32, k = 4: ROWS 60 us, ROWS_TMA
+    // 34).  Columns that allow no 128-bit access and many FP32 columns make the rows' lanes many
+    // and the blocks few: ROWS_DIRECT up to longer rows (50^3 stencil, FP64, k = 3: 27 and 30 us;
+    // 200,003 x 41, FP32, k = 13: 97 and 112)
+    c = gbs_config{};
+    const bool scalar = p->k % vec_of(p->dtype) != 0;
+    const double direct_to = p->k > 8 && p->dtype == GBS_F32 ? 64.0 : scalar ? 32.0 : 16.0;
+    c.variant = p->stats.mean_row < direct_to ? GBS_VARIANT_ROWS_DIRECT : GBS_VARIANT_ROWS_TMA;
+    c.threads = 256;
+    if (c.variant == GBS_VARIANT_ROWS_TMA) {
+      // 128 threads, fewer where two CTAs' double-buffered row blocks would not fit an SM
+      const int lanes = col_lanes(std::min(panel_cols(p->dtype, true), p->k), p->dtype, true);
+      c.threads = 128;
+      while (c.threads > 32 && c.threads > lanes &&
+             2.0 * c.threads / lanes * p->stats.mean_row * (double)(dsize(p->dtype) + 4) > 96.0 * 1024)
+        c.threads /= 2;
+    }
+    return normalize(c, p->dtype);
+  }
   c = gbs_config{};
   c.variant = p->k > 1 ? GBS_VARIANT_SPLIT : GBS_VARIANT_MERGE_DIRECT;
   c.threads = 128;
   c.items = p->k > 1 ? 0 : 8;
   return normalize(c, p->dtype);
+}
+
+// plan_prepare for plan_default_config's choice: ROWS where the row blocks do not fit ROWS_TMA.
+int plan_prepare_default(gbs_plan* p, cudaStream_t s) {
+  const int rc = plan_prepare(p, s);
+  if (rc != GBS_EUNSUPPORTED || p->cfg.variant != GBS_VARIANT_ROWS_TMA) return rc;
+  p->cfg = heuristic_config(p->stats, p->dtype, p->k);
+  return plan_prepare(p, s);
 }
 
 // Candidate configurations for the tuner.
@@ -1091,8 +1142,10 @@ std::vector<gbs_config> tune_candidates(const gbs_plan* p) {
 
 int plan_tune(gbs_plan* p, cudaStream_t s) {
   const size_t es = dsize(p->dtype);
-  const long long ld = p->k == 1 ? 1 : ((p->k + 1) / 2 * 2);  // even leading dimension keeps 16-byte rows for f64
-  const long long ldp = p->dtype == GBS_F64 ? ld : ((p->k + 3) / 4 * 4);
+  // operands without padding, as a contiguous X has: with an odd number of columns its rows allow no
+  // 128-bit access, which decides the kernels' instances and with them the order of the candidates
+  // (timed on padded rows, the 50^3 stencil's k = 3 took merge-path: 66 us where ROWS takes 29)
+  const long long ldp = p->k;
   void *vals = nullptr, *X = nullptr, *Y = nullptr;
   size_t bv = std::max<size_t>(16, (size_t)p->nnz * es);
   size_t bx = std::max<size_t>(16, (size_t)p->n * (p->k == 1 ? 1 : ldp) * es);
@@ -1242,7 +1295,7 @@ int plan_create_impl(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr,
   rc = compute_stats(m, n, nnz, row_ptr, &p->stats, s);
   if (rc == GBS_OK) {
     p->cfg = plan_default_config(p);
-    rc = (flags & GBS_PLAN_TUNE) && m > 0 ? plan_tune(p, s) : plan_prepare(p, s);
+    rc = (flags & GBS_PLAN_TUNE) && m > 0 ? plan_tune(p, s) : plan_prepare_default(p, s);
   }
   if (rc != GBS_OK) {
     plan_destroy_impl(p);
@@ -1314,7 +1367,7 @@ int gbs_plan_set_config(gbs_plan* plan, const gbs_config* cfg) {
   DeviceGuard guard(plan->device);
   quiesce(plan->away);
   plan->cfg = c;
-  return plan_prepare(plan, nullptr);
+  return cfg->variant == GBS_VARIANT_AUTO ? plan_prepare_default(plan, nullptr) : plan_prepare(plan, nullptr);
 }
 
 int spmv_csr_plan(const gbs_plan* plan, const void* vals, const void* x, void* y, void* stream) {
@@ -1806,10 +1859,11 @@ constexpr size_t kBatchSmemBudget = 54 * 1024;
 size_t rows_smem_host(int dtype, int rpc, int tile) {
   return dtype == GBS_F64 ? rows_smem_bytes<double>(rpc, tile) : rows_smem_bytes<float>(rpc, tile);
 }
-// Nonzeros per merge thread of a MERGE matrix from its configuration's items (0: the default).
-int batch_share(int items, int dtype, int k) {
+// Nonzeros per merge thread of a MERGE matrix from its configuration's items (0: the default for a
+// product of the whole batch's nonzeros).
+int batch_share(int items, int dtype, int k, int g, long long batch_nnz) {
   if (k == 1) return kSplitShare;
-  if (items <= 0) return dtype == GBS_F64 ? 64 : 32;
+  if (items <= 0) return split_block_share(batch_nnz, dtype, g);
   return std::min(256, (items + 31) / 32 * 32);
 }
 
@@ -2031,6 +2085,8 @@ int batched_plan_make(gbs_batch_plan** out, int nmat, const gbs_batch_item* item
   g_err.clear();
 
   // ---- work list, shared memory, merge scratch
+  long long batch_nnz = 0;
+  for (const gbs_batch_item& it : p->items) batch_nnz += it.nnz;
   p->item_begin.assign(nmat + 1, 0);
   p->fix_begin.assign(nmat + 1, 0);
   size_t scratch_total = 0;
@@ -2049,7 +2105,7 @@ int batched_plan_make(gbs_batch_plan** out, int nmat, const gbs_batch_item* item
       p->smem = std::max(p->smem, rows_smem_host(dtype, rpc, p->cfgs[b].tile_nnz));
     } else {
       auto& sp = p->splits[b];
-      sp.share = batch_share(c.items, dtype, k);
+      sp.share = batch_share(c.items, dtype, k, p->G, batch_nnz);
       sp.tiles = (int)split_tiles(it.nnz, p->G, sp.share);
       const int per = batch_item_tiles(k);
       nitems = it.m > 0 ? (sp.tiles + per - 1) / per : 0;

@@ -188,6 +188,30 @@ def test_small_one_shot(gbs, nnz, shape, dtype):
 
 
 @DT
+@pytest.mark.parametrize("k", [2, 3, 33, 40, 66, 70])
+@pytest.mark.parametrize("name", ["stencil2d_37", "even50", "random_rect"])
+def test_rows_tma_tiles_of_both_widths(gbs, name, k, dtype):
+    """ROWS_TMA block vectors whose calls have and lack 128-bit column access (different lanes, so
+    different row blocks and tiles), several column panels of which the last is narrow, and the
+    untuned choice for even rows."""
+    A = from_lengths(np.full(1001, 50), 700, 8) if name == "even50" else MATRICES[name]()
+    v = A.vals.astype(NP[dtype])
+    ld = -(-(k + 1) // 4) * 4
+    Xw = synth.uniform(A.n * ld, seed=38, stream=k).reshape(A.n, ld).astype(NP[dtype])
+    ref, r = oracle.spmm(A.m, A.row_ptr, A.col_idx, v, Xw[:, :k])
+    plan = gbs.Plan(dev(A.row_ptr), dev(A.col_idx), A.n, dtype, k)
+    for cfg in (None, dict(variant=3, threads=64), dict(variant=3, threads=256), dict(variant=3, lanes=8, threads=128)):
+        if cfg is not None:
+            try:
+                plan.set_config(cfg)
+            except gbs.GbsError as e:
+                assert e.status == -8 and cfg["threads"] == 256  # the widest row blocks exceed shared memory
+                continue
+        for X in (dev(Xw[:, :k]), dev(Xw)[:, :k]):
+            within(plan.spmm(dev(v), X), ref, r, dtype, f"{name} k={k} {cfg} ld={X.stride(0)}")
+
+
+@DT
 @pytest.mark.parametrize("length", [5, 20, 27, 50, 52])
 @pytest.mark.parametrize("lanes", [2, 4, 8])
 def test_rows_tma_row_order_in_a_warp(gbs, lanes, length, dtype):
@@ -200,3 +224,4 @@ def test_rows_tma_row_order_in_a_warp(gbs, lanes, length, dtype):
     for threads in (32, 96, 160, 256):
         plan.set_config(dict(variant=3, lanes=lanes, threads=threads))
         within(plan.spmv(dev(v), dev(x)), ref, r, dtype, f"lanes={lanes} threads={threads}")
+
