@@ -98,7 +98,7 @@ gbs_config normalize(const gbs_config& c, int dtype) {
   gbs_config r = c;
   if (r.threads <= 0) r.threads = 256;
   if (r.variant == GBS_VARIANT_ROWS_DIRECT && r.lanes <= 0) r.lanes = 1;
-  if (c.variant == GBS_VARIANT_SPLIT && c.threads <= 0) r.threads = 128;
+  if (c.variant == GBS_VARIANT_SPLIT && c.threads <= 0) r.threads = split_threads(dtype, 1);
   if (r.variant == GBS_VARIANT_ROWS || r.variant == GBS_VARIANT_ROWS_TMA) {
     if (r.lanes <= 0) r.lanes = 1;
     if (r.tile_nnz <= 0) r.tile_nnz = dtype == GBS_F64 ? 2048 : 3072;
@@ -302,8 +302,8 @@ int run_split_once(const CsrView& A, int dtype, int k, const void* X, long long 
   e = split_build(dtype, A.m, A.nnz, A.row_ptr, words, ids, nonempty, nullptr, counts, k, Y, ldy, s);
   for (int c0 = 0; e == cudaSuccess && c0 < k; c0 += P) {
     DenseView D{std::min(P, k - c0), static_cast<const char*>(X) + c0 * es, ldx, static_cast<char*>(Y) + c0 * es, ldy};
-    e = dtype == GBS_F64 ? launch_split_f64(A, I, D, vec16, 64, share, S, s)
-                         : launch_split_f32(A, I, D, vec16, 64, share, S, s);
+    e = dtype == GBS_F64 ? launch_split_f64(A, I, D, vec16, split_threads(dtype, k), share, S, s)
+                         : launch_split_f32(A, I, D, vec16, split_threads(dtype, k), share, S, s);
   }
   const cudaError_t e2 = scratch_free(base, s);
   if (e == cudaSuccess) e = e2;
@@ -1038,7 +1038,7 @@ gbs_config plan_default_config(const gbs_plan* p) {
   }
   c = gbs_config{};
   c.variant = p->k > 1 ? GBS_VARIANT_SPLIT : GBS_VARIANT_MERGE_DIRECT;
-  c.threads = 128;
+  c.threads = p->k > 1 ? split_threads(p->dtype, p->k) : 128;
   c.items = p->k > 1 ? 0 : 8;
   return normalize(c, p->dtype);
 }
@@ -1094,7 +1094,7 @@ std::vector<gbs_config> tune_candidates(const gbs_plan* p) {
     // power-law rows: SPLIT won on every skewed matrix measured (R-MAT 20 and 22, FP64 and FP32),
     // so the merge-path forms, which win where most rows are empty or of one nonzero, are tried
     // only at the shapes that led before it (15 items staged; the direct walk's 8 to 11)
-    for (int th : {64, 128}) add(GBS_VARIANT_SPLIT, 0, th, 0, 0);
+    for (int th : {64, 96}) add(GBS_VARIANT_SPLIT, 0, th, 0, 0);
     add(GBS_VARIANT_MERGE, 0, 256, 0, 15);
     for (int it : {8, 9, 11}) add(GBS_VARIANT_MERGE_DIRECT, 0, 128, 0, it);
     add(GBS_VARIANT_MERGE_DIRECT, 0, 64, 0, 8);
@@ -2247,8 +2247,8 @@ int spmv_csr_batched_looped(gbs_batch_plan* p, void* stream) {
     if (is_merge(c.variant)) {
       const auto& sp = p->splits[b];
       const DenseView D{p->k, it.X, p->k == 1 ? 1 : it.ldx, it.Y, p->k == 1 ? 1 : it.ldy};
-      const cudaError_t e = p->dtype == GBS_F64 ? launch_split_f64(A, sp.index, D, p->vec16, 64, sp.share, sp.scratch, s)
-                                                : launch_split_f32(A, sp.index, D, p->vec16, 64, sp.share, sp.scratch, s);
+      const cudaError_t e = p->dtype == GBS_F64 ? launch_split_f64(A, sp.index, D, p->vec16, split_threads(p->dtype, p->k), sp.share, sp.scratch, s)
+                                                : launch_split_f32(A, sp.index, D, p->vec16, split_threads(p->dtype, p->k), sp.share, sp.scratch, s);
       if (e != cudaSuccess) return cuda_fail(e, "batched loop launch");
       continue;
     }

@@ -3,6 +3,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "gbspmv.h"
+
 namespace gbs {
 
 // Stream-ordered device memory from the library's own pool (scratch.cu).
@@ -56,6 +58,10 @@ struct SplitScratch {
 
 // Nonzeros per merge thread of the SPLIT SpMV (x and y contiguous): one 32-byte sector of column ids.
 constexpr int kSplitShare = 8;
+// Threads per CTA of a SPLIT launch.  A float vector's CTAs of two warps end faster than new ones
+// begin: three warps there (2M x 50 banded: 64 threads 204 us, 96 175, 128 182); the others keep two,
+// which leave the smallest last wave (doubles: 281, 282, 282; R-MAT 22 257, 258, 261).
+inline int split_threads(int dtype, int k) { return k == 1 && dtype == GBS_F32 ? 96 : 64; }
 
 // SPLIT variant.  share: nonzeros per merge thread of SpMM (a multiple of 32).  vec16 as for ROWS; values through A.perm if set.
 cudaError_t launch_split_f64(const CsrView& A, const SplitIndex& I, const DenseView& D, bool vec16, int threads,

@@ -6,6 +6,7 @@
 // a long row are written by its whole warp.
 #include <algorithm>
 
+#include "dependent.cuh"
 #include "gbspmv.h"
 #include "launch.h"
 
@@ -36,6 +37,7 @@ __device__ __forceinline__ void split_mark(int s, int e, int number, SplitWord* 
 __global__ void __launch_bounds__(256) split_count_kernel(const int* __restrict__ rp, int m, int rows_per_block,
                                                           SplitWord* __restrict__ words, int nwords,
                                                           int* __restrict__ counts) {
+  allow_next();
   for (long long w = (long long)blockIdx.x * 256 + threadIdx.x; w < nwords; w += (long long)gridDim.x * 256)
     words[w] = SplitWord{0u, 0};
   const long long r0 = (long long)blockIdx.x * rows_per_block, r1 = min((long long)m, r0 + rows_per_block);
@@ -58,6 +60,8 @@ __global__ void __launch_bounds__(256) split_number_kernel(const int* __restrict
                                                          const int* __restrict__ counts, int k, T* __restrict__ Y,
                                                          long long ldy) {
   __shared__ int part[2][8];
+  wait_for_previous();
+  allow_next();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int before = 0;
   for (int b = threadIdx.x; b < (int)blockIdx.x; b += 256) before += counts[b];
@@ -105,12 +109,10 @@ cudaError_t split_build(int dtype, int m, int nnz, const int* row_ptr, SplitWord
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (dtype == GBS_F64)
-    split_number_kernel<double><<<grid, 256, 0, s>>>(row_ptr, m, per, words, ids, nonempty, empty, counts, k,
-                                                   static_cast<double*>(Y), ldy);
-  else
-    split_number_kernel<float><<<grid, 256, 0, s>>>(row_ptr, m, per, words, ids, nonempty, empty, counts, k,
-                                                  static_cast<float*>(Y), ldy);
-  return cudaGetLastError();
+    return launch_dependent(split_number_kernel<double>, grid, 256, s, row_ptr, m, per, words, ids, nonempty, empty,
+                            counts, k, static_cast<double*>(Y), ldy);
+  return launch_dependent(split_number_kernel<float>, grid, 256, s, row_ptr, m, per, words, ids, nonempty, empty, counts,
+                          k, static_cast<float*>(Y), ldy);
 }
 
 long long split_tiles(int nnz, int g, int share) {

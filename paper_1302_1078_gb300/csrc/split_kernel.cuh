@@ -37,6 +37,7 @@
 // 20, k = 8, forward: 238 -> 134 us; the staged merge walk issued about 150
 // warp instructions per 16 nonzeros, most of them in divergent row ends).
 #pragma once
+#include "dependent.cuh"
 #include "device_common.cuh"
 #include "launch.h"
 
@@ -226,6 +227,8 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
 
 template <typename T, bool PERM>
 __global__ void __launch_bounds__(256, 5) split_spmv_kernel(SplitArgs<T> a) {
+  wait_for_previous();
+  allow_next();
   const int tile = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   if (tile < a.tiles) split_spmv_tile<T, PERM>(a, tile);
 }
@@ -334,6 +337,8 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
 
 template <typename T, int VEC, int G, bool PERM>
 __global__ void __launch_bounds__(256, PERM && sizeof(T) == 8 ? 4 : 3) split_spmm_kernel(SplitArgs<T> a) {
+  wait_for_previous();
+  allow_next();
   const int tile = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
   if (tile < a.tiles) split_spmm_tile<T, VEC, G, PERM>(a, tile);
 }
@@ -414,6 +419,7 @@ __global__ void __launch_bounds__(256) split_fixup_kernel(int tiles, int k, int 
                                                           const T* __restrict__ carry_val, T* __restrict__ Y,
                                                           long long ldy, const int* __restrict__ empty, int nempty,
                                                           int carry_blocks) {
+  wait_for_previous();
   const int sub = threadIdx.x & ((1 << lg) - 1);
   if ((int)blockIdx.x >= carry_blocks) {
     split_zero_row<T>((((long long)blockIdx.x - carry_blocks) * 256 + threadIdx.x) >> lg, k, lg, sub, empty, nempty, Y, ldy);

@@ -225,3 +225,35 @@ def test_rows_tma_row_order_in_a_warp(gbs, lanes, length, dtype):
         plan.set_config(dict(variant=3, lanes=lanes, threads=threads))
         within(plan.spmv(dev(v), dev(x)), ref, r, dtype, f"lanes={lanes} threads={threads}")
 
+
+@pytest.mark.parametrize("k", [1, 8])
+def test_capture_of_split_products(gbs, k):
+    """A SPLIT plan, a one-shot product (its scratch becomes the graph's) and an untuned backward pass
+    captured in one CUDA graph behind an operation that makes their input; replays follow new inputs."""
+    A = MATRICES["hubs"]()
+    rp, ci, v = dev(A.row_ptr), dev(A.col_idx), dev(A.vals)
+    tail = () if k == 1 else (k,)
+    x0 = torch.zeros((A.n, *tail), dtype=torch.float64, device="cuda")
+    dY = torch.rand((A.m, *tail), dtype=torch.float64, device="cuda")
+    plan = gbs.Plan(rp, ci, A.n, torch.float64, k, config=dict(variant=6))
+    t = gbs.TransposePlan(rp, ci, A.n)
+
+    def work():
+        x = x0 * 2.0
+        once = gbs.spmv_csr(rp, ci, v, x) if k == 1 else gbs.spmm_csr(rp, ci, v, x)
+        return (plan.spmv(v, x) if k == 1 else plan.spmm(v, x)), once, *t.backward(v, x, dY)
+
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        work()
+    torch.cuda.current_stream().wait_stream(side)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = work()
+    for seed in (1, 2):
+        x0.copy_(dev(synth.uniform(x0.numel(), seed=seed)).reshape(x0.shape))
+        g.replay()
+        want = work()
+        for a, b in zip(got, want):
+            assert torch.equal(a, b)
