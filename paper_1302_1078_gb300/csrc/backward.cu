@@ -98,10 +98,10 @@ __global__ void __launch_bounds__(128, K1 ? 10 : VEC * sizeof(T) == 32 ? 6 : 8) 
       T x[H][V];
 #pragma unroll
       for (int u = 0; u < H; ++u)
-        if (c[h + u] >= 0) ld_slice<T, V>(X + (long long)c[h + u] * ldx + c0, pol_keep, x[u]);
+        if (c[h + u] >= 0) ld_slice<T, V>(X + c0 + (uint64_t)(uint32_t)c[h + u] * (uint32_t)ldx, pol_keep, x[u]);
 #pragma unroll
       for (int u = 0; u < H; ++u) {
-        if (h + u == 0 || row[h + u] != row[h + u - 1]) ld_slice<T, V>(yc + (long long)row[h + u] * lddy, pol_keep, y);
+        if (h + u == 0 || row[h + u] != row[h + u - 1]) ld_slice<T, V>(yc + (uint64_t)(uint32_t)row[h + u] * (uint32_t)lddy, pol_keep, y);
         if (c[h + u] >= 0) {
 #pragma unroll
           for (int j = 0; j < V; ++j) acc[h + u].add(y[j], x[u][j]);

@@ -246,6 +246,7 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
   const int w0 = (tile * MT + mt) * nwp, w1 = min(w0 + nwp, a.nwords);
   const T* __restrict__ Xc = a.X + c_lo;
   T* __restrict__ Yc = a.Y + c_lo;
+  const uint32_t ldx = (uint32_t)a.ldx;  // one 32 x 32 -> 64-bit product per gathered row
   auto store_row = [&](int ord, const T* out) {
     T* y = Yc + (long long)split_row(ids, ord) * a.ldy;
     if (col_full)
@@ -272,15 +273,15 @@ __device__ __forceinline__ void split_spmm_tile(const SplitArgs<T>& a, int tile)
 #pragma unroll
       for (int h = 0; h < 8; h += 4) {  // four gathers in flight: eight take 110 registers, half the warps
         Vec<T, VEC> x[4];
+        if (whole && col_full) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (col_full && c[h + u] >= 0) {
-            x[u] = ld_keep_vec<T, VEC>(Xc + (long long)c[h + u] * a.ldx, pol_keep);
-          } else {
+          for (int u = 0; u < 4; ++u) x[u] = ld_keep_vec<T, VEC>(Xc + (uint64_t)(uint32_t)c[h + u] * ldx, pol_keep);
+        } else {
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
 #pragma unroll
             for (int j = 0; j < VEC; ++j)
-              x[u].v[j] = c[h + u] >= 0 && c_lo + j < a.k ? ld_keep(Xc + (long long)c[h + u] * a.ldx + j, pol_keep) : T(0);
-          }
+              x[u].v[j] = c[h + u] >= 0 && c_lo + j < a.k ? ld_keep(Xc + (uint64_t)(uint32_t)c[h + u] * ldx + j, pol_keep) : T(0);
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
