@@ -95,6 +95,7 @@ KERNEL_SOURCES = {
     3: ["rows_tma.cuh", "rows_kernel.cuh", "device_common.cuh", "df64.cuh", "launch_impl.cuh"],
     4: ["merge_kernel.cuh", "device_common.cuh", "launch_impl.cuh"],
     5: ["rows_kernel.cuh", "device_common.cuh", "launch_impl.cuh"],
+    6: ["split_kernel.cuh", "device_common.cuh", "dependent.cuh", "split_impl.cuh", "launch_impl.cuh"],
 }
 
 
@@ -317,12 +318,12 @@ def run_reference(args, rank, world):
 # -------------------------------------------------------------------- GPU arm
 
 def launches_per_call(cfg: dict, k: int, dtype_vec: int = 2) -> int:
-    """Kernels one product call launches: ROWS and ROWS_TMA 1 per column panel; MERGE partition
-    is precomputed by the plan, then kernel + carry fix-up per panel; a relabelling plan adds
-    the scatter of x into the relabelled order."""
+    """Kernels one product call launches: ROWS, ROWS_TMA and ROWS_DIRECT 1 per column panel; MERGE
+    partition and SPLIT index are precomputed by the plan, then kernel + carry fix-up per panel; a
+    relabelling plan adds the scatter of x into the relabelled order."""
     panel = 32 * dtype_vec if k > 1 else 1
     panels = (k + panel - 1) // panel
-    return panels * (1 if cfg["variant"] in (1, 3) else 2) + (1 if cfg.get("relabel", 0) else 0)
+    return panels * (1 if cfg["variant"] in (1, 3, 5) else 2) + (1 if cfg.get("relabel", 0) else 0)
 
 
 def measure_spmm(gbs, torch, dev, items, steps, warmup, ks=(4, 8, 16)):

@@ -510,8 +510,9 @@ int spmv_csr_batched_plan(gbs_batch_plan** plan, int nmat, const gbs_batch_item*
  * The same plan with the caller's per-matrix configurations: cfgs (host,
  * nmat entries) gives each matrix GBS_VARIANT_ROWS or GBS_VARIANT_MERGE with
  * its lanes (k == 1; k > 1 uses the batch's column lanes), tile_nnz or items,
- * or GBS_VARIANT_AUTO for the heuristic / tuner choice of
- * spmv_csr_batched_plan.  threads is always 256; a MERGE matrix's items are
+ * or GBS_VARIANT_AUTO for MERGE or, with
+ * GBS_PLAN_TUNE, the fastest of the matrix's standalone products under MERGE
+ * and two ROWS tiles (this writes Y_b).  threads is always 256; a MERGE matrix's items are
  * its nonzeros per merge thread, rounded up to a multiple of 32 and at most
  * 256 (k = 1: always 8).  Errors: GBS_EUNSUPPORTED (another variant), GBS_EINVAL (as
  * gbs_plan_set_config).  cfgs == NULL is spmv_csr_batched_plan.

@@ -1918,13 +1918,29 @@ void batch_free(gbs_batch_plan* p) {
 int batched_plan_make(gbs_batch_plan** out, int nmat, const gbs_batch_item* items, int dtype, int k, int flags,
                       const gbs_config* cfgs, const std::vector<gbs_stats>* known, void* stream);
 
+// Matrix b's product by itself: MERGE on the plan's index of it, ROWS as any product.
+int batched_one(gbs_batch_plan* p, int b, gbs_config c, cudaStream_t s) {
+  const gbs_batch_item& it = p->items[b];
+  if (it.m == 0) return GBS_OK;
+  const CsrView A{it.m, it.n, it.nnz, it.row_ptr, it.col_idx, it.vals};
+  const DenseView D{p->k, it.X, p->k == 1 ? 1 : it.ldx, it.Y, p->k == 1 ? 1 : it.ldy};
+  if (is_merge(c.variant)) {
+    const auto& sp = p->splits[b];
+    const auto launch = p->dtype == GBS_F64 ? launch_split_f64 : launch_split_f32;
+    const cudaError_t e = launch(A, sp.index, D, p->vec16, split_threads(p->dtype, p->k), sp.share, sp.scratch, s);
+    return e == cudaSuccess ? GBS_OK : cuda_fail(e, "batched loop launch");
+  }
+  if (p->k > 1) c.lanes = p->G;
+  return run_product(A, p->dtype, p->k, D.X, D.ldx, D.Y, D.ldy, c, nullptr, true, s);
+}
+
 }  // namespace
 
 extern "C" {
 
 int spmv_csr_batched_plan(gbs_batch_plan** out, int nmat, const gbs_batch_item* items, int dtype, int k, int flags,
                           void* stream) {
-  int rc = spmv_csr_batched_plan_cfg(out, nmat, items, dtype, k, flags, nullptr, stream);
+  int rc = batched_plan_make(out, nmat, items, dtype, k, flags, nullptr, nullptr, stream);
   if (rc || !(flags & GBS_PLAN_TUNE) || !*out || !(*out)->exec) return rc;
   // Standalone timings of a small matrix measure its launch latency, not what its items cost
   // inside a full batch.  So whole-batch policies are built and timed on the batched kernel itself,
@@ -1985,7 +2001,42 @@ int spmv_csr_batched_plan(gbs_batch_plan** out, int nmat, const gbs_batch_item* 
 
 int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_item* items, int dtype, int k,
                               int flags, const gbs_config* cfgs, void* stream) {
-  return batched_plan_make(out, nmat, items, dtype, k, flags, cfgs, nullptr, stream);
+  if (!cfgs) return spmv_csr_batched_plan(out, nmat, items, dtype, k, flags, stream);
+  const int rc = batched_plan_make(out, nmat, items, dtype, k, flags, cfgs, nullptr, stream);
+  if (rc || !(flags & GBS_PLAN_TUNE)) return rc;
+  // with the tuner, a matrix without a configuration of its own gets the fastest of its standalone
+  // products (a per-matrix caller's choice): MERGE, or ROWS with one of two tiles
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  gbs_batch_plan* base = *out;
+  std::vector<gbs_config> cf(cfgs, cfgs + nmat);
+  const int base_tile = dtype == GBS_F64 ? 2048 : 3072;
+  for (int b = 0; b < nmat; ++b) {
+    if (cf[b].variant != GBS_VARIANT_AUTO || items[b].m == 0) continue;
+    gbs_config merge{};
+    merge.variant = GBS_VARIANT_MERGE;
+    gbs_config rows{};
+    rows.variant = GBS_VARIANT_ROWS;
+    rows.lanes = k == 1 ? heuristic_config(base->stats[b], GBS_F64, 1).lanes : base->G;
+    gbs_config cand[3] = {merge, rows, rows};
+    cand[1].tile_nnz = base_tile;
+    cand[2].tile_nnz = 2 * base_tile;
+    float best = 1e30f;
+    for (gbs_config c : cand) {
+      c.threads = kBatchThreads;
+      const float ms = time_median([&] { return batched_one(base, b, c, s) == GBS_OK; }, s);
+      if (ms >= 0 && ms < best) {
+        best = ms;
+        cf[b] = c;
+      }
+    }
+  }
+  gbs_batch_plan* tuned = nullptr;
+  if (batched_plan_make(&tuned, nmat, items, dtype, k, flags & ~GBS_PLAN_TUNE, cf.data(), &base->stats, stream) == GBS_OK) {
+    batch_free(base);
+    *out = tuned;
+  }
+  g_err.clear();
+  return GBS_OK;
 }
 
 }  // extern "C"
@@ -2240,21 +2291,7 @@ int spmv_csr_batched_looped(gbs_batch_plan* p, void* stream) {
   if (!p) return fail(GBS_EINVAL, "plan is NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   for (int b = 0; b < p->nmat; ++b) {
-    const gbs_batch_item& it = p->items[b];
-    if (it.m == 0) continue;
-    CsrView A{it.m, it.n, it.nnz, it.row_ptr, it.col_idx, it.vals};
-    gbs_config c = p->cfgs[b];
-    if (is_merge(c.variant)) {
-      const auto& sp = p->splits[b];
-      const DenseView D{p->k, it.X, p->k == 1 ? 1 : it.ldx, it.Y, p->k == 1 ? 1 : it.ldy};
-      const cudaError_t e = p->dtype == GBS_F64 ? launch_split_f64(A, sp.index, D, p->vec16, split_threads(p->dtype, p->k), sp.share, sp.scratch, s)
-                                                : launch_split_f32(A, sp.index, D, p->vec16, split_threads(p->dtype, p->k), sp.share, sp.scratch, s);
-      if (e != cudaSuccess) return cuda_fail(e, "batched loop launch");
-      continue;
-    }
-    if (c.variant == GBS_VARIANT_ROWS && p->k > 1) c.lanes = p->G;
-    const int rc = run_product(A, p->dtype, p->k, it.X, p->k == 1 ? 1 : it.ldx, it.Y, p->k == 1 ? 1 : it.ldy, c, nullptr,
-                               true, s);
+    const int rc = batched_one(p, b, p->cfgs[b], s);
     if (rc) return rc;
   }
   return GBS_OK;

@@ -184,7 +184,7 @@ cudaError_t permute_run(int n, int nnz, const int* row_ptr, const int* col_idx, 
 
 // Register-blocked CRS (bcsr.cu).  bcsr_count fills bptr[mb+1] and *nblocks (synchronises s)
 // and leaves the sorted block columns in *scratch (stream-ordered allocation) for bcsr_fill,
-// which writes bcol / bval; the caller frees scratch with cudaFreeAsync.
+// which writes bcol / bval; the caller frees scratch with scratch_free.
 cudaError_t bcsr_count(int m, int n, int nnz, const int* row_ptr, const int* col_idx, int a, int b, int* bptr,
                        int** bcol_sorted, int* nblocks, void** scratch, cudaStream_t s);
 cudaError_t bcsr_fill(int m, int n, int nnz, const int* row_ptr, const int* col_idx, const void* vals, int dtype,
@@ -195,9 +195,5 @@ cudaError_t bcsr_spmv(int dtype, int a, int b, int m, int n, const int* bptr, co
 
 // Message returned by gbs_last_error() on the calling thread (api.cu).
 void set_last_error(const char* msg);
-
-// Shared-memory bytes of one CTA (host helpers).
-size_t rows_smem(int dtype, int rows_per_cta, int tile);
-size_t merge_smem(int dtype, int g, bool vec16, int threads, int items);
 
 }  // namespace gbs

@@ -372,19 +372,4 @@ cudaError_t launch_merge_t(const CsrView& A, const DenseView& D, int g, bool vec
   }
 }
 
-template <typename T>
-size_t merge_smem_t(int g, bool vec16, bool direct, int threads, int items) {
-  constexpr int V = 16 / (int)sizeof(T);
-  const int vec = vec16 ? V : 1;
-  // same formula for every G: s_cval holds threads * vec elements
-  const int nt = threads / g;
-  const size_t ipc = (size_t)nt * items;
-  size_t a = ((ipc + 2) * sizeof(int) + 15) & ~(size_t)15;
-  size_t b = direct ? 0 : ((ipc + 4) * sizeof(T) + 15) & ~(size_t)15;
-  size_t c = direct ? 0 : ((ipc + 4) * sizeof(int) + 15) & ~(size_t)15;
-  size_t d = 2 * 32 * sizeof(int);
-  size_t e = 2 * (size_t)threads * vec * sizeof(T);
-  return a + b + c + d + e;
-}
-
 }  // namespace gbs
