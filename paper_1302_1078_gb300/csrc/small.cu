@@ -16,11 +16,17 @@ namespace gbs {
 
 constexpr int kSmallThreads = 512;
 
-// Both parts of a float sum, or the double, added over 2^j lanes by a fixed tree.
-__device__ __forceinline__ void tree_add(Acc<double>& a, int o) { a.s += __shfl_xor_sync(0xffffffffu, a.s, o); }
+// The other lane's sum added to a's.  float: the lanes of a row hold a few products each, so most of
+// the sum's roundings are made here: by TwoSum, both parts.
+__device__ __forceinline__ void merge(Acc<double>& a, double s, double) { a.s += s; }
+__device__ __forceinline__ void merge(Acc<float>& a, float s, float c) {
+  a.add_partial(s);
+  a.c = __fadd_rn(a.c, c);
+}
+__device__ __forceinline__ void tree_add(Acc<double>& a, int o) { merge(a, __shfl_xor_sync(0xffffffffu, a.s, o), 0.0); }
 __device__ __forceinline__ void tree_add(Acc<float>& a, int o) {
-  a.s = __fadd_rn(a.s, __shfl_xor_sync(0xffffffffu, a.s, o));
-  a.c = __fadd_rn(a.c, __shfl_xor_sync(0xffffffffu, a.c, o));
+  const float s = __shfl_xor_sync(0xffffffffu, a.s, o), c = __shfl_xor_sync(0xffffffffu, a.c, o);
+  merge(a, s, c);
 }
 
 // Products of nonzeros p, p + step, ... < e, four gathers in flight.
@@ -53,7 +59,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_spmv_kernel(int m, const 
   constexpr int R = kSmallThreads / L, LONG = 64 * L;
   __shared__ int long_rows[R];
   __shared__ int nlong;
-  __shared__ T part_s[kSmallThreads / 32], part_c[kSmallThreads / 32];
+  __shared__ T part_s[kSmallThreads / 32], part_c[kSmallThreads / 32];  // part_c: floats only
   if (threadIdx.x == 0) nlong = 0;
   __syncthreads();
   const int lane = threadIdx.x % L, row = blockIdx.x * R + threadIdx.x / L;
@@ -80,10 +86,7 @@ __global__ void __launch_bounds__(kSmallThreads) small_spmv_kernel(int m, const 
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int w = 1; w < kSmallThreads / 32; ++w) {
-        a.s += part_s[w];
-        if constexpr (sizeof(T) == 4) a.c += part_c[w];
-      }
+      for (int w = 1; w < kSmallThreads / 32; ++w) merge(a, part_s[w], sizeof(T) == 4 ? part_c[w] : T(0));
       y[r] = a.value();
     }
     __syncthreads();

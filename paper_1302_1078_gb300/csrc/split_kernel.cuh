@@ -1,4 +1,4 @@
-// Nonzero-split CSR kernel ("SPLIT" variant, plans only) for SpMV and SpMM.
+// Nonzero-split CSR kernel ("SPLIT" variant) for SpMV and SpMM.
 //
 // Power-law rows again (see merge_kernel.cuh), split by nonzeros alone: every
 // merge thread takes the same number of consecutive nonzeros, a multiple of 8
@@ -8,7 +8,7 @@
 // without a product, and the aligned shares are read in whole 32-byte sectors
 // with 256-bit loads, nothing masked.
 //
-// What a merge thread has to know about the rows comes from a plan-time index
+// What a merge thread has to know about the rows comes from an index (split_build.cu)
 // of 8 bytes per 32 nonzeros, which replaces row_ptr and the two binary
 // searches per thread of the merge-path walk: SplitWord w holds a bitmap of
 // the nonzeros 32w .. 32w+31 that are the last of their row, and the ordinal,
@@ -33,7 +33,7 @@
 // 48 registers on an SM, 16 per lane (80 registers) are 15-20% slower.  R-MAT
 // 22 FP64 338 us (direct merge walk) -> 257 us, 0.50 of the measured HBM rate;
 // R-MAT 20 forward 95 -> 75 us.  SpMM: FP64 is bound by its pipe (R-MAT 22,
-// k = 8: 1346 -> 1049 us, 0.78 of the pipe), FP32 by instruction issue (R-MAT
+// k = 8: 1346 -> 1041 us, 0.78 of the pipe), FP32 by instruction issue (R-MAT
 // 20, k = 8, forward: 238 -> 134 us; the staged merge walk issued about 150
 // warp instructions per 16 nonzeros, most of them in divergent row ends).
 #pragma once
@@ -116,10 +116,10 @@ __device__ __forceinline__ const int* split_ids(const SplitArgs<T>& a) {
 }
 __device__ __forceinline__ int split_row(const int* __restrict__ ids, int ord) { return ids ? __ldg(ids + ord) : ord; }
 
-// The open sum of a merge thread as the carry scan combines it.  float: the accumulator's two parts
-// are added separately, so that the compensation of every share reaches the row and only the few
-// sums of the scan round; SpMV, whose shares are short and their sums many, adds them with Knuth's
-// TwoSum (200,003 x 41 banded: error against 64 bits 6.0e-8 without it, 3.6e-8 with it; merge-path had 5.8e-8).
+// The open sum of a merge thread as the carry scan combines it.  float: both parts of the
+// accumulator, the sums added with Knuth's TwoSum, so that the scan does not round (error against 64
+// bits, two plain additions, TwoSum and merge-path: 200,003 x 41 banded SpMV 6.0e-8, 3.6e-8, 5.8e-8;
+// R-MAT 20, k = 8, forward and backward 6.4e-8, 4.3e-8, 6.8e-8, for 2% of the time).
 template <typename T>
 struct Open;
 template <>
@@ -132,7 +132,6 @@ struct Open<double> {
     return o;
   }
   __device__ __forceinline__ void add(const Open& o) { s += o.s; }
-  __device__ __forceinline__ void add_exact(const Open& o) { s += o.s; }
   __device__ __forceinline__ double value() const { return s; }
 };
 template <>
@@ -146,10 +145,6 @@ struct Open<float> {
     return o;
   }
   __device__ __forceinline__ void add(const Open& o) {
-    s = __fadd_rn(s, o.s);
-    c = __fadd_rn(c, o.c);
-  }
-  __device__ __forceinline__ void add_exact(const Open& o) {
     const float t = __fadd_rn(s, o.s), b = __fsub_rn(t, s);
     c = __fadd_rn(__fadd_rn(c, o.c), __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(o.s, b)));
     s = t;
@@ -208,13 +203,13 @@ __device__ __forceinline__ void split_spmv_tile(const SplitArgs<T>& a, int tile)
     const bool take = lane - d >= hs;
     if (__any_sync(0xffffffffu, take)) {
       const Open<T> o = S.up(d);
-      if (take) S.add_exact(o);
+      if (take) S.add(o);
     }
   }
   const Open<T> before = S.up(1);
   if (ends != 0) {
     Open<T> out(head);
-    if (lane > 0) out.add_exact(before);
+    if (lane > 0) out.add(before);
     st_stream(a.Y + split_row(ids, ord - __popc(ends)), out.value());
   }
   if (lane == 31) {
