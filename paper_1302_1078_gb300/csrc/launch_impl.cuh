@@ -238,8 +238,7 @@ static cudaError_t rows_tma_go(const RowsArgs<T>& a, int nblocks, int nnz, int* 
   const cudaError_t e = persistent_cap(kern, threads, smem, gc, &cap);
   if (e != cudaSuccess) return e;
   const int grid = std::min(nblocks, cap);
-  kern<<<grid, threads, smem, s>>>(a, nblocks, nnz, status);
-  return cudaGetLastError();
+  return launch_dependent(kern, grid, threads, smem, s, a, nblocks, nnz, status);
 }
 
 template <typename T, int VEC, int LANES, bool SPLIT>

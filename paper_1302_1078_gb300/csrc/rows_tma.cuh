@@ -29,6 +29,7 @@
 #pragma once
 #include <algorithm>
 
+#include "dependent.cuh"
 #include "df64.cuh"
 #include "device_common.cuh"
 #include "rows_kernel.cuh"
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(256) rows_tma_kernel(RowsArgs<T> a, int nblock
     mbar_init(&bars[1], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  wait_for_previous();
   {
     int v0, v1;
     load_rp(blk_of(0), v0, v1);
@@ -535,6 +537,7 @@ __global__ void __launch_bounds__(256) rows_tma_kernel(RowsArgs<T> a, int nblock
     mbar_wait_bounded(&bars[i & 1], (uint32_t)((i >> 1) & 1));
     return;
   }
+  allow_next();  // here and not at the start: see launch_dependent
   if (i > 0) finish_rows(i - 1);
 }
 

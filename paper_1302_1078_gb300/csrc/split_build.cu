@@ -109,9 +109,9 @@ cudaError_t split_build(int dtype, int m, int nnz, const int* row_ptr, SplitWord
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (dtype == GBS_F64)
-    return launch_dependent(split_number_kernel<double>, grid, 256, s, row_ptr, m, per, words, ids, nonempty, empty,
+    return launch_dependent(split_number_kernel<double>, grid, 256, 0, s, row_ptr, m, per, words, ids, nonempty, empty,
                             counts, k, static_cast<double*>(Y), ldy);
-  return launch_dependent(split_number_kernel<float>, grid, 256, s, row_ptr, m, per, words, ids, nonempty, empty, counts,
+  return launch_dependent(split_number_kernel<float>, grid, 256, 0, s, row_ptr, m, per, words, ids, nonempty, empty, counts,
                           k, static_cast<float*>(Y), ldy);
 }
 

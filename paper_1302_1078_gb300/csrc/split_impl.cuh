@@ -10,7 +10,7 @@ static cudaError_t split_spmv_go(const SplitArgs<T>& a, int grid, int threads, c
   static L1Split split;
   const cudaError_t e = prefer_l1(split_spmv_kernel<T, PERM>, threads, 0, split);
   if (e != cudaSuccess) return e;
-  return launch_dependent(split_spmv_kernel<T, PERM>, grid, threads, s, a);
+  return launch_dependent(split_spmv_kernel<T, PERM>, grid, threads, 0, s, a);
 }
 
 template <typename T, int VEC, int G, bool PERM>
@@ -18,7 +18,7 @@ static cudaError_t split_spmm_go(const SplitArgs<T>& a, int grid, int threads, c
   static L1Split split;
   const cudaError_t e = prefer_l1(split_spmm_kernel<T, VEC, G, PERM>, threads, 0, split);
   if (e != cudaSuccess) return e;
-  return launch_dependent(split_spmm_kernel<T, VEC, G, PERM>, grid, threads, s, a);
+  return launch_dependent(split_spmm_kernel<T, VEC, G, PERM>, grid, threads, 0, s, a);
 }
 
 template <typename T, int VEC, bool PERM>
@@ -85,7 +85,7 @@ cudaError_t launch_split_t(const CsrView& A, const SplitIndex& I, const DenseVie
   if (a.tiles <= 1 && I.nempty == 0) return cudaSuccess;
   const int lg = split_fixup_lg(a.k);
   const long long carry_blocks = (((long long)a.tiles << lg) + 255) >> 8, empty_blocks = (((long long)I.nempty << lg) + 255) >> 8;
-  return launch_dependent(split_fixup_kernel<T>, (unsigned)(carry_blocks + empty_blocks), 256, s, a.tiles, a.k, lg,
+  return launch_dependent(split_fixup_kernel<T>, (unsigned)(carry_blocks + empty_blocks), 256, 0, s, a.tiles, a.k, lg,
                           a.carry_row, a.carry_val, a.Y, a.ldy, I.empty, I.nempty, (int)carry_blocks);
 }
 

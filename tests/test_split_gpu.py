@@ -257,3 +257,37 @@ def test_capture_of_split_products(gbs, k):
         want = work()
         for a, b in zip(got, want):
             assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("k", [1, 3, 4])
+@pytest.mark.parametrize("m", [5, 20011])
+def test_rows_tma_products_in_a_chain(gbs, m, k):
+    """Each ROWS_TMA product begins while the one before ends: a chain in which every product reads
+    what the last one wrote, behind and before a SPLIT product, with two buffers taken in turn, gives
+    the bits of products that are waited for one by one, on a stream and captured."""
+    A = from_lengths(np.full(m, 9), m, 9)
+    rp, ci, v = dev(A.row_ptr), dev(A.col_idx), dev(A.vals / 3)
+    plans = [gbs.Plan(rp, ci, A.n, torch.float64, k, config=dict(variant=q)) for q in (3, 3, 6, 3)]
+    x0 = dev(synth.uniform(m * k, seed=41)).reshape((m,) if k == 1 else (m, k))
+    bufs = [torch.empty_like(x0), torch.empty_like(x0)]
+
+    def chain(wait):
+        x = x0
+        for i in range(24):
+            p, y = plans[i % 4], bufs[i % 2]
+            (p.spmv if k == 1 else p.spmm)(v, x, y)
+            x = y
+            if wait:
+                torch.cuda.synchronize()
+        return x
+
+    want = chain(True).clone()
+    assert want.abs().max() > 0
+    for _ in range(3):
+        assert torch.equal(chain(False), want)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = chain(False)
+    bufs[0].zero_(), bufs[1].zero_()
+    g.replay()
+    assert torch.equal(out, want)
