@@ -92,7 +92,7 @@ WORKLOAD_TEXT = {
 KERNEL_SOURCES = {
     1: ["rows_kernel.cuh", "device_common.cuh", "launch_impl.cuh"],
     2: ["merge_kernel.cuh", "device_common.cuh", "launch_impl.cuh"],
-    3: ["rows_tma.cuh", "rows_kernel.cuh", "device_common.cuh", "df64.cuh", "launch_impl.cuh"],
+    3: ["rows_tma.cuh", "rows_kernel.cuh", "device_common.cuh", "df64.cuh", "dependent.cuh", "launch_impl.cuh"],
     4: ["merge_kernel.cuh", "device_common.cuh", "launch_impl.cuh"],
     5: ["rows_kernel.cuh", "device_common.cuh", "launch_impl.cuh"],
     6: ["split_kernel.cuh", "device_common.cuh", "dependent.cuh", "split_impl.cuh", "launch_impl.cuh"],

@@ -453,8 +453,9 @@ int gbs_tplan_get_config(const gbs_tplan* plan, int dtype, int k, gbs_config* cf
  * calls that share such a plan must be ordered on one stream); dvals sums
  * each nonzero's k products in column order.  `plan` must come from
  * gbs_transpose_plan on the same (row_ptr, col_idx); row_ptr is unused.
- * When both dX and dvals are asked for, the dvals pass runs on a stream the
- * plan owns, concurrently with dX: it waits for the work enqueued on
+ * When both dX and dvals are asked for and A has at least 4,000,000 nonzeros,
+ * the dvals pass runs on a stream the plan owns, concurrently with dX (below
+ * that the two run one after the other on `stream`): it waits for the work enqueued on
  * `stream` before the call, and `stream` waits for it before anything
  * enqueued after the call (an event each way, which stream capture
  * follows), so the call is ordered on `stream` like any other.  The plan's

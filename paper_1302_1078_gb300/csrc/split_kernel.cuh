@@ -33,7 +33,7 @@
 // 48 registers on an SM, 16 per lane (80 registers) are 15-20% slower.  R-MAT
 // 22 FP64 338 us (direct merge walk) -> 257 us, 0.50 of the measured HBM rate;
 // R-MAT 20 forward 95 -> 75 us.  SpMM: FP64 is bound by its pipe (R-MAT 22,
-// k = 8: 1346 -> 1041 us, 0.78 of the pipe), FP32 by instruction issue (R-MAT
+// k = 8: 1346 -> 1008 us, 0.81 of the pipe), FP32 by instruction issue (R-MAT
 // 20, k = 8, forward: 238 -> 134 us; the staged merge walk issued about 150
 // warp instructions per 16 nonzeros, most of them in divergent row ends).
 #pragma once
