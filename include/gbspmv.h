@@ -374,6 +374,10 @@ int gbs_plan_create(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr, 
                     int dtype, int k, int flags, void* stream);
 int gbs_plan_destroy(gbs_plan* plan);
 int gbs_plan_get_config(const gbs_plan* plan, gbs_config* cfg);
+/*
+ * Replaces the configuration.  A call that is refused leaves the plan with the one it had (should
+ * the memory of that one not be had again, products return GBS_ENOMEM until a configuration is set).
+ */
 int gbs_plan_set_config(gbs_plan* plan, const gbs_config* cfg);
 int gbs_plan_get_stats(const gbs_plan* plan, gbs_stats* out);
 /*

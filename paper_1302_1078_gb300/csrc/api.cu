@@ -111,7 +111,8 @@ struct MergeGeom {
   int g, items, ctas, kp_max;
 };
 
-int check_cfg(const gbs_config& c) {
+// A resolved configuration for a product of k columns.
+int check_cfg(const gbs_config& c, int k) {
   if (c.variant != GBS_VARIANT_ROWS && !is_merge(c.variant) && c.variant != GBS_VARIANT_ROWS_TMA &&
       c.variant != GBS_VARIANT_ROWS_DIRECT && c.variant != GBS_VARIANT_SPLIT)
     return fail(GBS_EINVAL, "variant must be ROWS, MERGE, ROWS_TMA, MERGE_DIRECT, ROWS_DIRECT or SPLIT after resolution");
@@ -123,6 +124,9 @@ int check_cfg(const gbs_config& c) {
     return fail(GBS_EINVAL, "tile_nnz must be in [32, 16384]");
   if (is_merge(c.variant) && (c.items < 0 || c.items > 256)) return fail(GBS_EINVAL, "items must be in [0, 256]");
   if (c.variant == GBS_VARIANT_SPLIT && c.threads > 256) return fail(GBS_EINVAL, "SPLIT threads must be <= 256");
+  if (c.variant == GBS_VARIANT_SPLIT && c.items != 0 &&
+      (k == 1 ? c.items != kSplitShare : c.items % 32 || c.items < 32 || c.items > 256))
+    return fail(GBS_EINVAL, "SPLIT items must be 8 (k = 1), or a multiple of 32 up to 256 (k > 1)");
   if (c.emul < 0 || c.emul > 3) return fail(GBS_EINVAL, "emul must be in [0, 3]");
   if (c.relabel < 0 || c.relabel > 1024) return fail(GBS_EINVAL, "relabel must be in [0, 1024]");
   return GBS_OK;
@@ -724,7 +728,7 @@ static int product_entry(int m, int n, int nnz, const int* row_ptr, const int* c
   if (c.relabel != 0) return fail(GBS_EINVAL, "relabel needs a plan (gbs_plan_create / gbs_plan_set_config)");
   if (c.variant == GBS_VARIANT_SPLIT) return fail(GBS_EINVAL, "SPLIT needs a plan (gbs_plan_create / gbs_plan_set_config)");
   c = normalize(c, dtype);
-  rc = check_cfg(c);
+  rc = check_cfg(c, k);
   if (rc) return rc;
   return run_product(A, dtype, k, X, ldx, Y, ldy, c, nullptr, false, s);
 }
@@ -781,6 +785,7 @@ struct gbs_plan {
   void* split_carry = nullptr;
   SplitScratch split_scratch{};
   bool tuning = false;   // the tuner is trying configurations: keep the relabelling between them
+  bool ready = true;     // what cfg needs is there; false: no product runs (plan_run)
   // What the plan owns is stream-ordered memory.  It is freed on the stream that makes the plan
   // while it is being made and on the legacy default stream afterwards, which is ordered behind
   // every use of the plan only if there was none on another stream; if there was (away), the
@@ -850,8 +855,6 @@ int split_prepare(gbs_plan* p, cudaStream_t s) {
     const int g = std::min(32, pow2ceil((std::min(p->k, 64) + vec_of(p->dtype) - 1) / vec_of(p->dtype)));
     c.items = p->k == 1 ? kSplitShare : split_block_share(p->nnz, p->dtype, g);
   }
-  if (p->k == 1 ? c.items != kSplitShare : c.items % 32 || c.items < 32 || c.items > 256)
-    return fail(GBS_EINVAL, "SPLIT items must be 8 (k = 1), or a multiple of 32 up to 256 (k > 1)");
   cudaError_t e = cudaSuccess;
   if (!p->split_base) {
     const int nempty = p->stats.empty_rows, nrows = p->m - nempty;
@@ -967,6 +970,7 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
 }
 
 int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, void* Y, long long ldy, cudaStream_t s) {
+  if (!p->ready) return fail(GBS_ENOMEM, "the plan's scratch was lost: set a configuration again");
   if (s != nullptr) p->away.store(true, std::memory_order_relaxed);
   CsrView A{p->m, p->n, p->nnz, p->row_ptr, p->col_idx, vals, p->perm};
   A.alternate = p->alternate;
@@ -1206,7 +1210,7 @@ int plan_tune(gbs_plan* p, cudaStream_t s) {
     };
     std::vector<std::pair<float, gbs_config>> timed;
     for (const gbs_config& c : tune_candidates(p)) {
-      if (check_cfg(c) != GBS_OK) continue;
+      if (check_cfg(c, p->k) != GBS_OK) continue;
       p->cfg = c;
       if (plan_prepare(p, s) != GBS_OK) continue;
       const float ms = median_ms(7);
@@ -1362,12 +1366,22 @@ int gbs_plan_relabel_ids(const gbs_plan* plan, int* newid, void* stream) {
 int gbs_plan_set_config(gbs_plan* plan, const gbs_config* cfg) {
   if (!plan || !cfg) return fail(GBS_EINVAL, "NULL pointer");
   gbs_config c = cfg->variant == GBS_VARIANT_AUTO ? plan_default_config(plan) : normalize(*cfg, plan->dtype);
-  int rc = check_cfg(c);
+  int rc = check_cfg(c, plan->k);
   if (rc) return rc;
   DeviceGuard guard(plan->device);
   quiesce(plan->away);
+  const gbs_config before = plan->cfg;
   plan->cfg = c;
-  return cfg->variant == GBS_VARIANT_AUTO ? plan_prepare_default(plan, nullptr) : plan_prepare(plan, nullptr);
+  rc = cfg->variant == GBS_VARIANT_AUTO ? plan_prepare_default(plan, nullptr) : plan_prepare(plan, nullptr);
+  plan->ready = rc == GBS_OK;
+  if (rc != GBS_OK) {
+    // refused: the plan keeps the configuration it had, whose scratch is made again
+    const std::string why = g_err;
+    plan->cfg = before;
+    plan->ready = plan_prepare(plan, nullptr) == GBS_OK;
+    g_err = why;
+  }
+  return rc;
 }
 
 int spmv_csr_plan(const gbs_plan* plan, const void* vals, const void* x, void* y, void* stream) {
@@ -2101,7 +2115,7 @@ int batched_plan_make(gbs_batch_plan** out, int nmat, const gbs_batch_item* item
         g.emul = 0;
         if (g.variant == GBS_VARIANT_ROWS && k > 1) g.lanes = p->G;
         g = normalize(g, dtype);
-        rc = check_cfg(g);
+        rc = check_cfg(g, k);
       }
       if (rc) {
         batch_free(p);

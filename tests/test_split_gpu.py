@@ -291,3 +291,32 @@ def test_rows_tma_products_in_a_chain(gbs, m, k):
     bufs[0].zero_(), bufs[1].zero_()
     g.replay()
     assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("k", [1, 3, 8])
+@pytest.mark.parametrize("kept", [dict(variant=1), dict(variant=2), dict(variant=6), dict(variant=6, items=256),
+                                  dict(variant=6, relabel=1), dict(variant=3, threads=32)], ids=str)
+def test_refused_config_leaves_the_plan_as_it_was(gbs, kept, k):
+    """A configuration that is refused, by its arguments or by the row lengths (ROWS_TMA whose row
+    blocks do not fit), changes neither the plan's configuration nor its products."""
+    A = from_lengths(np.full(40000, 60), 900, 10)
+    rp, ci, v = dev(A.row_ptr), dev(A.col_idx), dev(A.vals)
+    if k == 1 and "items" in kept:
+        kept = dict(kept, items=8)
+    plan = gbs.Plan(rp, ci, A.n, torch.float64, k, config=kept)
+    X = dev(synth.uniform(A.n * k, seed=42)).reshape((A.n,) if k == 1 else (A.n, k))
+    run = plan.spmv if k == 1 else plan.spmm
+    config, want = plan.config, run(v, X)
+    refused = [dict(variant=6, items=7 if k == 1 else 33), dict(variant=6, items=16 if k == 1 else 512),
+               dict(variant=6, items=-32), dict(variant=6, threads=512), dict(variant=2, items=300), dict(variant=99)]
+    if k == 1:
+        refused.append(dict(variant=3, lanes=1, threads=256))  # row blocks of 15,360 nonzeros
+    for bad in refused:
+        with pytest.raises(gbs.GbsError):
+            plan.set_config(bad)
+        assert plan.config == config, bad
+        assert torch.equal(run(v, X), want), bad
+    plan.set_config(dict(variant=6))
+    assert plan.config["variant"] == 6
+    plan.set_config(kept)
+    assert torch.equal(run(v, X), want)
