@@ -360,9 +360,11 @@ int spmm_csr_cfg(int m, int n, int nnz, const int* row_ptr, const int* col_idx, 
  * products on the FP32 pipe).  With GBS_PLAN_CHECK it validates the structure first.  The plan
  * keeps row_ptr and col_idx as given: they must stay valid and unchanged
  * while the plan is used.  gbs_plan_create synchronises `stream`.
- * Executing a plan allocates nothing and can be captured in a CUDA graph; with
- * a MERGE, MERGE_DIRECT, SPLIT or relabelling configuration it writes carries
- * or a copy of x that the plan owns, so its calls must be ordered on one stream.
+ * Executing a plan can be captured in a CUDA graph.  It allocates nothing, except
+ * that a block product of a MERGE, MERGE_DIRECT or SPLIT configuration whose
+ * operands allow no 128-bit column access takes its scratch stream-ordered;
+ * otherwise these configurations, and relabelling ones in any case, write carries
+ * or a copy of x that the plan owns, so such calls must be ordered on one stream.
  */
 #define GBS_PLAN_TUNE 1
 #define GBS_PLAN_CHECK 2

@@ -274,6 +274,17 @@ int split_block_share(long long nnz, int dtype, int g) {
   return dtype == GBS_F64 && nnz >= 152LL * 24 * (32 / g) * 64 ? 64 : 32;
 }
 
+// Carries of a SPLIT product with g lanes per merge thread in one stream-ordered allocation.
+cudaError_t split_carries(int nnz, int dtype, int g, int share, int kp, void** base, SplitScratch* S, cudaStream_t s) {
+  const size_t tiles = (size_t)split_tiles(nnz, g, share);
+  const size_t b_row = (sizeof(int) * tiles + 255) & ~(size_t)255;
+  const cudaError_t e = scratch_alloc(base, b_row + tiles * (size_t)kp * dsize(dtype), s);
+  if (e != cudaSuccess) return e;
+  S->carry_row = static_cast<int*>(*base);
+  S->carry_val = static_cast<char*>(*base) + b_row;
+  return cudaSuccess;
+}
+
 // One product without a plan: the SPLIT index from two passes over row_ptr, then the nonzero-split
 // walk, whatever the row lengths.  GBS_ENOMEM (nothing launched) if its scratch cannot be had.
 int run_split_once(const CsrView& A, int dtype, int k, const void* X, long long ldx, void* Y, long long ldy,
@@ -879,19 +890,13 @@ int split_prepare(gbs_plan* p, cudaStream_t s) {
       if (e == cudaSuccess) e = e2;
     }
   }
-  // carries: a call without 128-bit column access has more lanes per merge thread, so more tiles
+  // carries of the calls with 128-bit column access (and of vectors); the others take their own
   if (p->split_carry) plan_free(p, p->split_carry);
   p->split_carry = nullptr;
   const int kp = std::min(panel_cols(p->dtype, true), p->k);
-  const int g = p->k == 1 ? 1 : std::min(32, pow2ceil(kp));
-  const size_t tiles = (size_t)split_tiles(p->nnz, g, c.items);
-  const size_t b_row = (sizeof(int) * tiles + 255) & ~(size_t)255;
-  if (e == cudaSuccess) e = scratch_alloc(&p->split_carry, b_row + tiles * (size_t)kp * dsize(p->dtype), s);
-  if (e == cudaSuccess) {
-    p->split_scratch.carry_row = static_cast<int*>(p->split_carry);
-    p->split_scratch.carry_val = static_cast<char*>(p->split_carry) + b_row;
-    e = cudaStreamSynchronize(s);
-  }
+  const int g = p->k == 1 ? 1 : col_lanes(kp, p->dtype, true);
+  if (e == cudaSuccess) e = split_carries(p->nnz, p->dtype, g, c.items, kp, &p->split_carry, &p->split_scratch, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     split_release(p);
     return cuda_fail(e, "SPLIT index");
@@ -991,14 +996,25 @@ int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, 
   if (p->cfg.variant == GBS_VARIANT_SPLIT) {
     const int P = panel_cols(p->dtype, vec16);
     const size_t es = dsize(p->dtype);
-    for (int c0 = 0; p->m > 0 && c0 < p->k; c0 += P) {
-      DenseView D{std::min(P, p->k - c0), static_cast<const char*>(X) + c0 * es, ldx, static_cast<char*>(Y) + c0 * es, ldy};
-      const cudaError_t e = p->dtype == GBS_F64
-          ? launch_split_f64(A, p->split, D, vec16, p->cfg.threads, p->cfg.items, p->split_scratch, s)
-          : launch_split_f32(A, p->split, D, vec16, p->cfg.threads, p->cfg.items, p->split_scratch, s);
-      if (e != cudaSuccess) return cuda_fail(e, "SPLIT launch");
+    // without 128-bit column access a merge thread has more lanes, so there are more tiles: their
+    // carries are the call's own, as those of a merge-path plan are, and such calls of one plan may
+    // run on several streams at a time
+    SplitScratch S = p->split_scratch;
+    void* own = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (p->k > 1 && !vec16 && p->m > 0) {
+      const int kp = std::min(P, p->k);
+      e = split_carries(p->nnz, p->dtype, col_lanes(kp, p->dtype, false), p->cfg.items, kp, &own, &S, s);
+      if (e != cudaSuccess) return cuda_fail(e, "scratch (SPLIT carries)");
     }
-    return GBS_OK;
+    const auto launch = p->dtype == GBS_F64 ? launch_split_f64 : launch_split_f32;
+    for (int c0 = 0; e == cudaSuccess && p->m > 0 && c0 < p->k; c0 += P) {
+      DenseView D{std::min(P, p->k - c0), static_cast<const char*>(X) + c0 * es, ldx, static_cast<char*>(Y) + c0 * es, ldy};
+      e = launch(A, p->split, D, vec16, p->cfg.threads, p->cfg.items, S, s);
+    }
+    const cudaError_t e2 = scratch_free(own, s);
+    if (e == cudaSuccess) e = e2;
+    return e == cudaSuccess ? GBS_OK : cuda_fail(e, "SPLIT launch");
   }
   if (is_merge(p->cfg.variant)) {
     // the partition was made for 128-bit column access; if this call cannot use it the

@@ -320,3 +320,23 @@ def test_refused_config_leaves_the_plan_as_it_was(gbs, kept, k):
     assert plan.config["variant"] == 6
     plan.set_config(kept)
     assert torch.equal(run(v, X), want)
+
+
+@DT
+def test_odd_block_products_of_one_plan_on_two_streams(gbs, dtype):
+    """Block products without 128-bit column access keep their carries to themselves, so one SPLIT
+    plan serves several streams at a time: the bits are those of products made one by one."""
+    A = synth.rmat(17, ef=16, seed=6)
+    rp, ci, v = dev(A.row_ptr), dev(A.col_idx), dev(A.vals.astype(NP[dtype]))
+    plan = gbs.Plan(rp, ci, A.n, dtype, 3, config=dict(variant=6))
+    X = [dev(synth.uniform(A.n * 3, seed=43, stream=i).astype(NP[dtype])).reshape(A.n, 3) for i in range(2)]
+    want = [plan.spmm(v, x).clone() for x in X]
+    Y = [[torch.empty_like(want[i]) for _ in range(20)] for i in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    for j in range(20):
+        for i in range(2):
+            plan.spmm(v, X[i], Y[i][j], stream=streams[i])
+    torch.cuda.synchronize()
+    for i in range(2):
+        assert all(torch.equal(y, want[i]) for y in Y[i])
