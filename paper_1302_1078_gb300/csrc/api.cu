@@ -809,9 +809,10 @@ namespace {
 
 void plan_free(gbs_plan* p, void* q) { scratch_free(q, p->owner); }
 
-// Before memory that earlier products of a plan may still read is freed.
-void quiesce(std::atomic<bool>& away) {
-  if (away.exchange(false)) cudaDeviceSynchronize();
+// Before memory that earlier products of a plan may still read is freed.  `away` stays set: a graph
+// that captured one of them may be replayed after this wait, and what it reads be freed later.
+void quiesce(const std::atomic<bool>& away) {
+  if (away.load()) cudaDeviceSynchronize();
 }
 
 // The current device is `dev` for the guard's lifetime.

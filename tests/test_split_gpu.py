@@ -340,3 +340,56 @@ def test_odd_block_products_of_one_plan_on_two_streams(gbs, dtype):
     torch.cuda.synchronize()
     for i in range(2):
         assert all(torch.equal(y, want[i]) for y in Y[i])
+
+
+@pytest.mark.parametrize("k", [1, 4])
+@pytest.mark.parametrize("what", ["destroy", "set_config", "graph", "transpose"])
+def test_plan_memory_outlives_work_on_another_stream(gbs, what, k):
+    """A plan is destroyed or given another configuration, or a transpose plan destroyed, while products
+    on a side stream still read what it owns, a graph's replay among them; one-shot products on the
+    default stream then draw on the same pool.  Every result is the one of products waited for one by one."""
+    A = synth.rmat(17, ef=16, seed=8)
+    rp, ci, v = dev(A.row_ptr), dev(A.col_idx), dev(A.vals)
+    shape = (A.n,) if k == 1 else (A.n, k)
+    X = dev(synth.uniform(A.n * k, seed=44)).reshape(shape)
+    once = (lambda: gbs.spmv_csr(rp, ci, v, X)) if k == 1 else (lambda: gbs.spmm_csr(rp, ci, v, X))
+    W = dev(synth.uniform(A.m * k, seed=45)).reshape(shape)
+    side = torch.cuda.Stream()
+
+    def make():
+        if what == "transpose":
+            t = gbs.TransposePlan(rp, ci, A.n)
+            t.set_config(torch.float64, k, dict(variant=6))
+            return t, lambda out, s: out.extend(t.backward(v, X, W, stream=s))
+        # (the relabelled ids and x of a graph's ROWS plan stay where they are when its threads change)
+        p = gbs.Plan(rp, ci, A.n, torch.float64, k, config=dict(variant=1 if what == "graph" else 6, relabel=1))
+        return p, lambda out, s: out.append(p.spmv(v, X, stream=s) if k == 1 else p.spmm(v, X, stream=s))
+
+    plan, go = make()
+    want, first = [], once()
+    go(want, None)
+    for _ in range(5):
+        plan, go = make()
+        torch.cuda.synchronize()
+        got = []
+        if what == "graph":
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                for _ in range(20):
+                    go(got, None)
+            plan.set_config(dict(variant=1, relabel=1, threads=128))
+            with torch.cuda.stream(side):
+                g.replay()
+        else:
+            for _ in range(20):
+                go(got, side)
+        if what == "set_config":
+            plan.set_config(dict(variant=4, items=11))
+        else:
+            del plan, go
+        later = [once() for _ in range(10)]
+        gbs.lib().gbs_release_scratch()
+        torch.cuda.synchronize()
+        for i, y in enumerate(got):
+            assert torch.equal(y, want[i % len(want)])
+        assert all(torch.equal(y, first) for y in later)
