@@ -204,15 +204,14 @@ __device__ __forceinline__ void stage_gather(T* __restrict__ s, const T* __restr
 
 // Accumulator for one output element.  double: plain fused multiply-add in
 // double.  float: compensated summation in two floats, so that long rows keep
-// their accuracy.  The new sum t = fma(a, x, s) rounds once; its error
-// a x - (t - s) is recovered by a second fused multiply-add (Dekker's
-// Fast2Sum with the exact product in place of the addend) and collected in c.
-// s - t is exact unless |s| < |a x| or the sum cancels below half of s; it then
-// rounds by at most half an ulp of a x, which is what rounding the product
-// before adding it would cost every time.  Four operations per product, where
-// rounding the product and Knuth's TwoSum take eight: the FP32 SpMM walks are
-// bound by instruction issue (R-MAT 20, k = 8, forward and backward:
-// 651 -> 631 us; error against 64 bits 7.0e-8 -> 6.7e-8 of the 2-norm).
+// their accuracy.  The new sum t = fma(a, x, s) rounds once; its error is
+// recovered as Knuth's TwoSum does it, with the exact product in the place of
+// the second addend (a x - b rounds only far below t), and collected in c.
+// Seven operations, where rounding the product first and then TwoSum take
+// eight and lose the product's rounding error.  (Dekker's Fast2Sum in this place
+// takes four, but drops up to half an ulp of a x whenever the sum so far is
+// smaller than the product: rows of the 5-point stencil were off by 3.2e-8 in
+// the 2-norm and by 1e-4 at worst, where these seven give 2.6e-8 and 6e-8.)
 template <typename T>
 struct Acc;
 
@@ -230,7 +229,8 @@ struct Acc<float> {
   float s = 0.f, c = 0.f;
   __device__ __forceinline__ void add(float a, float x) {
     const float t = __fmaf_rn(a, x, s);
-    c = __fadd_rn(c, __fmaf_rn(a, x, __fsub_rn(s, t)));
+    const float b = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fmaf_rn(a, x, -b)));
     s = t;
   }
   // partial sums of a row come in any order of magnitude: Knuth's TwoSum

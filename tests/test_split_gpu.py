@@ -393,3 +393,60 @@ def test_plan_memory_outlives_work_on_another_stream(gbs, what, k):
         for i, y in enumerate(got):
             assert torch.equal(y, want[i % len(want)])
         assert all(torch.equal(y, first) for y in later)
+
+
+def cancelling(m, seed):
+    """FP32 rows of up to 41 nonzeros whose products are exact (values +-1, 2 and 4, x of widely
+    different size) and whose large terms cancel, at most 256 nonzeros in all (one SPLIT tile, in
+    which sums keep both parts)."""
+    rng = np.random.default_rng(seed)
+    lens = rng.choice([3, 5, 9, 41], m, p=[0.4, 0.4, 0.1, 0.1])
+    lens = lens[np.cumsum(lens) <= 256]
+    A = from_lengths(lens, 64, seed)
+    x = (rng.uniform(0.5, 1, A.n) * 2.0 ** -rng.integers(0, 24, A.n)).astype(np.float32)
+    v = rng.choice([1.0, -1.0, 2.0, 4.0], A.nnz).astype(np.float32)
+    ci = A.col_idx.copy()
+    for i in range(A.m):  # small, large, -large, ...: the pair cancels
+        s = A.row_ptr[i]
+        ci[s + 1] = ci[s + 2] = int(np.argmax(x))
+        ci[s] = int(np.argmin(x))
+        v[s + 2] = -v[s + 1]
+    return synth.CSR(A.m, A.n, A.row_ptr, ci, v), x
+
+
+def exact_rows_bound(p):
+    """|error| of a compensated sum of the exact terms p (Ogita, Rump and Oishi, 2005): u |sum| +
+    (n u)^2 / (1 - n u)^2 * sum |p|, doubled for sums of partial sums."""
+    u = 2.0**-24
+    g = p.size * u / (1 - p.size * u)
+    return 2 * (u * abs(p.sum()) + g * g * np.abs(p).sum())
+
+
+@pytest.mark.parametrize("route", ["once", "SPLIT k=1", "SPLIT k=3", "SPLIT k=4", "ROWS k=1", "ROWS k=4", "dvals"])
+@pytest.mark.parametrize("seed", [1, 2, 3])
+def test_float_sums_keep_what_cancellation_leaves(gbs, seed, route):
+    A, x = cancelling(40, seed)
+    rp, ci, v = dev(A.row_ptr), dev(A.col_idx), dev(A.vals)
+    if route == "dvals":  # the same sums as dot products over the columns
+        k = 41
+        X, W = np.zeros((A.m, k), np.float32), np.zeros((A.m, k), np.float32)
+        for i in range(A.m):
+            s, e = A.row_ptr[i : i + 2]
+            X[i, : e - s], W[i, : e - s] = x[A.col_idx[s:e]], A.vals[s:e]
+        eye = np.arange(A.m + 1, dtype=np.int32)
+        t = gbs.TransposePlan(dev(eye), dev(eye[:-1]), A.m)
+        _, got = t.backward(torch.ones(A.m, device="cuda"), dev(X), dev(W), need_dX=False)
+        got = got.double().cpu().numpy()[:, None]
+    else:
+        k = int(route[-1]) if "=" in route else 1
+        X = dev(x) if k == 1 else dev(np.repeat(x[:, None], k, 1))
+        if route == "once":
+            got = gbs.spmv_csr(rp, ci, v, X)
+        else:
+            plan = gbs.Plan(rp, ci, A.n, torch.float32, k, config=dict(variant=6 if route[0] == "S" else 1))
+            got = plan.spmv(v, X) if k == 1 else plan.spmm(v, X)
+        got = got.double().cpu().numpy().reshape(A.m, k)
+    for i in range(A.m):
+        s, e = A.row_ptr[i : i + 2]
+        p = A.vals[s:e].astype(np.float64) * x[A.col_idx[s:e]]
+        assert np.all(np.abs(got[i] - p.sum()) <= exact_rows_bound(p)), (i, got[i], p)
