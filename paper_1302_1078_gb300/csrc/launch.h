@@ -77,7 +77,7 @@ constexpr int kSplitBlocks = 2048;
 cudaError_t split_build(int dtype, int m, int nnz, const int* row_ptr, SplitWord* words, int* ids, int* nonempty,
                         int* empty, int* counts, int k, void* Y, long long ldy, cudaStream_t s);
 
-// y = A x of a small matrix in one launch, without scratch (small.cu; contiguous x and y).
+// y = A x of a small matrix of any row lengths in one launch, without scratch (small.cu; contiguous x and y).
 constexpr int kSmallNnz = 98304;
 cudaError_t launch_small_spmv(int dtype, const CsrView& A, const void* x, void* y, cudaStream_t s);
 

@@ -136,6 +136,16 @@ struct Open<double> {
     o.s = __shfl_xor_sync(0xffffffffu, s, d);
     return o;
   }
+  __device__ __forceinline__ Open of(int lane) const {
+    Open o = *this;
+    o.s = __shfl_sync(0xffffffffu, s, lane);
+    return o;
+  }
+  __device__ __forceinline__ Acc<double> acc() const {
+    Acc<double> a;
+    a.s = s;
+    return a;
+  }
   __device__ __forceinline__ void add(const Open& o) { s += o.s; }
   __device__ __forceinline__ double value() const { return s; }
 };
@@ -154,6 +164,18 @@ struct Open<float> {
     o.s = __shfl_xor_sync(0xffffffffu, s, d);
     o.c = __shfl_xor_sync(0xffffffffu, c, d);
     return o;
+  }
+  __device__ __forceinline__ Open of(int lane) const {
+    Open o = *this;
+    o.s = __shfl_sync(0xffffffffu, s, lane);
+    o.c = __shfl_sync(0xffffffffu, c, lane);
+    return o;
+  }
+  __device__ __forceinline__ Acc<float> acc() const {
+    Acc<float> a;
+    a.s = s;
+    a.c = c;
+    return a;
   }
   __device__ __forceinline__ void add(const Open& o) {
     const float t = __fadd_rn(s, o.s), b = __fsub_rn(t, s);

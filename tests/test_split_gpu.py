@@ -472,3 +472,65 @@ def test_float_hub_rows_round_once(gbs, k, length):
     got = got.double().cpu().numpy().reshape(A.m, k)[::3]
     err = (got - want) / np.spacing(want.astype(np.float32)).astype(np.float64)
     assert np.sqrt(np.mean(err**2)) <= 0.35
+
+
+def small_lengths(shape, nnz):
+    """Row lengths of at most nnz nonzeros whose long rows lie together, in one cluster's rows."""
+    rng = np.random.default_rng(nnz)
+    if shape == "block":  # 192 apiece, the rest empty
+        lens = np.zeros(max(1, nnz // 192) + 60000, np.int64)
+        lens[5 : 5 + nnz // 192] = 192
+    elif shape == "just_long":  # just above what a lane or two take by themselves
+        lens = np.zeros(70000, np.int64)
+        lens[100 : 100 + nnz // 33] = 33
+    elif shape == "hub":
+        lens = np.zeros(70000, np.int64)
+        lens[[69000, 69001, 69002]] = nnz - 6, 5, 1
+    elif shape == "few":  # 32 lanes per row
+        lens = np.zeros(9, np.int64)
+        lens[[0, 3, 8]] = nnz // 2, nnz // 3, nnz // 7
+    elif shape == "powers":
+        lens = np.minimum(rng.zipf(1.7, 20000), nnz // 10)
+        lens[np.cumsum(lens) > nnz] = 0
+    return lens
+
+
+@DT
+@pytest.mark.parametrize("nnz", [600, 4097, 32768, 98304])
+@pytest.mark.parametrize("shape", ["block", "just_long", "hub", "few", "powers"])
+def test_small_one_shot_long_rows_together(gbs, shape, nnz, dtype):
+    """The single-launch SpMV whose long rows lie together, on and off a 32-byte boundary: the cluster
+    takes their nonzeros in equal parts."""
+    A = from_lengths(small_lengths(shape, nnz), 5000, 13)
+    v, x = A.vals.astype(NP[dtype]), synth.uniform(A.n, seed=46).astype(NP[dtype])
+    ref, r = oracle.spmv(A.m, A.row_ptr, A.col_idx, v, x)
+    for off in (0, 1):
+        ci = torch.empty(A.nnz + 8, dtype=torch.int32, device="cuda")[off : off + A.nnz].copy_(dev(A.col_idx))
+        vd = torch.empty(A.nnz + 8, dtype=dtype, device="cuda")[off : off + A.nnz].copy_(dev(v))
+        y = torch.full((A.m,), float("nan"), dtype=dtype, device="cuda")
+        gbs.spmv_csr(dev(A.row_ptr), ci, vd, dev(x), y)
+        within(y, ref, r, dtype, f"{shape} {nnz} off={off}")
+        assert torch.equal(y, gbs.spmv_csr(dev(A.row_ptr), ci, vd, dev(x)))
+
+
+@pytest.mark.parametrize("shape", ["block", "just_long", "hub"])
+def test_small_one_shot_time_does_not_follow_the_row_lengths(gbs, shape):
+    """Rows that one after another took forty times merge-path's time do not take twice as long."""
+    A = from_lengths(small_lengths(shape, 98304), 60000, 14)
+    args = [dev(A.row_ptr), dev(A.col_idx), dev(A.vals), dev(synth.uniform(A.n, seed=47))]
+    y = torch.empty(A.m, dtype=torch.float64, device="cuda")
+
+    def us(**kw):
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(20):
+                gbs.spmv_csr(*args, y, **kw)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) / 20 * 1e3)
+        return min(times)
+
+    assert us() <= 2 * us(config=dict(variant=4, threads=128, items=9))
