@@ -393,8 +393,9 @@ int gbs_plan_relabel_ids(const gbs_plan* plan, int* newid, void* stream);
 /* y <- A x (plan k must be 1) or Y <- A X (ldx, ldy >= plan k). */
 int spmv_csr_plan(const gbs_plan* plan, const void* vals, const void* x, void* y, void* stream);
 /*
- * Device status of the plan's bounded waits (host `*status`; bit 0: a pipeline
- * wait of GBS_VARIANT_ROWS_TMA timed out and its CTA returned early, so the
+ * Device status of the plan's bounded waits (host `*status`; bit 0: a copy of a
+ * GBS_VARIANT_ROWS_TMA product, which untuned block-vector plans on long even
+ * rows run too, had not come after a second and its CTA returned early, so the
  * result of that call is incomplete).  Reads and clears it; synchronises `stream`.
  */
 int gbs_plan_status(gbs_plan* plan, int* status, void* stream);

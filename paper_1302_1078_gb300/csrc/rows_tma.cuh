@@ -75,9 +75,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   const uint64_t t0 = global_ns();
   for (int i = 0; i < (1 << 22); ++i) {
     if (mbar_try_wait(bar, parity)) return true;
-    if (global_ns() - t0 > limit_ns) return false;
+    if (global_ns() - t0 > limit_ns) break;
   }
-  return false;
+  // a last look: a CTA that did not run for a while (another process's turn, a debugger) may find the
+  // time up and the copy there
+  return mbar_try_wait(bar, parity);
 }
 
 
