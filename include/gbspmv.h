@@ -446,7 +446,10 @@ int gbs_tplan_prepare(gbs_tplan* plan, int dtype, int k, int flags, void* stream
  * gbs_plan_set_config.  Synchronises `stream`.
  */
 int gbs_tplan_set_config(gbs_tplan* plan, int dtype, int k, const gbs_config* cfg, void* stream);
-/* The configuration dX uses for (dtype, k): the prepared one, else the one from A^T's row statistics. */
+/*
+ * The configuration dX uses for (dtype, k): the prepared one, else the one from A^T's row statistics
+ * (SPLIT for skewed rows, with its items for operands of 128-bit column access).
+ */
 int gbs_tplan_get_config(const gbs_tplan* plan, int dtype, int k, gbs_config* cfg);
 
 /*

@@ -1677,7 +1677,13 @@ int gbs_tplan_get_config(const gbs_tplan* t, int dtype, int k, gbs_config* cfg) 
     if (pp.dtype == dtype && pp.k == k) return gbs_plan_get_config(pp.plan, cfg);
   if (!valid_dtype(dtype) || k < 1) return fail(GBS_EINVAL, "dtype or k");
   gbs_config c = heuristic_config(t->statsT, dtype, k);
-  if (c.variant == GBS_VARIANT_MERGE) c.variant = GBS_VARIANT_MERGE_DIRECT;
+  if (c.variant == GBS_VARIANT_MERGE) {  // run_split_once
+    c = gbs_config{};
+    c.variant = GBS_VARIANT_SPLIT;
+    c.threads = split_threads(dtype, k);
+    c.items = k == 1 ? kSplitShare
+                     : split_block_share(t->nnz, dtype, col_lanes(std::min(panel_cols(dtype, true), k), dtype, true));
+  }
   *cfg = c;
   return GBS_OK;
 }

@@ -534,3 +534,23 @@ def test_small_one_shot_time_does_not_follow_the_row_lengths(gbs, shape):
         return min(times)
 
     assert us() <= 2 * us(config=dict(variant=4, threads=128, items=9))
+
+
+@DT
+@pytest.mark.parametrize("k", [1, 4, 8])
+def test_config_of_an_unprepared_transpose(gbs, k, dtype):
+    """What a transpose plan reports for a (dtype, k) it has no plan for is what its dX runs: the same
+    bits when it is set."""
+    A = synth.rmat(14, ef=16, seed=9)
+    shape = (A.m,) if k == 1 else (A.m, k)
+    W = dev(synth.uniform(A.m * k, seed=49).astype(NP[dtype])).reshape(shape)
+    v, X = dev(A.vals.astype(NP[dtype])), torch.zeros_like(W)
+    t = gbs.TransposePlan(dev(A.row_ptr), dev(A.col_idx), A.n)
+    cfg = t.config(dtype, k)
+    assert cfg["variant"] == 6 and cfg["items"] > 0 and cfg["threads"] > 0
+    want, _ = t.backward(v, X, W, need_dvals=False)
+    t.set_config(dtype, k, cfg)
+    assert t.config(dtype, k) == cfg
+    assert torch.equal(t.backward(v, X, W, need_dvals=False)[0], want)
+    even = synth.stencil2d(37)
+    assert gbs.TransposePlan(dev(even.row_ptr), dev(even.col_idx), even.n).config(dtype, k)["variant"] == 1
