@@ -2194,6 +2194,7 @@ int batched_plan_make(gbs_batch_plan** out, int nmat, const gbs_batch_item* item
     } else {
       auto& sp = p->splits[b];
       sp.share = batch_share(c.items, dtype, k, p->G, batch_nnz);
+      p->cfgs[b].items = sp.share;  // the value used, for spmv_csr_batched_info
       sp.tiles = (int)split_tiles(it.nnz, p->G, sp.share);
       const int per = batch_item_tiles(k);
       nitems = it.m > 0 ? (sp.tiles + per - 1) / per : 0;

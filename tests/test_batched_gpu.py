@@ -203,3 +203,25 @@ def test_batched_hub_row_equals_looped(gbs, k, dtype):
     torch.cuda.synchronize()
     for b in range(len(Ys)):
         assert torch.equal(Ys[b], batched[b]), f"batched != looped for matrix {b}"
+
+
+@pytest.mark.parametrize("k,dtype", [(8, torch.float64), (1, torch.float64), (4, torch.float32)],
+                         ids=["k8f64", "k1f64", "k4f32"])
+@pytest.mark.parametrize("given", [None, 5, 100])
+def test_batched_info_reports_the_items_used(gbs, given, k, dtype):
+    """info() gives the nonzeros per merge thread that a MERGE matrix runs with, default or rounded from the caller's:
+    a plan made with what it reports gives the same bits."""
+    mats, Xs, Ys, _ = make_batch(SMALL[:9], k, dtype, seed=11)
+    configs = None if given is None else [dict(variant=2, items=given)] * len(mats)
+    plan = gbs.BatchedPlan(mats, Xs, Ys, configs=configs)
+    got = plan.info()["configs"]
+    assert all(c["variant"] == 2 for c in got)
+    assert {c["items"] for c in got} <= ({8} if k == 1 else {32, 64} if given is None else {32 if given == 5 else 128})
+    plan.run()
+    want = [y.clone() for y in Ys]
+    again = gbs.BatchedPlan(mats, Xs, Ys, configs=got)
+    assert again.info()["configs"] == got
+    for y in Ys:
+        y.fill_(float("nan"))
+    again.run()
+    assert all(torch.equal(y, w) for y, w in zip(Ys, want))
