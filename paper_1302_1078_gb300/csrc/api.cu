@@ -466,6 +466,15 @@ int block_max_nnz(const int* rp, int m, int rpc, int* out, cudaStream_t s) {
   return e == cudaSuccess ? GBS_OK : cuda_fail(e, "block max nnz");
 }
 
+// Lanes per row of a ROWS SpMV.  FP64: one lane per row keeps every FMA lane busy and needs no
+// reduction; long rows get more lanes so that a warp's rows finish together.
+int rows_lanes(double mean_row, int dtype) {
+  const double per = dtype == GBS_F64 ? 64.0 : 16.0;
+  int l = 1;
+  while (l < 32 && mean_row > per * l) l <<= 1;
+  return l;
+}
+
 gbs_config heuristic_config(const gbs_stats& st, int dtype, int k) {
   gbs_config c{};
   c.threads = 256;
@@ -477,16 +486,7 @@ gbs_config heuristic_config(const gbs_stats& st, int dtype, int k) {
     c.items = 0;
   } else {
     c.variant = GBS_VARIANT_ROWS;
-    if (k == 1) {
-      // FP64: one lane per row keeps every FMA lane busy and needs no reduction;
-      // long rows get more lanes so that a warp's rows finish together.
-      const double per = dtype == GBS_F64 ? 64.0 : 16.0;
-      int l = 1;
-      while (l < 32 && mean > per * l) l <<= 1;
-      c.lanes = l;
-    } else {
-      c.lanes = 0;  // column lanes follow k
-    }
+    c.lanes = k == 1 ? rows_lanes(mean, dtype) : 0;  // (k > 1: column lanes follow k)
     c.tile_nnz = dtype == GBS_F64 ? 2048 : 3072;
   }
   return normalize(c, dtype);
@@ -2053,7 +2053,7 @@ int spmv_csr_batched_plan_cfg(gbs_batch_plan** out, int nmat, const gbs_batch_it
     merge.variant = GBS_VARIANT_MERGE;
     gbs_config rows{};
     rows.variant = GBS_VARIANT_ROWS;
-    rows.lanes = k == 1 ? heuristic_config(base->stats[b], GBS_F64, 1).lanes : base->G;
+    rows.lanes = k == 1 ? rows_lanes(base->stats[b].mean_row, dtype) : base->G;
     gbs_config cand[3] = {merge, rows, rows};
     cand[1].tile_nnz = base_tile;
     cand[2].tile_nnz = 2 * base_tile;

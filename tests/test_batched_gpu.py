@@ -225,3 +225,30 @@ def test_batched_info_reports_the_items_used(gbs, given, k, dtype):
         y.fill_(float("nan"))
     again.run()
     assert all(torch.equal(y, w) for y, w in zip(Ys, want))
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32], ids=["f64", "f32"])
+def test_batched_tuned_auto_entries_take_the_lanes_of_their_dtype(gbs, dtype):
+    """The tuner's ROWS candidates for entries without a configuration: lanes from the mean row length by
+    the batch's own dtype, for skewed matrices too (whose statistics suggest no lanes)."""
+    import synth
+
+    matrices = [synth.banded(m, hbw=60, per_row=per, seed=per) for m in (100, 1000, 30000) for per in (18, 20, 48)]
+    matrices.append(synth.rmat(13, ef=8, seed=10))
+    mats, Xs, Ys, host = [], [], [], []
+    for i, A in enumerate(matrices):
+        v = torch.from_numpy(A.vals.astype(NP[dtype])).cuda()
+        x = synth.uniform(A.n, seed=50, stream=i).astype(NP[dtype])
+        mats.append((torch.from_numpy(A.row_ptr).cuda(), torch.from_numpy(A.col_idx).cuda(), v, A.n))
+        Xs.append(torch.from_numpy(x).cuda())
+        Ys.append(torch.empty(A.m, dtype=dtype, device="cuda"))
+        host.append((A, x.reshape(A.n, 1)))
+    plan = gbs.BatchedPlan(mats, Xs, Ys, configs=[None] * len(mats), tune=True)
+    for A, c in zip(matrices, plan.info()["configs"]):
+        want = 1
+        while want < 32 and A.nnz / A.m > (64.0 if dtype == torch.float64 else 16.0) * want:
+            want *= 2
+        assert c["variant"] == 2 or c["lanes"] == want, (A.name, c)
+    plan.run()
+    torch.cuda.synchronize()
+    check_vs_oracle(host, Ys, dtype)
