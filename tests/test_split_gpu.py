@@ -554,3 +554,19 @@ def test_config_of_an_unprepared_transpose(gbs, k, dtype):
     assert torch.equal(t.backward(v, X, W, need_dvals=False)[0], want)
     even = synth.stencil2d(37)
     assert gbs.TransposePlan(dev(even.row_ptr), dev(even.col_idx), even.n).config(dtype, k)["variant"] == 1
+
+
+@pytest.mark.parametrize("scale,ef", [(14, 16), (16, 16), (16, 4)])
+def test_untuned_float_vectors_are_as_accurate_as_merge_path(gbs, scale, ef):
+    """The default plan of skewed rows, FP32: no further from the exact product than the staged merge-path
+    form (a twentieth is what the order of the sums makes on one matrix)."""
+    A = synth.rmat(scale, ef=ef, seed=12, vals="u0.5_1.5")
+    v, x = A.vals.astype(np.float32), synth.uniform(A.n, seed=51).astype(np.float32)
+    ref, _ = oracle.spmv(A.m, A.row_ptr, A.col_idx, v, x)
+    rp, ci = dev(A.row_ptr), dev(A.col_idx)
+
+    def error(config):
+        y = gbs.Plan(rp, ci, A.n, torch.float32, 1, config=config).spmv(dev(v), dev(x))
+        return np.linalg.norm(y.double().cpu().numpy() - ref)
+
+    assert error(None) <= 1.05 * error(dict(variant=2))
