@@ -22,12 +22,20 @@ from ._capi import GbsError, gbs_config, gbs_stats  # noqa: F401
 __all__ = [
     "spmv_csr", "spmm_csr", "Plan", "csr_stats", "validate_csr", "default_config", "GbsError", "lib",
     "TransposePlan", "CsrOperator", "SpMMFunction", "spmm_autograd", "BatchedPlan",
+    "release_scratch",
 ]
 
 
 def lib():
     """The loaded C library (built on first use if needed)."""
     return _capi._lib or _capi.load()
+
+
+def release_scratch(device=None) -> None:
+    """Give back the device memory that the library keeps for later calls (at most 256 MB; nothing
+    in use is touched)."""
+    with torch.cuda.device(device):
+        _capi.check(lib().gbs_release_scratch(), "gbs_release_scratch")
 
 
 def _dtype_code(t: torch.Tensor) -> int:

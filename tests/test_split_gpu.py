@@ -570,3 +570,15 @@ def test_untuned_float_vectors_are_as_accurate_as_merge_path(gbs, scale, ef):
         return np.linalg.norm(y.double().cpu().numpy() - ref)
 
     assert error(None) <= 1.05 * error(dict(variant=2))
+
+
+def test_release_scratch_gives_memory_back(gbs):
+    """What one-shot products leave with the library goes back to the driver, and the next one takes it anew."""
+    A = synth.banded(400000, hbw=100, per_row=40, seed=13)
+    args = dev(A.row_ptr), dev(A.col_idx), dev(A.vals), dev(synth.uniform(A.n * 4, seed=52)).reshape(A.n, 4)
+    want = gbs.spmm_csr(*args)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    gbs.release_scratch()
+    assert torch.cuda.mem_get_info()[0] > before
+    assert torch.equal(gbs.spmm_csr(*args), want)
