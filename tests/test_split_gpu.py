@@ -582,3 +582,44 @@ def test_release_scratch_gives_memory_back(gbs):
     gbs.release_scratch()
     assert torch.cuda.mem_get_info()[0] > before
     assert torch.equal(gbs.spmm_csr(*args), want)
+
+
+@DT
+@pytest.mark.parametrize("k,ld", [(2, 2), (3, 3), (3, 4), (5, 5), (4, 4), (7, 8), (8, 8), (12, 12), (13, 13), (13, 16), (16, 16)])
+@pytest.mark.parametrize("name", ["rmat_17", "stencil2d_600"])
+def test_dvals_of_large_matrices(gbs, name, k, ld, dtype):
+    """dvals of matrices whose nonzeros a grid takes in several rounds, rows short and long, in every
+    layout of the columns."""
+    A = synth.rmat(17, ef=16, seed=14) if name == "rmat_17" else synth.stencil2d(600)
+    X = synth.uniform(A.n * ld, seed=53, stream=k).reshape(A.n, ld).astype(NP[dtype])
+    W = synth.uniform(A.m * ld, seed=54, stream=k).reshape(A.m, ld).astype(NP[dtype])
+    rows = np.repeat(np.arange(A.m), np.diff(A.row_ptr))
+    p = W[rows, :k].astype(np.float64) * X[A.col_idx, :k]
+    t = gbs.TransposePlan(dev(A.row_ptr), dev(A.col_idx), A.n)
+    _, got = t.backward(dev(A.vals.astype(NP[dtype])), dev(X)[:, :k], dev(W)[:, :k], need_dX=False)
+    within(got, p.sum(1), np.abs(p).sum(1), dtype, f"{name} k={k} ld={ld}")
+
+
+@DT
+def test_dvals_time_of_odd_columns(gbs, dtype):
+    """Thirteen columns in rows of thirteen, which no slice fits, do not take longer than sixteen (by a
+    fifth): an X row's lines are used up while they are in L1."""
+    A = synth.stencil2d(1000)
+    t = gbs.TransposePlan(dev(A.row_ptr), dev(A.col_idx), A.n)
+    v = dev(A.vals.astype(NP[dtype]))
+
+    def us(k):
+        X, W = (torch.rand((A.n, k), dtype=dtype, device="cuda") for _ in range(2))
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(10):
+                t.backward(v, X, W, need_dX=False)
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 100)
+        return min(times)
+
+    assert us(13) <= 1.2 * us(16)
