@@ -412,8 +412,7 @@ int spmm_csr_plan(const gbs_plan* plan, const void* vals, const void* X, int ldx
  *   A of each entry of A^T) and the SPLIT index of A's rows (the dvals
  *   pass); plus, only if a configuration that permutes the values first is
  *   chosen, nnz doubles of scratch.
- * It does not keep row_ptr / col_idx.  It also creates a non-blocking
- * stream and two events on the current device (spmv_csr_backward).
+ * It does not keep row_ptr / col_idx.
  * Synchronises `stream`.  The transpose is the one-time set-up of the
  * backward pass.
  */
@@ -463,9 +462,10 @@ int gbs_tplan_get_config(const gbs_tplan* plan, int dtype, int k, gbs_config* cf
  * calls that share such a plan must be ordered on one stream); dvals sums
  * each nonzero's k products in column order.  `plan` must come from
  * gbs_transpose_plan on the same (row_ptr, col_idx); row_ptr is unused.
- * When both dX and dvals are asked for and A has at least 4,000,000 nonzeros,
- * the dvals pass runs on a stream the plan owns, concurrently with dX (below
- * that the two run one after the other on `stream`): it waits for the work enqueued on
+ * When both dX and dvals are asked for and A has at least 800,000 nonzeros
+ * (4,000,000 for k = 1 in doubles), the dvals pass runs on a stream the plan
+ * owns, concurrently with dX, from the second such call on (which makes the
+ * stream; below, the two run one after the other on `stream`): it waits for the work enqueued on
  * `stream` before the call, and `stream` waits for it before anything
  * enqueued after the call (an event each way, which stream capture
  * follows), so the call is ordered on `stream` like any other.  The plan's

@@ -1441,12 +1441,15 @@ struct gbs_tplan {
   // caller's stream, concurrently with the dX product
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  bool again = false;  // a pass of both outputs has run: the next one may make the stream
 };
 
 namespace {
-// Nonzeros from which a backward pass runs dvals beside dX on a second stream.  Below, the overlap
-// gives less than the stream, its events and their calls cost (R-MAT 17, 1.9 M nonzeros: dvals 15 us).
-constexpr int kForkNnz = 4000000;
+// Nonzeros from which a backward pass runs dvals beside dX on a second stream.  Below, the events and
+// their calls cost more than the overlap gives (R-MAT 15, 0.46 M: 27 and 29 us, R-MAT 16, 0.94 M, k = 3: 44
+// and 38; banded 50,000 x 40, FP32, k = 4: 57 and 50).  A vector of doubles gains later and loses where
+// even rows keep the value gathers of dX busy (R-MAT 17 44 and 38, banded 90,000 x 40 103 and 189).
+constexpr int kForkNnz = 800000, kForkVectorNnz = 4000000;
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
@@ -1472,6 +1475,33 @@ float time_median(F fn, cudaStream_t s) {
   if (!ok) return -1.0f;
   std::sort(t, t + 3);
   return t[1];
+}
+
+// Whether this pass of both outputs runs dvals on the side stream.  The second such pass makes it (a
+// transpose that is used once does not earn it back), unless `s` is being captured.
+bool tplan_forks(gbs_tplan* t, int dtype, int k, cudaStream_t s) {
+  if (t->nnz < (dtype == GBS_F64 && k == 1 ? kForkVectorNnz : kForkNnz)) return false;
+  if (t->side) return true;
+  if (!t->again) {
+    t->again = true;
+    return false;
+  }
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
+  cudaStream_t side = nullptr;
+  cudaEvent_t a = nullptr, b = nullptr;
+  if (cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess &&
+      cudaEventCreateWithFlags(&a, cudaEventDisableTiming) == cudaSuccess &&
+      cudaEventCreateWithFlags(&b, cudaEventDisableTiming) == cudaSuccess) {
+    t->side = side;
+    t->ev_fork = a;
+    t->ev_join = b;
+    return true;
+  }
+  cudaGetLastError();
+  if (a) cudaEventDestroy(a);
+  if (side) cudaStreamDestroy(side);
+  return false;
 }
 
 // Keep `plan` as the prepared plan of A^T for (dtype, k), replacing an earlier one.
@@ -1561,12 +1591,6 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
   }
   rc = compute_stats(n, m, nnz, t->rptrT, &t->statsT, s);  // waits for s (without columns: nothing ran)
   if (rc == GBS_OK && n == 0 && cudaStreamSynchronize(s) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "transpose");
-  if (rc == GBS_OK && nnz >= kForkNnz) {
-    e = cudaStreamCreateWithFlags(&t->side, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&t->ev_join, cudaEventDisableTiming);
-    if (e != cudaSuccess) rc = cuda_fail(e, "backward stream and events");
-  }
   if (rc) {
     gbs_tplan_destroy(t);
     return rc;
@@ -1703,10 +1727,10 @@ int spmv_csr_backward(gbs_tplan* t, const int* row_ptr, const int* col_idx, cons
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (s != nullptr) t->away.store(true, std::memory_order_relaxed);
   cudaError_t e;
-  // both outputs: the dvals pass runs on the plan's side stream while dX runs on `stream`; the
+  // both outputs, of a large A: the dvals pass runs on the plan's side stream while dX runs on `stream`; the
   // two read the same inputs and write different outputs, and `stream` waits for the side
   // stream before anything after this call
-  const bool fork = dX && dvals && t->nnz > 0 && t->side;
+  const bool fork = dX && dvals && tplan_forks(t, dtype, k, s);
   if (fork) {
     e = cudaEventRecord(t->ev_fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(t->side, t->ev_fork, 0);

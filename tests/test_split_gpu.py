@@ -623,3 +623,36 @@ def test_dvals_time_of_odd_columns(gbs, dtype):
         return min(times)
 
     assert us(13) <= 1.2 * us(16)
+
+
+@DT
+@pytest.mark.parametrize("k", [1, 4])
+def test_backward_beside_itself(gbs, k, dtype):
+    """A backward pass whose dvals run beside dX, from the second call on (a transpose used once makes no
+    stream): the bits of the two outputs asked for one by one, on two streams and captured before and after."""
+    A = synth.rmat(17 if k > 1 or dtype == torch.float32 else 19, ef=16, seed=16)
+    shape = (A.m,) if k == 1 else (A.m, k)
+    v = dev(A.vals.astype(NP[dtype]))
+    X, W = (dev(synth.uniform(A.m * k, seed=55, stream=i).astype(NP[dtype])).reshape(shape) for i in range(2))
+    t = gbs.TransposePlan(dev(A.row_ptr), dev(A.col_idx), A.n)
+    want = t.backward(v, X, W, need_dvals=False)[0], t.backward(v, X, W, need_dX=False)[1]
+
+    def capture():
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            out = t.backward(v, X, W)
+        return g, out
+
+    graphs = [capture(), capture()]  # the second such call is captured: no stream can be made then
+    runs = [t.backward(v, X, W) for _ in range(3)]
+    graphs.append(capture())
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    runs += [t.backward(v, X, W, stream=side) for _ in range(3)]
+    for g, out in graphs:
+        out[0].zero_(), out[1].zero_()
+        g.replay()
+        runs.append(out)
+    torch.cuda.synchronize()
+    for got in runs:
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
