@@ -357,7 +357,9 @@ int spmm_csr_cfg(int m, int n, int nnz, const int* row_ptr, const int* col_idx, 
  * on the device (on scratch values it allocates itself, each run after a
  * write of twice the L2's size so that it starts cold) and keeps the
  * fastest (with GBS_PLAN_EMULATE also candidates that run part of the FP64
- * products on the FP32 pipe).  With GBS_PLAN_CHECK it validates the structure first.  The plan
+ * products on the FP32 pipe).  Where k columns do not fill whole 16 bytes it does
+ * so for contiguous operands, whose configuration is the plan's, and again for
+ * rows padded to 16 bytes, whose calls take theirs until one is set.  With GBS_PLAN_CHECK it validates the structure first.  The plan
  * keeps row_ptr and col_idx as given: they must stay valid and unchanged
  * while the plan is used.  gbs_plan_create synchronises `stream`.
  * Executing a plan can be captured in a CUDA graph.  It allocates nothing, except

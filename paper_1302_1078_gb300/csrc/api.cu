@@ -797,6 +797,9 @@ struct gbs_plan {
   SplitScratch split_scratch{};
   bool tuning = false;   // the tuner is trying configurations: keep the relabelling between them
   bool ready = true;     // what cfg needs is there; false: no product runs (plan_run)
+  // a tuned plan whose k columns fill no whole 16 bytes: the plan of calls whose operands are padded to
+  // 128-bit column access, tuned on such operands, if another configuration is faster for them
+  gbs_plan* padded = nullptr;
   // What the plan owns is stream-ordered memory.  It is freed on the stream that makes the plan
   // while it is being made and on the legacy default stream afterwards, which is ordered behind
   // every use of the plan only if there was none on another stream; if there was (away), the
@@ -983,6 +986,7 @@ int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, 
   // the caller's operands decide the column access (and with it the merge geometry), also when
   // the product reads the relabelled copy of X, so that relabelling never changes a result
   const bool vec16 = dense_vec16(p->dtype, p->k, X, ldx, Y, ldy);
+  if (p->padded && vec16) return plan_run(p->padded, vals, X, ldx, Y, ldy, s);
   if (p->cfg.relabel != 0 && p->newid && p->m > 0 && p->k > 0) {
     // x' = x in the relabelled column order, then the product with the relabelled column ids
     const bool src16 = p->k > 1 && aligned16(X) && (ldx * (long long)dsize(p->dtype)) % 16 == 0;
@@ -1163,12 +1167,14 @@ std::vector<gbs_config> tune_candidates(const gbs_plan* p) {
   return c;
 }
 
-int plan_tune(gbs_plan* p, cudaStream_t s) {
+// Operands without padding, as a contiguous X has, or with rows padded to 16 bytes: with an odd number
+// of columns the former allow no 128-bit access, which decides the kernels' instances and with them
+// the order of the candidates (timed on padded rows, the 50^3 stencil's k = 3 took merge-path, 66 us where
+// ROWS takes 29; timed on contiguous ones, 400,003 x 41 banded, FP64, k = 5, 474 us on padded operands where
+// 336 were to be had).
+int plan_tune(gbs_plan* p, bool padded, cudaStream_t s) {
   const size_t es = dsize(p->dtype);
-  // operands without padding, as a contiguous X has: with an odd number of columns its rows allow no
-  // 128-bit access, which decides the kernels' instances and with them the order of the candidates
-  // (timed on padded rows, the 50^3 stencil's k = 3 took merge-path: 66 us where ROWS takes 29)
-  const long long ldp = p->k;
+  const long long ldp = padded ? (p->k + vec_of(p->dtype) - 1) / vec_of(p->dtype) * vec_of(p->dtype) : p->k;
   void *vals = nullptr, *X = nullptr, *Y = nullptr;
   size_t bv = std::max<size_t>(16, (size_t)p->nnz * es);
   size_t bx = std::max<size_t>(16, (size_t)p->n * (p->k == 1 ? 1 : ldp) * es);
@@ -1230,6 +1236,7 @@ int plan_tune(gbs_plan* p, cudaStream_t s) {
     std::vector<std::pair<float, gbs_config>> timed;
     for (const gbs_config& c : tune_candidates(p)) {
       if (check_cfg(c, p->k) != GBS_OK) continue;
+      if (padded && (c.relabel || c.emul)) continue;
       p->cfg = c;
       if (plan_prepare(p, s) != GBS_OK) continue;
       const float ms = median_ms(7);
@@ -1278,6 +1285,7 @@ int plan_tune(gbs_plan* p, cudaStream_t s) {
 }
 
 void plan_destroy_impl(gbs_plan* p) {
+  if (p->padded) plan_destroy_impl(p->padded);
   DeviceGuard guard(p->device);
   quiesce(p->away);
   relabel_release(p);
@@ -1285,6 +1293,39 @@ void plan_destroy_impl(gbs_plan* p) {
   if (p->mb.base) plan_free(p, p->mb.base);
   if (p->status) plan_free(p, p->status);
   delete p;
+}
+
+// The plan of `p`'s padded calls (gbs_plan::padded), after p has been tuned on contiguous operands.
+// Without memory for it, p serves them.
+void plan_tune_padded(gbs_plan* p, cudaStream_t s) {
+  if (p->k % vec_of(p->dtype) == 0 || p->k == 1) return;
+  gbs_plan* q = new (std::nothrow) gbs_plan();
+  if (!q) return;
+  q->m = p->m;
+  q->n = p->n;
+  q->nnz = p->nnz;
+  q->k = p->k;
+  q->dtype = p->dtype;
+  q->device = p->device;
+  q->row_ptr = p->row_ptr;
+  q->col_idx = p->col_idx;
+  q->stats = p->stats;
+  q->flags = p->flags;
+  q->perm = p->perm;
+  q->owner = s;
+  q->cfg = plan_default_config(q);
+  q->col_max_deg = 0;  // no relabelled candidates
+  const bool ok = plan_tune(q, true, s) == GBS_OK;
+  const gbs_config &a = p->cfg, &b = q->cfg;
+  if (!ok || (a.variant == b.variant && a.lanes == b.lanes && a.threads == b.threads && a.tile_nnz == b.tile_nnz &&
+              a.items == b.items && a.relabel == 0 && a.emul == 0)) {
+    plan_destroy_impl(q);
+    g_err.clear();
+    return;
+  }
+  q->owner = nullptr;
+  q->away.store(false, std::memory_order_relaxed);
+  p->padded = q;
 }
 
 // gbs_plan_create with an optional permutation through which the values are read
@@ -1318,7 +1359,9 @@ int plan_create_impl(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr,
   rc = compute_stats(m, n, nnz, row_ptr, &p->stats, s);
   if (rc == GBS_OK) {
     p->cfg = plan_default_config(p);
-    rc = (flags & GBS_PLAN_TUNE) && m > 0 ? plan_tune(p, s) : plan_prepare_default(p, s);
+    const bool tune = (flags & GBS_PLAN_TUNE) && m > 0;
+    rc = tune ? plan_tune(p, false, s) : plan_prepare_default(p, s);
+    if (tune && rc == GBS_OK) plan_tune_padded(p, s);
   }
   if (rc != GBS_OK) {
     plan_destroy_impl(p);
@@ -1349,14 +1392,16 @@ int gbs_plan_status(gbs_plan* plan, int* status, void* stream) {
   if (!plan || !status) return fail(GBS_EINVAL, "NULL pointer");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   *status = 0;
-  if (!plan->status) {  // no bounded waits in the plan's configuration
-    const cudaError_t e = cudaStreamSynchronize(s);
-    return e == cudaSuccess ? GBS_OK : cuda_fail(e, "plan status");
+  cudaError_t e = cudaSuccess;
+  int words[2] = {0, 0}, i = 0;  // (a plan without bounded waits in its configuration has no word)
+  for (gbs_plan* p = plan; p && e == cudaSuccess; p = p->padded, ++i) {
+    if (!p->status) continue;
+    if (s != nullptr) p->away.store(true, std::memory_order_relaxed);
+    e = cudaMemcpyAsync(words + i, p->status, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p->status, 0, sizeof(int), s);
   }
-  if (s != nullptr) plan->away.store(true, std::memory_order_relaxed);
-  cudaError_t e = cudaMemcpyAsync(status, plan->status, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(plan->status, 0, sizeof(int), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  *status = words[0] | words[1];
   return e == cudaSuccess ? GBS_OK : cuda_fail(e, "plan status");
 }
 
@@ -1393,6 +1438,10 @@ int gbs_plan_set_config(gbs_plan* plan, const gbs_config* cfg) {
   plan->cfg = c;
   rc = cfg->variant == GBS_VARIANT_AUTO ? plan_prepare_default(plan, nullptr) : plan_prepare(plan, nullptr);
   plan->ready = rc == GBS_OK;
+  if (rc == GBS_OK && plan->padded) {  // the configuration is every call's
+    plan_destroy_impl(plan->padded);
+    plan->padded = nullptr;
+  }
   if (rc != GBS_OK) {
     // refused: the plan keeps the configuration it had, whose scratch is made again
     const std::string why = g_err;

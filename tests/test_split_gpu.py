@@ -1,6 +1,8 @@
 """SPLIT plans (equal shares of nonzeros per merge thread) against the oracle: nonzero counts at the
 edges of a share, a word and a tile, rows that span many tiles, runs of empty rows, ragged and
 strided columns, arrays off a 32-byte boundary, values through a permutation, relabelled columns."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -656,3 +658,46 @@ def test_backward_beside_itself(gbs, k, dtype):
     torch.cuda.synchronize()
     for got in runs:
         assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@DT
+@pytest.mark.parametrize("k", [3, 5])
+def test_tuned_plans_of_odd_columns_serve_padded_operands(gbs, k, dtype):
+    """A tuned plan whose columns fill no whole 16 bytes, with contiguous and padded operands, after its
+    configuration is set; the padded calls take at most 1.25 times the plan that
+    is best for them among the row-wise, merge and split forms (the tuner times cold products, this one warm ones)."""
+    A = synth.banded(200000, hbw=500, per_row=41, seed=17)
+    v = dev(A.vals.astype(NP[dtype]))
+    ld = -(-k // 4) * 4
+    Xh = synth.uniform(A.n * ld, seed=56).reshape(A.n, ld).astype(NP[dtype])
+    ref, r = oracle.spmm(A.m, A.row_ptr, A.col_idx, A.vals.astype(NP[dtype]), Xh[:, :k])
+    X = dev(Xh)
+    Y = torch.empty((A.m, ld), dtype=dtype, device="cuda")
+    rp, ci = dev(A.row_ptr), dev(A.col_idx)
+    plan = gbs.Plan(rp, ci, A.n, dtype, k, tune=True)
+
+    def us(p):
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(10):
+                p.spmm(v, X[:, :k], Y[:, :k])
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b) * 100)
+        return min(times)
+
+    tuned = us(plan)
+    within(Y[:, :k], ref, r, dtype, "tuned, padded")
+    within(plan.spmm(v, X[:, :k].contiguous()), ref, r, dtype, "tuned, contiguous")
+    status = ctypes.c_int(7)
+    assert gbs.lib().gbs_plan_status(plan._h, ctypes.byref(status), None) == 0 and status.value == 0
+    others = []
+    for cfg in (dict(variant=1), dict(variant=2), dict(variant=3, threads=128), dict(variant=5, threads=128), dict(variant=6)):
+        plan.set_config(cfg)
+        assert plan.config["variant"] == cfg["variant"]
+        others.append(us(plan))
+        within(Y[:, :k], ref, r, dtype, str(cfg))
+    assert tuned <= 1.25 * min(others), (tuned, others)
