@@ -163,7 +163,11 @@ int gbs_validate_csr(int m, int n, int nnz, const int* row_ptr, const int* col_i
  */
 int gbs_csr_stats(int m, int n, int nnz, const int* row_ptr, gbs_stats* out, void* stream);
 
-/* The configuration the library would pick for these statistics and k (host only). */
+/*
+ * The row-wise or merge-path configuration that these statistics suggest for k (host only).  An
+ * untuned plan takes it for vectors on even rows; for the rest it starts from the same two cases and
+ * takes ROWS_DIRECT, ROWS_TMA, MERGE_DIRECT or SPLIT (gbs_plan_get_config tells).
+ */
 int gbs_default_config(const gbs_stats* stats, int dtype, int k, gbs_config* out);
 
 /*

@@ -1,7 +1,7 @@
 // C-ABI entry points of gbspmv (declared in include/gbspmv.h): argument
 // checks, configuration choice, plans, the autotuner, CSR statistics and
-// validation.  Every product runs in the kernels of rows_kernel.cuh and
-// merge_kernel.cuh; nothing here computes on the host.
+// validation.  Every product runs in the kernels of rows_kernel.cuh, rows_tma.cuh,
+// merge_kernel.cuh, split_kernel.cuh and small.cu; nothing here computes on the host.
 #include <algorithm>
 #include <atomic>
 #include <climits>
@@ -191,7 +191,7 @@ int run_product(const CsrView& A, int dtype, int k, const void* X, long long ldx
   cudaError_t e = cudaSuccess;
   const bool perm = A.perm != nullptr;
   if (perm && cfg.variant == GBS_VARIANT_ROWS_TMA)
-    return fail(GBS_EUNSUPPORTED, "values read through a permutation need the ROWS, MERGE or MERGE_DIRECT variant");
+    return fail(GBS_EUNSUPPORTED, "values read through a permutation need the ROWS, MERGE, MERGE_DIRECT or SPLIT variant");
   if (cfg.variant == GBS_VARIANT_ROWS_TMA && status && aligned16(A.vals) && aligned16(A.col_idx)) {
     // the widest panel's lanes for every panel: the tile holds the row blocks of that many lanes,
     // and a narrower last panel with its own fewer lanes would have longer ones
@@ -714,7 +714,8 @@ static int product_entry(int m, int n, int nnz, const int* row_ptr, const int* c
     return e == cudaSuccess ? GBS_OK : cuda_fail(e, "small SpMV launch");
   }
   // a vector product of fewer items than this is bound by its launches, of which merge-path has
-  // three and SPLIT four (64 x 64 grid: 25.1 and 25.5 us; 1.3 M nonzeros: 31.8 and 25.8 us)
+  // three and SPLIT four.  (The line is from before SPLIT's were dependent launches; at 434,600 items it takes
+  // 13.8 us where merge-path takes 19.9, so the line could lie lower.)
   const bool small = k == 1 && (long long)m + nnz < 400000;
   if (unset && !small) {
     // SPLIT, which needs no row statistics and balances any row lengths (27-point 100^3, k = 4:
@@ -967,7 +968,7 @@ int plan_prepare(gbs_plan* p, cudaStream_t s) {
   cudaError_t e = scratch_alloc(&p->mb.base, p->mb.bytes, s);
   if (e != cudaSuccess) {
     p->mb = MergeBuffers{};
-    return cuda_fail(e, "cudaMalloc (plan scratch)");
+    return cuda_fail(e, "memory of the plan's merge scratch");
   }
   merge_carve(p->mb, G.ctas, G.kp_max, p->dtype);
   CsrView A{p->m, p->n, p->nnz, p->row_ptr, p->col_idx, nullptr};
@@ -1329,7 +1330,7 @@ void plan_tune_padded(gbs_plan* p, cudaStream_t s) {
 }
 
 // gbs_plan_create with an optional permutation through which the values are read
-// (perm != nullptr: the plan is restricted to the ROWS and MERGE_DIRECT variants).
+// (perm != nullptr: the plan is restricted to the ROWS, MERGE, MERGE_DIRECT and SPLIT variants).
 int plan_create_impl(gbs_plan** plan, int m, int n, int nnz, const int* row_ptr, const int* col_idx, int dtype, int k,
                      int flags, const int* perm, void* stream) {
   if (plan == nullptr) return fail(GBS_EINVAL, "plan is NULL");

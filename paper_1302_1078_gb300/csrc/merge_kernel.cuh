@@ -510,8 +510,7 @@ __device__ __forceinline__ void merge_fixup_one(int b, int ctas, int k, const in
 // tiles (a hub row; on R-MAT 22 one row spans 85 tiles), which the thread's warp takes over: the
 // run's end is found 32 tiles per step by a ballot, and its carries are loaded 32 at a time by
 // the lanes and added in tile order from shuffles.  The additions are merge_fixup_one's, in the
-// same order (so the batched kernel's fix-up gives the same bits); only the chain of dependent
-// loads is shortened.
+// same order; only the chain of dependent loads is shortened.
 template <typename T>
 __global__ void merge_fixup_kernel(int ctas, int k, const int* __restrict__ carry_row, const T* __restrict__ carry_val,
                                    T* __restrict__ Y, long long ldy) {

@@ -219,7 +219,7 @@ cudaError_t radix_sort_pairs(int n, int bits, int* keys_a, int* keys_b, int* val
   return radix_sort(n, bits, keys_a, vals_a, keys_a, keys_b, vals_a, vals_b, nullptr, hist, scan_ws, keys_out, vals_out, s);
 }
 
-// Transpose with caller-provided device buffers (see tplan_create for sizes).
+// Transpose with caller-provided device buffers (sizes: launch.h).
 // Returns a CUDA error.  tmp must hold 2 * nnz + 2 * nnz ints + hist + scan workspace.
 cudaError_t transpose_run(int m, int n, int nnz, const int* row_ptr, const int* col_idx, int* rptrT, int* colT,
                           int* perm, int* rows, int* keys_a, int* keys_b, int* vals_a, int* vals_b, int* hist,

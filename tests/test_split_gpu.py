@@ -513,6 +513,12 @@ def test_small_one_shot_long_rows_together(gbs, shape, nnz, dtype):
         gbs.spmv_csr(dev(A.row_ptr), ci, vd, dev(x), y)
         within(y, ref, r, dtype, f"{shape} {nnz} off={off}")
         assert torch.equal(y, gbs.spmv_csr(dev(A.row_ptr), ci, vd, dev(x)))
+    rp, xd = dev(A.row_ptr), dev(x)
+    with torch.cuda.graph(g := torch.cuda.CUDAGraph()):
+        out = gbs.spmv_csr(rp, ci, vd, xd)
+    out.zero_()
+    g.replay()
+    assert torch.equal(out, y)
 
 
 @pytest.mark.parametrize("shape", ["block", "just_long", "hub"])
