@@ -470,8 +470,8 @@ int gbs_tplan_get_config(const gbs_tplan* plan, int dtype, int k, gbs_config* cf
  * gbs_transpose_plan on the same (row_ptr, col_idx); row_ptr is unused.
  * When both dX and dvals are asked for and A has at least 800,000 nonzeros
  * (4,000,000 for k = 1 in doubles), the dvals pass runs on a stream the plan
- * owns, concurrently with dX, from the second such call on (which makes the
- * stream; below, the two run one after the other on `stream`): it waits for the work enqueued on
+ * owns, concurrently with dX, below 4,000,000 from the second such call on (which makes
+ * the stream; else the two run one after the other on `stream`): it waits for the work enqueued on
  * `stream` before the call, and `stream` waits for it before anything
  * enqueued after the call (an event each way, which stream capture
  * follows), so the call is ordered on `stream` like any other.  The plan's

@@ -1527,17 +1527,8 @@ float time_median(F fn, cudaStream_t s) {
   return t[1];
 }
 
-// Whether this pass of both outputs runs dvals on the side stream.  The second such pass makes it (a
-// transpose that is used once does not earn it back), unless `s` is being captured.
-bool tplan_forks(gbs_tplan* t, int dtype, int k, cudaStream_t s) {
-  if (t->nnz < (dtype == GBS_F64 && k == 1 ? kForkVectorNnz : kForkNnz)) return false;
-  if (t->side) return true;
-  if (!t->again) {
-    t->again = true;
-    return false;
-  }
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
+// The side stream and its events (about 50 us); false, and none of them, if they cannot be had.
+bool tplan_make_side(gbs_tplan* t) {
   cudaStream_t side = nullptr;
   cudaEvent_t a = nullptr, b = nullptr;
   if (cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking) == cudaSuccess &&
@@ -1552,6 +1543,21 @@ bool tplan_forks(gbs_tplan* t, int dtype, int k, cudaStream_t s) {
   if (a) cudaEventDestroy(a);
   if (side) cudaStreamDestroy(side);
   return false;
+}
+
+// Whether this pass of both outputs runs dvals on the side stream.  Where the transpose has not made it,
+// the second such pass does (a transpose that is used once does not earn it back), unless `s` is being
+// captured.
+bool tplan_forks(gbs_tplan* t, int dtype, int k, cudaStream_t s) {
+  if (t->nnz < (dtype == GBS_F64 && k == 1 ? kForkVectorNnz : kForkNnz)) return false;
+  if (t->side) return true;
+  if (!t->again) {
+    t->again = true;
+    return false;
+  }
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone) return false;
+  return tplan_make_side(t);
 }
 
 // Keep `plan` as the prepared plan of A^T for (dtype, k), replacing an earlier one.
@@ -1641,6 +1647,7 @@ int gbs_transpose_plan(gbs_tplan** out, int m, int n, int nnz, const int* row_pt
   }
   rc = compute_stats(n, m, nnz, t->rptrT, &t->statsT, s);  // waits for s (without columns: nothing ran)
   if (rc == GBS_OK && n == 0 && cudaStreamSynchronize(s) != cudaSuccess) rc = cuda_fail(cudaGetLastError(), "transpose");
+  if (rc == GBS_OK && nnz >= kForkVectorNnz) tplan_make_side(t);
   if (rc) {
     gbs_tplan_destroy(t);
     return rc;
