@@ -287,10 +287,10 @@ static cudaError_t sddmm_t(int nnz, int k, const SplitIndex& I, int m, const int
   // and 74), up to four slices of 32 bytes: FP32 k = 32 133 and 157.
   const bool short_rows = nnz < 6LL * m;
   if constexpr (sizeof(T) == 8) {
-    // one 16-byte slice: banded 200,003 x 41, k = 2 36 and 45 us; k = 4 66 and 66, 8 121 and 119, 12 175
-    // and 170, 16 230 and 256; R-MAT 20, k = 8 227 and 231, k = 12 333 and 325
+    // one 16-byte slice: banded 200,003 x 41, k = 2 36 and 45 us; k = 4 66 and 66, 12 175 and 170, 16 230 and
+    // 256; k = 8 R-MAT 20 (15 in a row) 227 and 235, banded 500,000 x 9 76 and 71
     if (k < 4 && k >= H && all % 16 == 0) return go(sddmm_kernel<T, H, false>);
-    if (k > 12 && all % 32 == 0 && !short_rows) return go(sddmm_kernel<T, W, false>);
+    if (all % 32 == 0 && (k > 12 ? !short_rows : k == 8 && nnz >= 12LL * m)) return go(sddmm_kernel<T, W, false>);
     if (k >= H && all % 16 == 0) return go_lanes(sddmm_lane_kernel<T, H, false>);
     // single columns; registers for more loads from k = 8 (banded 500,000 x 9: k = 5 51 and 51 us, k = 3
     // 34 and 35, k = 13 135 and 124)
