@@ -1240,7 +1240,7 @@ int plan_tune(gbs_plan* p, bool padded, cudaStream_t s) {
       if (padded && (c.relabel || c.emul)) continue;
       p->cfg = c;
       if (plan_prepare(p, s) != GBS_OK) continue;
-      const float ms = median_ms(7);
+      const float ms = median_ms(padded ? 3 : 7);
       if (ms < 0) continue;
       if (tune_log())
         std::fprintf(stderr, "gbspmv tune m=%d nnz=%d k=%d: variant=%d lanes=%d threads=%d tile=%d items=%d emul=%d "
@@ -1249,10 +1249,11 @@ int plan_tune(gbs_plan* p, bool padded, cudaStream_t s) {
       timed.emplace_back(ms, c);
     }
     // the leaders often differ by a few per cent, about the spread of seven runs: the three best
-    // are timed again, fifteen runs each, and the best of those medians is kept
+    // are timed again, fifteen runs each, and the best of those medians is kept (not for padded operands,
+    // which are rare: a third of the time)
     std::stable_sort(timed.begin(), timed.end(),
                      [](const std::pair<float, gbs_config>& x, const std::pair<float, gbs_config>& y) { return x.first < y.first; });
-    const size_t lead = std::min<size_t>(3, timed.size());
+    const size_t lead = std::min<size_t>(padded ? 1 : 3, timed.size());
     for (size_t i = 0; i < lead; ++i) {
       float ms = timed[i].first;
       p->cfg = timed[i].second;
