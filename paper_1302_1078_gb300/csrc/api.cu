@@ -1035,7 +1035,7 @@ int plan_run(const gbs_plan* p, const void* vals, const void* X, long long ldx, 
 }
 
 // The untuned configuration of a plan: heuristic_config's, except that skewed rows take the forms a
-// plan can afford: SPLIT for block vectors (R-MAT 20, k = 8, FP32: 223 us staged merge-path, 134 us
+// plan can afford: SPLIT for block vectors (R-MAT 20, k = 8, FP32: 233 us staged merge-path, 122 us
 // SPLIT); a vector takes the direct merge walk, which needs no index beyond the tiles' coordinates.
 gbs_config plan_default_config(const gbs_plan* p) {
   gbs_config c = heuristic_config(p->stats, p->dtype, p->k);

@@ -59,7 +59,7 @@ struct SplitScratch {
 // Nonzeros per merge thread of the SPLIT SpMV (x and y contiguous): one 32-byte sector of column ids.
 constexpr int kSplitShare = 8;
 // Threads per CTA of a SPLIT launch.  A float vector's CTAs of two warps end faster than new ones
-// begin: three warps there (2M x 50 banded: 64 threads 204 us, 96 175, 128 182); the others keep two,
+// begin: three warps there (2M x 50 banded: 64 threads 204 us, 96 181, 128 187); the others keep two,
 // which leave the smallest last wave (doubles: 281, 282, 282; R-MAT 22 257, 258, 261).
 inline int split_threads(int dtype, int k) { return k == 1 && dtype == GBS_F32 ? 96 : 64; }
 

@@ -34,7 +34,7 @@
 // 22 FP64 338 us (direct merge walk) -> 257 us, 0.50 of the measured HBM rate;
 // R-MAT 20 forward 95 -> 75 us.  SpMM: FP64 is bound by its pipe (R-MAT 22,
 // k = 8: 1346 -> 1008 us, 0.81 of the pipe), FP32 by instruction issue (R-MAT
-// 20, k = 8, forward: 238 -> 134 us; the staged merge walk issued about 150
+// 20, k = 8, forward: 233 us staged merge walk, 122 us; the staged walk issued about 150
 // warp instructions per 16 nonzeros, most of them in divergent row ends).
 #pragma once
 #include "dependent.cuh"
@@ -118,8 +118,9 @@ __device__ __forceinline__ int split_row(const int* __restrict__ ids, int ord) {
 
 // The open sum of a merge thread as the carry scan combines it.  float: both parts of the
 // accumulator, the sums added with Knuth's TwoSum, so that the scan does not round (error against 64
-// bits, two plain additions, TwoSum and merge-path: 200,003 x 41 banded SpMV 6.0e-8, 3.6e-8, 5.8e-8;
-// R-MAT 20, k = 8, forward and backward 6.4e-8, 4.3e-8, 6.8e-8, for 2% of the time).
+// bits, with the accumulator of the time: 200,003 x 41 banded SpMV 6.0e-8 by two plain additions, 3.6e-8 by
+// TwoSum, merge-path 5.8e-8, for 2% of the time; now 2.7e-8, and R-MAT 20, k = 8, forward and backward
+// 3.4e-8, merge-path 6.8e-8).
 template <typename T>
 struct Open;
 template <>
