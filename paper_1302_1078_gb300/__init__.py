@@ -298,7 +298,8 @@ def default_config(stats: dict, dtype: torch.dtype, k: int = 1) -> dict:
 class Plan:
     """A fixed CSR structure with its chosen (optionally autotuned) configuration.
 
-    The plan keeps references to row_ptr and col_idx; executing it allocates nothing."""
+    The plan keeps references to row_ptr and col_idx; executing it allocates nothing but the scratch of
+    some block products whose operands allow no 128-bit column access (stream-ordered)."""
 
     def __init__(self, row_ptr, col_idx, n: int, dtype=torch.float64, k: int = 1, *, tune: bool = False,
                  check: bool = False, emulate: bool = False, config=None, stream=None):
