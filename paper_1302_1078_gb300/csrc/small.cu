@@ -14,6 +14,8 @@
 // Back to back, FP64 and FP32: 64 x 64 grid, 20,224 nonzeros, 7 us, of which 6 are the Python call
 // (merge-path 23 before the library had a pool of its own, 18 with it); 512 rows of 192 together 17 and
 // 13; one row of 98,304 19 and 15 (23 and 21); six rows of 16,000 15 and 11 (20 and 18).
+// The kernel alone under ncu, long rows by the CTA that owns them and by the cluster: R-MAT 13 x 9 37 and 10
+// us, FP32 22 and 10; 390,000 rows, most of them empty, whose ends eight CTAs look at, 7 and 10.
 #include <algorithm>
 
 #include "device_common.cuh"
